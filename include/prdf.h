@@ -318,8 +318,9 @@ uint64_t pr_kernel_launches(void);
  * must be serialised by the caller.  A call clears what it needs cleared at its start.
  * Errors: PR_ERR_INVALID_ARG (NULL or host pointers, pointers on another device than the
  * current one, bad params, malformed offsets, a vertex with no out-edge),
- * PR_ERR_VERTEX_RANGE (a column id >= n), PR_ERR_CUDA; ranks are written only after the
- * CSR has passed these checks. */
+ * PR_ERR_VERTEX_RANGE (a column id >= n), PR_ERR_DEVICE_TIMEOUT (a bounded wait of the
+ * iteration kernel gave up; ranks are undefined), PR_ERR_CUDA; ranks are written only after
+ * the CSR has passed these checks. */
 #define PR_NOALLOC_MAX_VERTICES (1u << 18)
 #define PR_NOALLOC_SCRATCH_BYTES (256u + 20u * PR_NOALLOC_MAX_VERTICES)
 pr_status pr_static_noalloc(uint32_t n, int64_t m, const uint64_t *in_off, const uint32_t *in_col,

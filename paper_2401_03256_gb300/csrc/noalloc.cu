@@ -26,12 +26,12 @@ namespace {
 
 constexpr uint32_t kMaxN = PR_NOALLOC_MAX_VERTICES;
 constexpr int kThreads = 256;
-constexpr int kChunkIters = 8;     // iteration launches between reads of the control block
 constexpr int kMaxDevices = 64;
 
 struct NaCtl {
-  unsigned long long dmax;  // max |Delta R| of the running iteration (bits of a double >= 0)
-  uint32_t arrived;         // blocks finished with the running iteration
+  unsigned long long dmax[3];  // max |Delta R| by iteration modulo 3 (bits of a double >= 0)
+  uint32_t arrived;         // arrivals at the grid barrier (monotonic)
+  uint32_t timeout;         // 1 once a barrier wait ran out
   uint32_t done;            // 1 once an iteration's max change was <= tol
   uint32_t bad;             // 1 malformed offsets, 2 column id >= n, 4 vertex without out-edges
   int32_t iterations;
@@ -75,51 +75,255 @@ __global__ void k_na_check_deg(const uint32_t *deg, uint32_t n, NaCtl *ctl) {
   if (v < n && deg[v] == 0) atomicOr(&ctl->bad, 4u);
 }
 
-// R = 1/n, c = R / |out(u)|.
-__global__ void k_na_init(uint32_t n, const uint32_t *deg, double *R, double *c) {
-  uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= n) return;
-  const double r = 1.0 / (double)n;
-  R[v] = r;
-  c[v] = r / (double)deg[v];
-}
-
+// The iterations: one persistent cooperative launch, one block of kLoopThreads threads per SM.
+//
+// What bounds it: latency (an iteration's gathers hit L2; 60 K rows are about 1 M of them) and
+// the FP64 rate (2 adds per clock and SM), so lanes are kept full wherever FP64 is issued.
+// A block owns a run of consecutive rows holding 1/grid of the work (edges + kRowWeight a
+// row, found by binary search in the offsets once).  Rows of at most kLaneRow edges take four
+// lanes each; longer ones are listed once and cut into segments of kSegment edges, which take
+// four lanes each too: a warp-wide tree costs five full FP64 instructions (16 clocks each) for
+// every row.  The division is left to a pass with a thread per row, the sums meeting in
+// shared memory.  Every row's sum has one fixed order of additions.
+// On the 60,013-vertex R-MAT graph of 1 M edges: a thread per row 450 us an iteration (29.5 ms
+// a call), because of its hub rows; segments of 512 edges summed by warps and finished by one
+// lane 35 us (2.4 ms); this 20 us (1.47 ms).
+//
 // One Jacobi iteration of Eq. 1: R[v] = (1 - alpha) / n + alpha * sum over in-edges (u, v)
 // of c_in[u]; c_out[v] = R[v] / |out(v)|.  The rank is updated in place (the sums read only
-// c_in).  The last block to finish folds the iteration's L-inf change into the control
-// block and sets done once it is <= tol; launches after that return at once.
-__global__ void __launch_bounds__(kThreads) k_na_iter(uint32_t n, const uint64_t *off, const uint32_t *col,
-                                                      const uint32_t *deg, double base, double alpha, double tol,
-                                                      const double *c_in, double *c_out, double *R, NaCtl *ctl,
-                                                      int32_t it) {
-  __shared__ double s_max[kThreads / 32];
-  if (*(volatile uint32_t *)&ctl->done) return;
-  double lmax = 0.0;
-  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (uint64_t e = off[v], end = off[v + 1]; e < end; e++) s += c_in[col[e]];
-    const double r = base + alpha * s;
-    lmax = fmax(lmax, fabs(r - R[v]));
-    R[v] = r;
-    c_out[v] = r / (double)deg[v];
+// c_in, through L2: other SMs wrote it during this launch).  After each iteration's barrier
+// every block reads the same L-inf change and all stop together.
+constexpr int kLoopThreads = 1024;
+constexpr int kLoopWarps = kLoopThreads / 32;
+constexpr uint32_t kRowWeight = 4;     // work of a row beside its edges, in edges
+constexpr uint32_t kLaneRow = 16;      // edges of a row summed by four lanes at once
+constexpr uint32_t kSegment = 64;      // edges of a segment of a longer row
+constexpr uint32_t kMaxSegs = 1024;    // segments of one row at most (more edges each for huge rows)
+constexpr uint32_t kLongCap = 1024, kSegCap = 2048;  // listed rows and their segments per block
+constexpr uint32_t kTile = 2048;       // rows whose sums are in shared memory together
+constexpr unsigned long long kBarrierNs = 4000000000ull;  // a barrier wait gives up after 4 s
+
+__device__ __forceinline__ double na_warp_sum(double s) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// Sum of c_in over columns [s, e) by a whole warp, eight gathers a lane in flight.
+__device__ __forceinline__ double na_warp_row(const uint32_t *col, const double *c_in, uint64_t s, uint64_t e,
+                                              uint32_t lane) {
+  double t = 0.0;
+  for (uint64_t j0 = s; j0 < e; j0 += 256) {
+    double x[8];
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+      const uint64_t j = j0 + 32u * k + lane;
+      x[k] = j < e ? __ldcg(c_in + __ldg(col + j)) : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; k += 2)
+      if (j0 + 32u * k < e) t += x[k] + x[k + 1];  // the same in every lane
   }
-  for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-  if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = lmax;
+  return na_warp_sum(t);
+}
+
+__global__ void __launch_bounds__(kLoopThreads, 1)
+    k_na_loop(uint32_t n, uint64_t m, const uint64_t *off, const uint32_t *col, const uint32_t *deg, double base,
+              double alpha, double tol, double *c0, double *c1, double *R, NaCtl *ctl, int32_t max_iter) {
+  __shared__ double s_sum[kTile], s_part[kSegCap], s_max[kLoopWarps];
+  __shared__ uint32_t s_long[kLongCap], s_first[kLongCap + 1], s_seglen[kLongCap], s_nlong, s_list_end;
+  __shared__ uint32_t s_range[2], s_cnt[kLoopWarps];
+  __shared__ int s_stop;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+  const uint32_t gtid = blockIdx.x * kLoopThreads + tid, nthreads = gridDim.x * kLoopThreads;
+  if (*(volatile uint32_t *)&ctl->bad) return;  // the CSR failed its checks: ranks stay untouched
+  // this block's rows: the first v with off[v] + kRowWeight v at or above its share
+  if (tid < 2) {
+    const uint64_t total = m + (uint64_t)kRowWeight * n, share = (total + gridDim.x - 1) / gridDim.x;
+    const uint64_t at = share * (blockIdx.x + tid);
+    uint32_t lo = 0, hi = n;
+    while (lo < hi) {
+      const uint32_t mid = lo + (hi - lo) / 2;
+      if (__ldg(off + mid) + (uint64_t)kRowWeight * mid < at) lo = mid + 1; else hi = mid;
+    }
+    s_range[tid] = lo;
+  }
+  const double r0 = 1.0 / (double)n;
+  for (uint32_t v = gtid; v < n; v += nthreads) {  // R = 1/n, c = R / |out(u)|
+    R[v] = r0;
+    c0[v] = r0 / (double)deg[v];
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double bmax = s_max[0];
-    for (int w = 1; w < kThreads / 32; w++) bmax = fmax(bmax, s_max[w]);
-    atomicMax(&ctl->dmax, (unsigned long long)__double_as_longlong(bmax));
-    __threadfence();
-    if (atomicAdd(&ctl->arrived, 1u) == gridDim.x - 1) {
+  const uint32_t lo = s_range[0], hi = s_range[1];
+  uint32_t listed_rows = 0;  // rows longer than kLaneRow so far, in row order
+  for (uint32_t b0 = lo; b0 < hi; b0 += kLoopThreads) {
+    const uint32_t v = b0 + tid;
+    const bool f = v < hi && __ldg(off + v + 1) - __ldg(off + v) > kLaneRow;
+    const uint32_t mask = __ballot_sync(0xffffffffu, f);
+    if (lane == 0) s_cnt[wib] = __popc(mask);
+    __syncthreads();
+    uint32_t at = listed_rows + __popc(mask & prdf::lanemask_lt());
+    for (uint32_t w = 0; w < (uint32_t)kLoopWarps; w++) {
+      at += w < wib ? s_cnt[w] : 0u;
+      listed_rows += s_cnt[w];
+    }
+    if (f && at < kLongCap) s_long[at] = v;
+    __syncthreads();
+  }
+  if (tid == 0) {
+    // segments of the listed rows; rows from s_list_end on, which the lists have no room for,
+    // are summed by the warps that meet them
+    const uint32_t nl = listed_rows < kLongCap ? listed_rows : kLongCap;
+    uint32_t at = 0, k = 0;
+    for (; k < nl; k++) {
+      const uint64_t len = off[s_long[k] + 1] - off[s_long[k]];
+      uint64_t sl = kSegment;
+      if (len > (uint64_t)kMaxSegs * sl) sl = ((len + kMaxSegs - 1) / kMaxSegs + 31) / 32 * 32;
+      const uint32_t ns = sl > 0xFFFFFFFFull ? kSegCap + 1 : (uint32_t)((len + sl - 1) / sl);
+      if (at + ns > kSegCap) break;
+      s_first[k] = at;
+      s_seglen[k] = (uint32_t)sl;
+      at += ns;
+    }
+    s_list_end = k == listed_rows ? hi : (k ? s_long[k - 1] + 1 : lo);
+    s_nlong = k;
+    s_first[k] = at;
+  }
+  uint32_t bar = 0;
+  auto grid_barrier = [&]() -> bool {  // false after a wait that ran out (here or in another block)
+    __syncthreads();
+    bar++;
+    if (tid == 0) {
       __threadfence();
-      const double d = __longlong_as_double((long long)atomicAdd(&ctl->dmax, 0ull));
+      prdf::red_release_add_u32(&ctl->arrived, 1u);
+      const uint32_t want = bar * gridDim.x;
+      unsigned long long t0 = 0;
+      for (uint32_t spins = 0; prdf::ld_acquire_u32(&ctl->arrived) < want; spins++) {
+        if (*(volatile uint32_t *)&ctl->timeout) break;
+        if ((spins & 255u) == 255u) {
+          const unsigned long long t = prdf::globaltimer_ns();
+          if (t0 == 0) t0 = t;
+          else if (t - t0 > kBarrierNs) atomicExch(&ctl->timeout, 1u);
+        }
+      }
+      __threadfence();
+      s_stop = *(volatile uint32_t *)&ctl->timeout != 0;
+    }
+    __syncthreads();
+    return s_stop == 0;
+  };
+  if (!grid_barrier()) return;
+  const uint32_t nlong = s_nlong, nseg = s_first[nlong];
+  const uint32_t list_end = s_list_end;
+  for (int32_t it = 0; it < max_iter; it++) {
+    const double *c_in = it & 1 ? c1 : c0;
+    double *c_out = it & 1 ? c0 : c1;
+    double lmax = 0.0;
+    auto finish = [&](uint32_t v, double sum) {
+      const double r = base + alpha * sum;
+      lmax = fmax(lmax, fabs(r - R[v]));
+      R[v] = r;
+      c_out[v] = r / (double)__ldg(deg + v);
+    };
+    // segments of the listed rows, eight a warp
+    for (uint32_t k0 = wib * 8; k0 < nseg; k0 += kLoopWarps * 8) {
+      const uint32_t k = k0 + (lane >> 2), gl = lane & 3;
+      uint64_t s = 0, e = 0;
+      if (k < nseg) {
+        uint32_t a = 0, b = nlong;  // the row: last with s_first <= k
+        while (b - a > 1) {
+          const uint32_t mid = (a + b) >> 1;
+          if (s_first[mid] <= k) a = mid; else b = mid;
+        }
+        const uint32_t v = s_long[a];
+        s = __ldg(off + v) + (uint64_t)(k - s_first[a]) * s_seglen[a];
+        e = __ldg(off + v + 1);
+        if (s + s_seglen[a] < e) e = s + s_seglen[a];
+      }
+      const uint32_t len = (uint32_t)(e - s), longest = __reduce_max_sync(0xffffffffu, len);
+      double t = 0.0;
+      for (uint32_t j0 = 0; j0 < longest; j0 += 32) {
+        double x[8];
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+          const uint32_t j = j0 + 4u * q + gl;
+          x[q] = j < len ? __ldcg(c_in + __ldg(col + s + j)) : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; q += 2)
+          if (j0 + 4u * q < longest) t += x[q] + x[q + 1];
+      }
+      t += __shfl_xor_sync(0xffffffffu, t, 1);
+      t += __shfl_xor_sync(0xffffffffu, t, 2);
+      if (gl == 0 && k < nseg) s_part[k] = t;
+    }
+    for (uint32_t t0 = lo; t0 < hi; t0 += kTile) {
+      const uint32_t t1 = hi - t0 < kTile ? hi : t0 + kTile;
+      // eight rows a warp, four lanes a row
+      for (uint32_t b0 = t0 + wib * 8; b0 < t1; b0 += kLoopWarps * 8) {
+        const uint32_t v = b0 + (lane >> 2), gl = lane & 3;
+        uint64_t s = 0, e = 0;
+        if (v < t1) {
+          s = __ldg(off + v);
+          e = __ldg(off + v + 1);
+        }
+        const uint64_t len = e - s;
+        const uint32_t mine = len <= kLaneRow ? (uint32_t)len : 0u;
+        const uint32_t longest = __reduce_max_sync(0xffffffffu, mine);
+        double t = 0.0, x[kLaneRow / 4];
+#pragma unroll
+        for (int k = 0; k < (int)kLaneRow / 4; k++) {
+          const uint32_t j = 4u * k + gl;
+          x[k] = j < mine ? __ldcg(c_in + __ldg(col + s + j)) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < (int)kLaneRow / 4; k += 2)
+          if (4u * k < longest) t += x[k] + x[k + 1];
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        if (gl == 0 && v < t1 && len <= kLaneRow) s_sum[v - t0] = t;
+        // longer rows among the eight that are not listed, the whole warp on each
+        uint32_t more = __ballot_sync(0xffffffffu, gl == 0 && len > kLaneRow && v >= list_end);
+        while (more) {
+          const int src = __ffs(more) - 1;
+          more &= more - 1;
+          const uint64_t rs = __shfl_sync(0xffffffffu, s, src), re = __shfl_sync(0xffffffffu, e, src);
+          const uint32_t rv = __shfl_sync(0xffffffffu, v, src);
+          const double x = na_warp_row(col, c_in, rs, re, lane);
+          if (lane == 0) s_sum[rv - t0] = x;
+        }
+      }
+      __syncthreads();  // also after the segments of the long rows
+      for (uint32_t v = t0 + tid; v < t1; v += kLoopThreads) {
+        const bool listed = v < list_end && __ldg(off + v + 1) - __ldg(off + v) > kLaneRow;
+        if (!listed) finish(v, s_sum[v - t0]);
+      }
+      __syncthreads();  // s_sum is free again
+    }
+    for (uint32_t k = tid; k < nlong; k += kLoopThreads) {
+      double t = 0.0;
+      for (uint32_t j = s_first[k]; j < s_first[k + 1]; j++) t += s_part[j];
+      finish(s_long[k], t);
+    }
+    for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
+    if (lane == 0) s_max[wib] = lmax;
+    __syncthreads();
+    // the maximum of this iteration: three slots in turn, the next one cleared meanwhile (it was
+    // last read two iterations ago, before the previous barrier)
+    if (tid == 0) {
+      double bmax = s_max[0];
+      for (int w = 1; w < kLoopWarps; w++) bmax = fmax(bmax, s_max[w]);
+      if (blockIdx.x == 0) ctl->dmax[(it + 1) % 3] = 0;
+      atomicMax(&ctl->dmax[it % 3], (unsigned long long)__double_as_longlong(bmax));
+    }
+    if (!grid_barrier()) return;
+    const double d = __longlong_as_double((long long)__ldcg(&ctl->dmax[it % 3]));
+    if (gtid == 0) {
       ctl->last_delta = d;
       ctl->iterations = it + 1;
-      if (d <= tol) ctl->done = 1;
-      ctl->dmax = 0;
-      ctl->arrived = 0;
+      ctl->done = d <= tol;
     }
+    if (d <= tol) break;
   }
 }
 
@@ -196,36 +400,31 @@ extern "C" pr_status pr_static_noalloc(uint32_t n, int64_t m, const uint64_t *in
   }
   k_na_check_deg<<<blocks_for(n), kThreads, 0, st>>>(deg, n, ctl);
   prdf::count_launch();
-  NaCtl h{};
+  // the iterations are queued behind the checks and return at once if one failed: one launch
+  // and one synchronisation a call
+  const double base = (1.0 - p.alpha) / (double)n;
+  const uint64_t share = 4096;  // edges and row weights a block is worth launching for
+  const uint64_t want = ((uint64_t)m + (uint64_t)kRowWeight * n + share - 1) / share;
+  const unsigned grid = (unsigned)std::min<uint64_t>(std::max<uint64_t>(want, 1), (uint64_t)sm_count);
+  uint64_t m_u = (uint64_t)m;
+  double alpha = p.alpha, tol = p.tol, *c0 = c[0], *c1 = c[1];
+  int32_t max_iter = p.max_iter;
+  void *args[] = {&n, &m_u, (void *)&in_off, (void *)&in_col, &deg, (void *)&base, &alpha, &tol, &c0, &c1, &ranks,
+                  &ctl, &max_iter};
   e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = cudaLaunchCooperativeKernel((const void *)k_na_loop, dim3(grid), dim3(kLoopThreads), args, 0, st);
+  prdf::count_launch();
+  NaCtl h{};
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h, ctl, sizeof(NaCtl), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return PR_ERR_CUDA;
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return PR_ERR_CUDA;
+  }
   if (h.bad & 2u) return PR_ERR_VERTEX_RANGE;
   if (h.bad) return PR_ERR_INVALID_ARG;  // malformed offsets, or a vertex without out-edges
-
-  k_na_init<<<blocks_for(n), kThreads, 0, st>>>(n, deg, ranks, c[0]);
-  prdf::count_launch();
-  const double base = (1.0 - p.alpha) / (double)n;
-  const unsigned grid = std::min<unsigned>(blocks_for(n), (unsigned)sm_count * 8u);  // grid-stride rows
-  int32_t it = 0;
-  while (it < p.max_iter) {
-    const int32_t k = std::min<int32_t>(kChunkIters, p.max_iter - it);
-    for (int32_t j = 0; j < k; j++, it++) {
-      k_na_iter<<<grid, kThreads, 0, st>>>(n, in_off, in_col, deg, base, p.alpha, p.tol, c[it & 1],
-                                           c[(it + 1) & 1], ranks, ctl, it);
-      prdf::count_launch();
-    }
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, ctl, sizeof(NaCtl), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return PR_ERR_CUDA;
-    if (h.done) break;
-  }
-  if (p.max_iter == 0) {
-    e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return PR_ERR_CUDA;
-  }
+  if (h.timeout) return PR_ERR_DEVICE_TIMEOUT;
   if (stats) {
     stats->iterations = h.iterations;
     stats->converged = h.done ? 1 : 0;
