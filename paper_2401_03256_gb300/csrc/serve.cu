@@ -89,7 +89,11 @@ pr_status apply_group(pr_graph *h, const std::vector<Request> &group) {
 }
 
 void worker_loop(pr_server *s, int32_t gi) {
-  pr_graph *h = s->graphs[gi];
+  pr_graph *h;
+  {
+    std::lock_guard<std::mutex> lk(s->mu);  // graphs being added move the vector
+    h = s->graphs[gi];
+  }
   for (;;) {
     std::vector<Request> group;
     {
