@@ -93,8 +93,9 @@ typedef struct {
                              the model finds it cheaper; 2: always; 3: PR_ERR_INVALID_ARG).
                              Ids are translated at every call: results, ranks, affected sets
                              and the CSR export are in the caller's numbering (a renumbered
-                             handle keeps 8 B per vertex of translation tables on the device
-                             and 4 B on the host).  Computing a numbering takes a second,
+                             handle keeps 8 B per vertex of translation tables on the device,
+                             16 B in FP32 where it has vertices of large out-degree, and 4 B on
+                             the host).  Those vertices come first in the numbering.  Computing a numbering takes a second,
                              transient build of the graph on the device; without room for it
                              the caller's numbering is kept (0) or creation fails with
                              PR_ERR_OUT_OF_MEMORY (2, 3).  Other values: PR_ERR_INVALID_ARG. */
@@ -147,9 +148,10 @@ pr_status pr_get_component_stats(const pr_graph *g, pr_stats *stats, int32_t nco
  * compacted affected set once it exceeds n / dense_div vertices), the resident blocks per
  * SM of the persistent launch, and df_split (1, the default: a Dynamic Frontier, Dynamic
  * Traversal or asynchronous call on a single-graph handle in self-loop mode continues in
- * per-iteration launches once its affected set is dense (after its search for Dynamic
+ * sweep launches once its affected set is dense (after its search for Dynamic
  * Traversal), growing the set by pulling marks from per-vertex change flags or pushing the
- * out-rows of first expansions; 0: everything in the one persistent launch), and the sweep
+ * out-rows of first expansions; 0: everything in the one persistent launch.  Static and
+ * Naive-dynamic run all their iterations in one launch with 1, one launch each with 0), and the sweep
  * tiles: rows of bin_lo < in-degree <= max(bin_lo, group_max) take an 8-lane group each,
  * longer rows are cut into chunks of chunk_len in-edges taken by whole warps.  ms is the
  * time the autotuner measured (0 otherwise).  With PR_F64 results do not depend on any of

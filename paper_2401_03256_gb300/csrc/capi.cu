@@ -382,6 +382,22 @@ static pr_status create_impl(uint32_t n, int64_t m, const uint32_t *src, const u
         if (rc == PR_OK && (best < 0 || cost[k][1] < cost[best][1])) best = k;
       }
       bool keep = rc == PR_OK && best >= 0 && (p.vertex_order >= 2 || cost[best][1] * 20 < cost[best][0] * 19);
+      // single-graph self-loop handles sweep with the contributions of the first vertices in
+      // shared memory; the hot vertices go first in the numbering that is kept
+      if (keep && !comp_n && !g.teleport) {
+        if (g.f32) {
+          e = cudaMalloc((void **)&g.lab, 4ull * n);
+          if (e == cudaSuccess) e = cudaMalloc((void **)&g.at, 4ull * n);
+          if (e != cudaSuccess) rc = prdf::cuda_fail(&g0, e, "vertex numbering");
+        }
+        if (rc == PR_OK) rc = prdf::hot_order(&g0, prdf::hot_limit(g.f32), cp[best], ci[best], &g.hot, g.lab, g.at);
+        keep = rc == PR_OK;
+        if (!g.hot) {
+          cudaFree(g.lab);
+          cudaFree(g.at);
+          g.lab = g.at = nullptr;
+        }
+      }
       for (int k = 0; k < 2; k++) {
         if (keep && k == best) {
           g.perm = cp[k];

@@ -93,11 +93,12 @@ __global__ void k_compact_unique(const uint64_t *keys, const uint32_t *pos, uint
   if (i == m - 1) *count = pos[i] + f;
 }
 
-__global__ void k_transpose_keys(const uint64_t *keys, uint64_t m, int b, uint64_t *out) {
+// (v, u) keys; u by its place in the in-rows' order (lab), where that is another than by id
+__global__ void k_transpose_keys(const uint64_t *keys, uint64_t m, int b, const uint32_t *lab, uint64_t *out) {
   uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m) return;
   uint64_t k = keys[i], mask = (1ull << b) - 1;
-  out[i] = ((k & mask) << b) | (k >> b);
+  out[i] = ((k & mask) << b) | (lab ? (uint64_t)lab[k >> b] : k >> b);
 }
 
 // off[r] = index of the first key of row r (rows are key >> b); off[n] = m.
@@ -120,12 +121,13 @@ __global__ void k_row_desc(const uint32_t *start, const uint32_t *off, uint32_t 
 }
 
 __global__ void k_scatter_cols(const uint64_t *keys, uint64_t m, int b, const uint32_t *off, const uint2 *rd,
-                               uint32_t *col) {
+                               uint32_t *col, const uint32_t *at) {
   uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m) return;
   uint64_t k = keys[i];
   uint32_t r = (uint32_t)(k >> b);
-  col[rd[r].x + (uint32_t)(i - off[r])] = (uint32_t)(k & ((1ull << b) - 1));
+  const uint32_t c = (uint32_t)(k & ((1ull << b) - 1));
+  col[rd[r].x + (uint32_t)(i - off[r])] = at ? at[c] : c;
 }
 
 template <bool F32>
@@ -247,14 +249,15 @@ __global__ void k_last_op(const uint64_t *keys, const uint32_t *vals, uint64_t N
 // Tagged change keys: (key << 1) | is_insertion, in row-major (u, v) order and a
 // transposed (v, u) copy.
 __global__ void k_emit_changes(const uint64_t *keys, const uint32_t *vals, uint64_t N, const uint32_t *flags,
-                               const uint32_t *pos, int b, uint64_t *chg, uint64_t *chg_t, ApplyCtl *actl) {
+                               const uint32_t *pos, int b, const uint32_t *lab, uint64_t *chg, uint64_t *chg_t,
+                               ApplyCtl *actl) {
   uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   if (flags[i]) {
     const uint64_t k = keys[i];
     const uint64_t tag = vals[i] & 1u;
     const uint64_t mask = (1ull << b) - 1;
-    const uint64_t kt = ((k & mask) << b) | (k >> b);
+    const uint64_t kt = ((k & mask) << b) | (lab ? (uint64_t)lab[k >> b] : k >> b);
     chg[pos[i]] = (k << 1) | tag;
     chg_t[pos[i]] = (kt << 1) | tag;
     if (!tag) atomicAdd(&actl->n_eff_del, 1u);
@@ -317,6 +320,7 @@ struct RowHook {
   uint32_t gmax, chunk;       // sweep tiers of the handle (sweep_tier)
   uint4 *items;               // in-rows: sweep items to patch (tier and chunk count unchanged)
   const uint32_t *item_pos;
+  const uint32_t *lab, *at;   // in-rows ordered by another key than the id (see the graph handle), or null
 };
 
 __device__ __forceinline__ int degree_bin(uint32_t d, uint32_t lo, uint32_t hi) {
@@ -354,7 +358,10 @@ __device__ void merge_row(uint32_t s, uint2 *rd, uint32_t *cap, uint32_t *col, c
   __syncthreads();
   if (!s_ok) return;  // no room: the row is left as it was and the host reports the failure
   if (len > kSmemRow) src_row = big + s_big;
-  for (uint32_t j = tid; j < len; j += kMergeThreads) src_row[j] = col[d.x + j];
+  for (uint32_t j = tid; j < len; j += kMergeThreads) {
+    const uint32_t x = col[d.x + j];
+    src_row[j] = hook.lab ? hook.lab[x] : x;
+  }
   __syncthreads();
   uint32_t *dst = col + s_dest;
   // A thread's entries ascend, so the first change with column >= x lies at or after the
@@ -377,7 +384,7 @@ __device__ void merge_row(uint32_t s, uint2 *rd, uint32_t *cap, uint32_t *col, c
     if (lo < e && chg_col(chg[lo], b) == x) continue;  // deleted
     uint32_t ib = tagpref[lo] - tagpref[s0];
     uint32_t db = (lo - s0) - ib;
-    dst[j - db + ib] = x;
+    dst[j - db + ib] = hook.at ? hook.at[x] : x;
   }
   for (uint32_t q = s0 + tid; q < e; q += kMergeThreads) {
     uint64_t c = chg[q];
@@ -390,7 +397,7 @@ __device__ void merge_row(uint32_t s, uint2 *rd, uint32_t *cap, uint32_t *col, c
     }
     uint32_t ib = tagpref[q] - tagpref[s0];
     uint32_t db = (q - s0) - ib;
-    dst[lo - db + ib] = y;
+    dst[lo - db + ib] = hook.at ? hook.at[y] : y;
   }
   if (hook.is_out) {
     for (uint32_t q = s0 + tid; q < e; q += kMergeThreads) {
@@ -637,7 +644,7 @@ __global__ void k_compact_ids(const uint32_t *flags, const uint32_t *pos, uint32
 // ------------------------------------------------------------------ host side ---
 
 static pr_status build_adj(Graph *g, const uint64_t *keys, uint64_t m, Adj &A, uint32_t *off, uint32_t *tmp,
-                           uint32_t *scan_tmp) {
+                           uint32_t *scan_tmp, const uint32_t *at) {
   const uint32_t n = g->n;
   cudaStream_t st = g->st;
   CK(dalloc(&A.rd, n));
@@ -660,7 +667,7 @@ static pr_status build_adj(Graph *g, const uint64_t *keys, uint64_t m, Adj &A, u
   CK(dalloc(&A.col, A.col_cap));
   CK(cudaMemsetAsync(A.col, 0, sizeof(uint32_t) * A.col_cap, st));
   k_row_desc<<<grid_for(n), 256, 0, st>>>(tmp, off, n, A.rd); count_launch();
-  k_scatter_cols<<<grid_for(m), 256, 0, st>>>(keys, m, g->b, off, A.rd, A.col); count_launch();
+  k_scatter_cols<<<grid_for(m), 256, 0, st>>>(keys, m, g->b, off, A.rd, A.col, at); count_launch();
   A.used = total;
   A.garbage = 0;
   CK(cudaGetLastError());
@@ -728,15 +735,15 @@ pr_status graph_build(Graph *g, uint64_t m_in, const uint32_t *src_d, const uint
     }
     g->m = m;
     // out-adjacency from keys sorted by (u, v)
-    rc = build_adj(g, other, m, g->out, flags, pos, stmp);
+    rc = build_adj(g, other, m, g->out, flags, pos, stmp, nullptr);
     if (rc != PR_OK) break;
     // in-adjacency from transposed keys sorted by (v, u)
     if (m) {
-    k_transpose_keys<<<grid_for(m), 256, 0, st>>>(other, m, g->b, sorted);
+    k_transpose_keys<<<grid_for(m), 256, 0, st>>>(other, m, g->b, g->lab, sorted);
     count_launch();
   }
     uint64_t *tsorted = sort_u64(sorted, other, m, 2 * g->b, hist, stmp, st);
-    rc = build_adj(g, tsorted, m, g->in, flags, pos, stmp);
+    rc = build_adj(g, tsorted, m, g->in, flags, pos, stmp, g->at);
     if (rc != PR_OK) break;
     e = cudaStreamSynchronize(st);
   } while (0);
@@ -881,7 +888,7 @@ pr_status graph_apply(Graph *g, uint64_t nd, const uint32_t *ds, const uint32_t 
   sort_u64_kv(&keys, &vals, s.tmp, s.vals2, N, 2 * b, s.radix_hist, s.scan_tmp, st);
   k_last_op<<<grid_for(N), 256, 0, st>>>(keys, vals, N, g->out.rd, g->out.col, b, s.flags); count_launch();
   exclusive_scan_u32(s.flags, s.pos, N, s.scan_tmp, st);
-  k_emit_changes<<<grid_for(N), 256, 0, st>>>(keys, vals, N, s.flags, s.pos, b, s.chg, s.chg_t, g->actl); count_launch();
+  k_emit_changes<<<grid_for(N), 256, 0, st>>>(keys, vals, N, s.flags, s.pos, b, g->lab, s.chg, s.chg_t, g->actl); count_launch();
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(&h, g->actl, sizeof(ApplyCtl), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -966,10 +973,11 @@ pr_status graph_apply(Graph *g, uint64_t nd, const uint32_t *ds, const uint32_t 
   if (g->f32) {
     using S = Store<true>;
     RowHook<true> ho{true, g->p.alpha, (S::A *)g->adeg, (S::R *)g->R[0], (S::C *)g->C[0], (S::C *)g->C[1],
-                     g->pend_src, g->pend_tgt, g->pend_cap, lo, hi_b, g->group_max, g->chunk_len, nullptr, nullptr};
+                     g->pend_src, g->pend_tgt, g->pend_cap, lo, hi_b, g->group_max, g->chunk_len, nullptr, nullptr,
+                     nullptr, nullptr};
     RowHook<true> hin{false,   g->p.alpha,   nullptr,      nullptr,       nullptr, nullptr, nullptr,
                       nullptr, 0,            lo,           hi_b,          g->group_max, g->chunk_len,
-                      g->items, g->item_pos};
+                      g->items, g->item_pos, g->lab,       g->at};
     CK(cudaMemsetAsync(&dctl->n_long, 0, 4, st));
     k_merge<true><<<K, kMergeThreads, 0, st>>>(g->out.rd, g->out.cap, g->out.col, co, b, seg_o, &dctl->n_seg_out,
                                                tp_o, &dctl->tail_out, &dctl->garbage_out, g->big, &dctl->big_cursor,
@@ -991,10 +999,11 @@ pr_status graph_apply(Graph *g, uint64_t nd, const uint32_t *ds, const uint32_t 
   } else {
     using S = Store<false>;
     RowHook<false> ho{true, g->p.alpha, (S::A *)g->adeg, (S::R *)g->R[0], (S::C *)g->C[0], (S::C *)g->C[1],
-                      g->pend_src, g->pend_tgt, g->pend_cap, lo, hi_b, g->group_max, g->chunk_len, nullptr, nullptr};
+                      g->pend_src, g->pend_tgt, g->pend_cap, lo, hi_b, g->group_max, g->chunk_len, nullptr, nullptr,
+                     nullptr, nullptr};
     RowHook<false> hin{false,   g->p.alpha,   nullptr,      nullptr,       nullptr, nullptr, nullptr,
                        nullptr, 0,            lo,           hi_b,          g->group_max, g->chunk_len,
-                       g->items, g->item_pos};
+                       g->items, g->item_pos, nullptr,      nullptr};
     CK(cudaMemsetAsync(&dctl->n_long, 0, 4, st));
     k_merge<false><<<K, kMergeThreads, 0, st>>>(g->out.rd, g->out.cap, g->out.col, co, b, seg_o, &dctl->n_seg_out,
                                                 tp_o, &dctl->tail_out, &dctl->garbage_out, g->big, &dctl->big_cursor,
@@ -1293,6 +1302,8 @@ void graph_free(Graph *g) {
   cudaFree(g->gen_tmp2);
   cudaFree(g->perm);
   cudaFree(g->inv);
+  cudaFree(g->lab);
+  cudaFree(g->at);
   cudaFree(g->scan_tmp);
   if (g->cg_exec) cudaGraphExecDestroy(g->cg_exec);
   if (g->cg) cudaGraphDestroy(g->cg);

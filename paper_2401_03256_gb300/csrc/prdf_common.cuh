@@ -146,6 +146,7 @@ struct RankCtl {
   uint32_t xneed[kMaxIterLimit + 2];                  // continuation: a recorded expansion would mark
   // per-iteration sweep launches (sweep.cu): what one launch leaves for the next
   uint32_t ticket;        // blocks of the current sweep launch that have finished
+  uint32_t lbar;          // grid barrier arrivals of the current run of iterations (k_loop)
   uint32_t it_cur;        // iteration the next sweep launch computes
   uint32_t sw_all[3];     // sweep items per tier (all vertices)
   uint32_t sw_off[2];     // first item of tiers 1 and 2 (in the item and compacted arrays)

@@ -45,6 +45,10 @@ struct Graph {
   // null when the handle keeps the caller's numbering
   uint32_t *perm = nullptr, *inv = nullptr;
   std::vector<uint32_t> perm_h;
+  uint32_t hot = 0;                  // vertices of largest out-degree numbered first (multiple of 4; order.cu)
+  // FP32 handles with hot vertices: in-rows are ordered by the numbering without the hot part
+  // (lab[v] = v's place in it, at[place] = v), so that float sums are added in its order
+  uint32_t *lab = nullptr, *at = nullptr;
   // Sweep items (16 B each) in tier order: tier 0 and 1 items {v, start, len, 0}, then the
   // chunk_len-edge chunks of tier-2 rows {v, start of chunk, len | index in row << 10 |
   // several-chunks flag << 31, chunk number}.  items_cmp holds the affected subset during
@@ -116,10 +120,9 @@ struct Graph {
   // iterations and the CUDA graphs that loop over the iterations on the device
   uint8_t *emap = nullptr;           // [2][n] rank change above tau_f, by iteration parity; 0 between calls
   void *loops = nullptr;             // sweep.cu's cached graphs
-  int sweep_grid = 0;                // blocks of a full-sweep launch
-  int dfsweep_grid = 0;              // blocks of an all-item dense Dynamic Frontier sweep launch
-  int cmpsweep_grid = 0;             // blocks of a compacted dense Dynamic Frontier sweep launch
+  int loop_grid = 0;                 // blocks of a run of iterations (one persistent launch)
   int pro_grid = 0;                  // blocks of the cooperative prologue launch
+  int pro_grid_max = 0;              // blocks of it that can be resident
   bool loop_sweeps = true;           // single-graph self-loop handles iterate in per-iteration launches
   std::string err;
 };
@@ -135,6 +138,13 @@ constexpr int kOrderFromMax = 0, kOrderFromSeeds = 1, kOrderPerGraph = 2;
 pr_status vertex_order(Graph *g, int kind, uint32_t *perm, uint32_t *inv,
                        const std::vector<uint32_t> *comp_n = nullptr);
 pr_status order_cost(Graph *g, const uint32_t *perm, const uint32_t *inv, uint64_t cost[2]);  // order.cu, on a built graph
+// Puts the vertices of largest out-degree first in the numbering (perm, inv), up to hot_max of
+// them, the rest in the order they had; *hot = their number, or 0 (numbering unchanged) where
+// their out-edges are too few to matter.
+// lab and at (null, or n each) receive the order before: lab[new number] = old, at[old] = new.
+pr_status hot_order(Graph *g, uint32_t hot_max, uint32_t *perm, uint32_t *inv, uint32_t *hot, uint32_t *lab,
+                    uint32_t *at);
+uint32_t hot_limit(bool f32);  // sweep.cu: contributions a block's shared-memory copy holds
 void map_ids(const uint32_t *inv, uint32_t *a, uint64_t m, cudaStream_t st);
 pr_status graph_export(Graph *g, int dir, uint64_t *offs_h, uint32_t *cols_h);
 pr_status graph_refresh_ident(Graph *g);
@@ -161,6 +171,7 @@ bool sweep_eligible(const Graph *g);  // single graph, self-loop mode, no graph-
 pr_status sweep_full(Graph *g, bool from_init);                  // all vertices, every iteration
 pr_status sweep_dense(Graph *g, RankMode mode, const void *rank_args);  // after the marking launch's handoff
 void sweep_free(Graph *g);
+void sweep_share(Graph *g, int slots);  // cooperative launches of at most 1/slots of the device
 
 }  // namespace prdf
 

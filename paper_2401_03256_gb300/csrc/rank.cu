@@ -1304,6 +1304,14 @@ pr_status rank_run(Graph *g, RankMode mode, pr_stats *stats) {
   count_launches(g->ctl_h->launches);
   const RankCtl &h = *g->ctl_h;
   if (h.err) {
+    // the blocks left where they were: the per-call marks and the chunk counters start clean again
+    const uint64_t words = ((uint64_t)g->n + 31) / 32;
+    CK(cudaMemsetAsync(g->bitmap, 0, 4 * words, g->st));
+    CK(cudaMemsetAsync(g->xbits, 0, 4 * words, g->st));
+    CK(cudaMemsetAsync(g->stamp, 0xFF, 2ull * g->n, g->st));
+    CK(cudaMemsetAsync(g->chunk_done, 0, 4ull * g->n, g->st));
+    if (g->emap) CK(cudaMemsetAsync(g->emap, 0, 2ull * g->n, g->st));
+    CK(cudaStreamSynchronize(g->st));
     g->err = (h.err & 1u) ? "rank kernel: a grid barrier wait timed out"
                           : "sweep kernel: a staged copy into shared memory did not complete";
     return PR_ERR_DEVICE_TIMEOUT;

@@ -1,15 +1,14 @@
-// sweep.cu - rank iterations as one launch each, looped on the device by a CUDA graph.
+// sweep.cu - the rank iterations of single-graph handles in self-loop mode.
 //
 // Static and Naive-dynamic PageRank (Section 3.1, Section 3.3.1) and the dense iterations
 // of Dynamic Frontier (Algorithm 1), its asynchronous form (Section 4.2) and Dynamic
-// Traversal (Section 3.3.2) run here on single-graph handles in self-loop mode.  One
-// iteration of Eq. 1 is one launch of k_sweep: no grid barrier and no loop state, so its
-// register budget allows five resident blocks per SM (the persistent kernel holds four),
-// and the dependent item -> column -> contribution loads of the sweep have more warps to
-// overlap them.  The last block to finish an iteration reads its L-inf
-// change, decides whether another iteration follows (L-inf <= tau stops, as does
-// max_iter) and sets the condition of the graph's WHILE node; the host is not involved
-// between iterations.
+// Traversal (Section 3.3.2) run here.  An iteration of Eq. 1 is one pass over sweep items
+// (sweep_pass).  Iterations that need nothing from other kernels in between (all of Static
+// and Naive-dynamic, the settled iterations of a dense Dynamic Frontier call) follow one
+// another in one persistent cooperative launch (k_loop), a grid barrier apart; the
+// iterations of a growing Dynamic Frontier set are a launch each (k_sweep).  A CUDA graph with
+// conditional nodes strings these launches together on the device; the host is not
+// involved between iterations.
 //
 // The dense iterations of a Dynamic Frontier call grow the affected set in one of two
 // ways, which give the same set: Algorithm 1 marks the out-neighbours of every vertex
@@ -27,7 +26,7 @@
 // few expansions without long out-rows by a plain launch, the rest by a cooperative one).
 // Leaving pull for push rebuilds the compacted items, as does a set that grew by more
 // than 1/16 since they were last rebuilt.  The settled compacted iterations, which need
-// no prologue, run in an inner loop of the graph.  Sums are taken per vertex exactly as in the
+// no prologue, stay in one k_loop launch.  Sums are taken per vertex exactly as in the
 // persistent kernel's dense sweeps, so results equal a single marking launch bit for bit.
 #include <cstring>
 #include <vector>
@@ -36,19 +35,17 @@
 
 namespace prdf {
 
-#ifndef PRDF_SWEEP_MIN_BLOCKS
-#define PRDF_SWEEP_MIN_BLOCKS 5  // resident blocks per SM the full sweep's register budget allows
-#endif
-#ifndef PRDF_DF_MIN_BLOCKS
-#define PRDF_DF_MIN_BLOCKS 5  // all-item Dynamic Frontier sweeps: five (some spills, measured faster than four)
-#endif
-constexpr int kSweepMinBlocks = PRDF_SWEEP_MIN_BLOCKS;
-constexpr int kDfMinBlocks = PRDF_DF_MIN_BLOCKS;
+// One block of 32 warps per SM, so that the SM holds one copy of the hot contributions.  The
+// sweep waits on memory: R-MAT scale 22, 64-bit, full sweep 0.235 ms with 32 warps of 64
+// registers, 0.248 with 28 of 72, 0.270 with 24 of 80, 0.286 with 16; two blocks of 20 warps and
+// 48 registers (spills, two copies of 64 KB) 0.234.
+constexpr int kSweepBlock = 1024;
+constexpr int kSweepWarps = kSweepBlock / 32;
 constexpr uint32_t kPullDiv = 256;  // more than n / kPullDiv first expansions: the next iteration pulls
 constexpr uint32_t kPullMin = 64;   // and at least this many
 constexpr uint32_t kLightPush = 16384;  // at most this many first expansions: the light push may mark them
 
-// Kernel parameters of k_sweep (fixed for a handle until a buffer moves; the per-call
+// Kernel parameters of a sweep (fixed for a handle until a buffer moves; the per-call
 // sizes travel in the control block).
 template <bool F32>
 struct SweepArgs {
@@ -71,6 +68,7 @@ struct SweepArgs {
   uint8_t *emap;
   const uint2 *out_rd;     // out-row descriptors (the compacted iterations' expansion path reads lengths)
   RankCtl *ctl;
+  uint32_t hot;            // contributions of vertices [0, hot) are kept in shared memory
   typename S::R base;      // (1 - alpha) / n
   typename Num<F32>::B ftol;
   unsigned long long tol_key;
@@ -78,7 +76,6 @@ struct SweepArgs {
   uint32_t chunk;          // edges per chunk of a tier-2 row
   int max_iter;
   cudaGraphConditionalHandle h_loop, h_pro, h_mode, h_fin;
-  cudaGraphConditionalHandle h_inner;  // dense loops: the next iteration is a plain compacted one
 };
 
 // First expansions found by a dense sweep, appended to the expansion list (one atomic per
@@ -101,10 +98,11 @@ __device__ __forceinline__ void note_expansion(RankCtl *ctl, uint32_t *xlist, bo
   if (base + __popc(mask) >= cap_end) xfull = true;
 }
 
-// End of an iteration, run by one thread of the last block to finish: L-inf test, the
-// next iteration's way of marking (dense Dynamic Frontier), trace, loop condition.
-template <bool F32, bool DF>
-__device__ void sweep_decide(const SweepArgs<F32> &a, uint32_t it, bool all_items) {
+// End of an all-item iteration, or of a run of compacted iterations it_first ... it, by one
+// thread of the last block to finish: L-inf test, the next iteration's way of marking, trace,
+// loop condition.
+template <bool F32>
+__device__ void sweep_decide(const SweepArgs<F32> &a, uint32_t it_first, uint32_t it, bool all_items) {
   RankCtl *ctl = a.ctl;
   const unsigned long long dR = __ldcg(&ctl->dR_bits[it]);
   const uint32_t iters = it + 1;
@@ -116,104 +114,122 @@ __device__ void sweep_decide(const SweepArgs<F32> &a, uint32_t it, bool all_item
   ctl->last_key = dR;
   ctl->it_cur = iters;
   ctl->ticket = 0;
-  ctl->bar = 0;  // a prologue's grid barriers count from zero
+  ctl->bar = 0;  // a prologue's grid barriers count from zero, and so do a run's
+  ctl->lbar = 0;
+  ctl->launches += 1;
+  uint32_t total = 0;
+  for (int b = 0; b < 3; b++) {  // only the first iteration of a run has marks of its own
+    const uint32_t d = __ldcg(&ctl->dcnt[b]) + __ldcg(&ctl->tail[it_first][b]);
+    ctl->dcnt[b] = d;
+    ctl->final_cnt[b] = d;
+    total += d;
+  }
+  const uint32_t jt = __ldcg(&ctl->jtotal) + __ldcg(&ctl->tail[it_first][3]);
+  ctl->jtotal = jt;
+  total += jt;
+  if (all_items) {
+    ctl->t_ns[it + 2] = globaltimer_ns();
+  } else {
+    // compacted iterations swept exactly the compacted items (counted here, not by the
+    // sweep: its loops keep the registers of a full sweep)
+    const unsigned long long runs = it - it_first + 1;
+    ctl->vproc += runs * (__ldcg(&ctl->cmp_total) + __ldcg(&ctl->app_since));
+    ctl->eproc += runs * __ldcg(&ctl->cmp_edges);
+  }
+  ctl->eprev = __ldcg(&ctl->eproc);
+  for (uint32_t k = it_first; k <= it; k++) {
+    ctl->it_aff[k] = total;
+    ctl->it_kind[k] = (uint8_t)(k == it_first ? __ldcg(&ctl->kind_cur) : 5u);
+  }
+  uint32_t pro = 0, all = 1;
+  if (!cont && __ldcg(&ctl->dexpand)) {
+    // the loop ends: this iteration's first expansions still mark their out-neighbours
+    // (the affected set of Algorithm 1 includes the last iteration's marks), by a pull
+    // over every tier when the change flags were recorded and the list may be partial,
+    // by a push otherwise
+    const uint32_t xend = __ldcg(&ctl->xcnt), lo = __ldcg(&ctl->xdone);
+    const uint32_t x = xend - lo;
+    const bool recorded = __ldcg(&ctl->erec) != 0;
+    const uint32_t pull_at = max(kPullMin, a.n / kPullDiv);
+    ctl->xdone = xend;
+    ctl->compact_now = 0;
+    ctl->push_items = 0;
+    uint32_t fin = 0;
+    if (x && recorded && (x > pull_at || x > __ldcg(&ctl->xcap))) {
+      ctl->pull_check = 1;
+      ctl->pull_all = 1;
+      fin = 1;
+    } else if (x) {
+      ctl->push_lo = lo;
+      ctl->push_n = x;
+      fin = 2;
+    }
+    cudaGraphSetConditional(a.h_fin, fin);
+  }
+  if (cont) {
+    const uint32_t xend = __ldcg(&ctl->xcnt), lo = __ldcg(&ctl->xdone);
+    const uint32_t x = __ldcg(&ctl->dexpand) ? xend - lo : 0u;
+    const bool recorded = __ldcg(&ctl->erec) != 0;
+    const uint32_t pull_at = max(kPullMin, a.n / kPullDiv);
+    ctl->xdone = xend;
+    ctl->pull_check = 0;
+    ctl->erec = 0;
+    ctl->push_lo = lo;
+    ctl->push_n = 0;
+    ctl->compact_now = 0;
+    ctl->push_items = 0;
+    ctl->xcap = 0xFFFFFFFFu;
+    const bool x_long = __ldcg(&ctl->x_long) != 0;
+    ctl->x_long = 0;
+    if (all_items && recorded && x > pull_at) {
+      // many first expansions after an iteration that recorded its change flags: the next
+      // iteration pulls (tiers 0 and 1 inline, tier-2 rows in a prologue); its own first
+      // expansions are listed only while few enough to be pushed
+      ctl->pull_check = 1;
+      ctl->erec = 1;
+      ctl->xcap = pull_at + 1;
+      ctl->kind_cur = 7;
+      pro = 1;
+    } else {
+      // otherwise the compacted items of the affected vertices (rebuilt when this
+      // iteration swept every item: its joins are not among them), with pushed marks
+      // appending their items
+      ctl->push_n = x;
+      ctl->compact_now = all_items ? 1u : 0u;
+      ctl->push_items = all_items ? 0u : 1u;
+      ctl->kind_cur = all_items ? 8u : 5u;
+      pro = (x || all_items) ? 2u : 0u;
+      // a few first expansions after a compacted iteration, none with a long out-row:
+      // the light push (no grid barrier) marks them
+      if (!all_items && x && x <= kLightPush && !x_long) pro = 3u;
+      all = 0;
+    }
+  }
+  cudaGraphSetConditional(a.h_pro, pro);
+  cudaGraphSetConditional(a.h_mode, all);
+  if (!cont) ctl->status = kStatusDone;
+  cudaGraphSetConditional(a.h_loop, cont ? 1u : 0u);
+}
+
+// End of an iteration over every vertex that is a launch of its own.
+template <bool F32>
+__device__ void sweep_decide_every(const SweepArgs<F32> &a, uint32_t it) {
+  RankCtl *ctl = a.ctl;
+  const unsigned long long dR = __ldcg(&ctl->dR_bits[it]);
+  const uint32_t iters = it + 1;
+  const bool conv = dR <= a.tol_key;
+  const bool cont = !conv && (int)iters < a.max_iter && __ldcg(&ctl->err) == 0;
+  ctl->iterations = iters;
+  ctl->converged = conv ? 1u : 0u;
+  ctl->last_key = dR;
+  ctl->it_cur = iters;
+  ctl->ticket = 0;
   ctl->launches += 1;
   ctl->t_ns[it + 2] = globaltimer_ns();
-  if constexpr (DF) {
-    uint32_t total = 0;
-    for (int b = 0; b < 3; b++) {
-      const uint32_t d = __ldcg(&ctl->dcnt[b]) + __ldcg(&ctl->tail[it][b]);
-      ctl->dcnt[b] = d;
-      ctl->final_cnt[b] = d;
-      total += d;
-    }
-    const uint32_t jt = __ldcg(&ctl->jtotal) + __ldcg(&ctl->tail[it][3]);
-    ctl->jtotal = jt;
-    total += jt;
-    if (!all_items) {
-      // a compacted iteration swept exactly the compacted items (counted here, not by the
-      // sweep: its loops keep the registers of a full sweep)
-      ctl->vproc += __ldcg(&ctl->cmp_total) + __ldcg(&ctl->app_since);
-      ctl->eproc += __ldcg(&ctl->cmp_edges);
-    }
-    ctl->eprev = __ldcg(&ctl->eproc);
-    ctl->it_aff[it] = total;
-    ctl->it_kind[it] = (uint8_t)__ldcg(&ctl->kind_cur);
-    uint32_t pro = 0, all = 1;
-    if (!cont && __ldcg(&ctl->dexpand)) {
-      // the loop ends: this iteration's first expansions still mark their out-neighbours
-      // (the affected set of Algorithm 1 includes the last iteration's marks), by a pull
-      // over every tier when the change flags were recorded and the list may be partial,
-      // by a push otherwise
-      const uint32_t xend = __ldcg(&ctl->xcnt), lo = __ldcg(&ctl->xdone);
-      const uint32_t x = xend - lo;
-      const bool recorded = __ldcg(&ctl->erec) != 0;
-      const uint32_t pull_at = max(kPullMin, a.n / kPullDiv);
-      ctl->xdone = xend;
-      ctl->compact_now = 0;
-      ctl->push_items = 0;
-      uint32_t fin = 0;
-      if (x && recorded && (x > pull_at || x > __ldcg(&ctl->xcap))) {
-        ctl->pull_check = 1;
-        ctl->pull_all = 1;
-        fin = 1;
-      } else if (x) {
-        ctl->push_lo = lo;
-        ctl->push_n = x;
-        fin = 2;
-      }
-      cudaGraphSetConditional(a.h_fin, fin);
-    }
-    if (cont) {
-      const uint32_t xend = __ldcg(&ctl->xcnt), lo = __ldcg(&ctl->xdone);
-      const uint32_t x = __ldcg(&ctl->dexpand) ? xend - lo : 0u;
-      const bool recorded = __ldcg(&ctl->erec) != 0;
-      const uint32_t pull_at = max(kPullMin, a.n / kPullDiv);
-      ctl->xdone = xend;
-      ctl->pull_check = 0;
-      ctl->erec = 0;
-      ctl->push_lo = lo;
-      ctl->push_n = 0;
-      ctl->compact_now = 0;
-      ctl->push_items = 0;
-      ctl->xcap = 0xFFFFFFFFu;
-      const bool x_long = __ldcg(&ctl->x_long) != 0;
-      ctl->x_long = 0;
-      if (all_items && recorded && x > pull_at) {
-        // many first expansions after an iteration that recorded its change flags: the next
-        // iteration pulls (tiers 0 and 1 inline, tier-2 rows in a prologue); its own first
-        // expansions are listed only while few enough to be pushed
-        ctl->pull_check = 1;
-        ctl->erec = 1;
-        ctl->xcap = pull_at + 1;
-        ctl->kind_cur = 7;
-        pro = 1;
-      } else {
-        // otherwise the compacted items of the affected vertices (rebuilt when this
-        // iteration swept every item: its joins are not among them), with pushed marks
-        // appending their items
-        ctl->push_n = x;
-        ctl->compact_now = all_items ? 1u : 0u;
-        ctl->push_items = all_items ? 0u : 1u;
-        ctl->kind_cur = all_items ? 8u : 5u;
-        pro = (x || all_items) ? 2u : 0u;
-        // a few first expansions after a compacted iteration, none with a long out-row:
-        // the light push (no grid barrier) marks them
-        if (!all_items && x && x <= kLightPush && !x_long) pro = 3u;
-        all = 0;
-      }
-    }
-    cudaGraphSetConditional(a.h_pro, pro);
-    cudaGraphSetConditional(a.h_mode, all);
-    // a compacted iteration with no prologue next runs in the inner loop, whose iterations
-    // have the launch cost of a full sweep's (one conditional node each)
-    cudaGraphSetConditional(a.h_inner, cont && pro == 0 && all == 0 ? 1u : 0u);
-  } else {
-    ctl->it_aff[it] = a.n;
-    ctl->it_kind[it] = 3;
-    ctl->vproc += a.n;
-    ctl->eproc += __ldcg(&ctl->m_cur);
-  }
+  ctl->it_aff[it] = a.n;
+  ctl->it_kind[it] = 3;
+  ctl->vproc += a.n;
+  ctl->eproc += __ldcg(&ctl->m_cur);
   if (!cont) ctl->status = kStatusDone;
   cudaGraphSetConditional(a.h_loop, cont ? 1u : 0u);
 }
@@ -227,7 +243,7 @@ __device__ void sweep_decide(const SweepArgs<F32> &a, uint32_t it, bool all_item
 // compaction it is rare, and the sweep loops keep the registers of a full sweep.
 __device__ __noinline__ void expand_cmp(RankCtl *ctl, uint16_t *stamp, const uint32_t *xbits, uint32_t *xlist,
                                         uint4 *items_cmp, const uint2 *out_rd, uint32_t v, uint32_t ci,
-                                        bool has_item) {
+                                        bool has_item, uint32_t it) {
   const uint16_t s2 = __ldcg(reinterpret_cast<const unsigned short *>(stamp + v));
   const bool was = (s2 & kStampExp) || ((__ldcg(xbits + (v >> 5)) >> (v & 31)) & 1u);
   if (!was) {
@@ -240,7 +256,10 @@ __device__ __noinline__ void expand_cmp(RankCtl *ctl, uint16_t *stamp, const uin
   if (!want) return;
   const uint32_t lane = threadIdx.x & 31, leader = __ffs(want) - 1;
   uint32_t base = 0;
-  if (lane == leader) base = atomicAdd(&ctl->xcnt, (uint32_t)__popc(want));
+  if (lane == leader) {
+    base = atomicAdd(&ctl->xcnt, (uint32_t)__popc(want));
+    atomicAdd(&ctl->xit[it], (uint32_t)__popc(want));  // ends a run of iterations after this one
+  }
   base = __shfl_sync(mask, base, leader);
   if (!was) {
     const uint32_t x0 = __ldcg(&ctl->xdone), xc = __ldcg(&ctl->xcap);
@@ -250,9 +269,99 @@ __device__ __noinline__ void expand_cmp(RankCtl *ctl, uint16_t *stamp, const uin
   }
 }
 
-// One iteration of Eq. 1 over sweep items.  MODE 0: every vertex (Static, Naive-dynamic).
-// MODE 1: a dense Dynamic Frontier iteration over every item, vertices not affected
-// skipped; when pulling, a tier-0/1 vertex not yet affected first checks its in-row
+// ------------------------------------------------------------ contribution gathers ----
+// The sweep's cost is its gathers: 32 random contributions a warp instruction are 32 lines
+// to look up, one per clock and SM (L1 and L2 both about 75% busy).  A handle's internal
+// numbering puts the vertices of largest out-degree first, and every SM keeps the
+// contributions of the first `hot` vertices in shared memory for the iteration, where 32
+// random reads take a few clocks.  The copy takes part of the SM's L1, which also holds the
+// lines of loads in flight.  Full sweep of R-MAT scale 22 (69 M edges) in 64-bit mode: 0.318 ms with
+// every gather through L1; 0.246 with 64 KB hot (31% of the gathers), 0.238 with 96 KB, 0.234
+// with 128 KB (38%), 0.239 with 160 KB; of 1.3 M vertices and 21.6 M edges in FP32: 0.128;
+// 0.071, 0.068, 0.067, 0.067.
+constexpr uint32_t kHotBytes = 131072;
+static_assert(kHotBytes % 128 == 0, "copied in eight pieces of a multiple of 16 bytes");
+
+// Volatile: the contributions change between the iterations of one launch.
+__device__ __forceinline__ void cold_load(long long &r, const long long *p, bool on, unsigned long long pol) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p ld.global.ca.L2::cache_hint.b64 %0, [%1], %3;\n}\n"
+               : "+l"(r)
+               : "l"(p), "r"((uint32_t)on), "l"(pol));
+}
+__device__ __forceinline__ void cold_load(float &r, const float *p, bool on, unsigned long long pol) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p ld.global.ca.L2::cache_hint.f32 %0, [%1], %3;\n}\n"
+               : "+f"(r)
+               : "l"(p), "r"((uint32_t)on), "l"(pol));
+}
+__device__ __forceinline__ void hot_load(long long &r, uint32_t p, bool on) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p ld.shared.b64 %0, [%1];\n}\n"
+               : "+l"(r)
+               : "r"(p), "r"((uint32_t)on));
+}
+__device__ __forceinline__ void hot_load(float &r, uint32_t p, bool on) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p ld.shared.f32 %0, [%1];\n}\n"
+               : "+f"(r)
+               : "r"(p), "r"((uint32_t)on));
+}
+// s plus the contributions of RUNS column runs, in order: run k holds the entries first + k * stride ...
+// + 3 of a row of len.  The hot ones come from shared memory (sbase) into the registers that
+// the others are then loaded into, all in flight together.
+template <int RUNS, class C>
+__device__ __forceinline__ C gather_runs(C s, const C *Cv, const uint4 *q, uint32_t len, uint32_t first, uint32_t stride,
+                                         uint32_t sbase, uint32_t hot, unsigned long long pol) {
+  C x[RUNS][4];
+#pragma unroll
+  for (int k = 0; k < RUNS; k++) {
+    const uint32_t w[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+      x[k][e] = (C)0;
+      hot_load(x[k][e], sbase + w[e] * (uint32_t)sizeof(C), first + k * stride + e < len && w[e] < hot);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < RUNS; k++) {
+    const uint32_t w[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
+#pragma unroll
+    for (int e = 0; e < 4; e++)
+      cold_load(x[k][e], Cv + w[e], first + k * stride + e < len && w[e] >= hot, pol);
+  }
+#pragma unroll
+  for (int k = 0; k < RUNS; k++) s += ((x[k][0] + x[k][1]) + x[k][2]) + x[k][3];
+  return s;
+}
+
+// The block's copy of the hot contributions: eight bulk copies issued by one thread (blocks
+// start at different pieces), completion on the block's mbarrier, pass number `pass` (from 0) of the
+// launch.  The contributions were written by other SMs through the generic proxy.
+__device__ __forceinline__ void stage_hot(const void *Cin, uint32_t bytes, uint32_t sbase, uint32_t bar) {
+  asm volatile("fence.proxy.async;" ::: "memory");
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+  const uint32_t piece = ((bytes >> 3) + 15u) & ~15u;
+  for (uint32_t k = 0; k < 8; k++) {
+    const uint32_t at = ((k + blockIdx.x) & 7u) * piece;
+    if (at >= bytes) continue;
+    asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(sbase + at),
+                 "l"((const char *)Cin + at), "r"(min(piece, bytes - at)), "r"(bar)
+                 : "memory");
+  }
+}
+
+// What a pass over sweep items needs beside the handle's arguments, and what it leaves.
+template <bool F32>
+struct Pass {
+  uint32_t it, n0, n1, n2, off1, off2;
+  bool expand, pulling, erec;
+  uint32_t cap_end;
+  uint32_t sbase;
+  uint32_t *next;  // shared memory: rounds of each tier the block's warps have taken (0 before a pass)
+  typename Num<F32>::B my_max;
+  uint32_t my_v, my_e, xloc, jloc;
+};
+
+// One iteration of Eq. 1 over sweep items by the whole grid.  MODE 0: every vertex (Static,
+// Naive-dynamic).  MODE 1: a dense Dynamic Frontier iteration over every item, vertices not
+// affected skipped; when pulling, a tier-0/1 vertex not yet affected first checks its in-row
 // against the previous iteration's change flags and joins if one is set (tier-2 rows were
 // decided by the prologue).  MODE 2: a dense iteration over the compacted items of the
 // affected vertices.  Dynamic Frontier modes record change flags when asked, and first
@@ -261,44 +370,25 @@ __device__ __noinline__ void expand_cmp(RankCtl *ctl, uint16_t *stamp, const uin
 // persistent kernel's sweeps: thread rows in runs of eight, 8-lane groups, chunk-edge
 // chunks added in chunk order.
 template <bool F32, int MODE>
-__global__ void __launch_bounds__(kRankBlock, MODE == 1 ? kDfMinBlocks : kSweepMinBlocks) k_sweep(const SweepArgs<F32> a) {
-  constexpr bool DF = MODE != 0, ALL = MODE == 1, CMP = MODE == 2;
+__device__ __forceinline__ void sweep_pass(const SweepArgs<F32> &a, Pass<F32> &io) {
+  constexpr bool ALL = MODE == 1, CMP = MODE == 2;
   using S = Store<F32>;
   using R = typename S::R;
   using C = typename S::C;
   using A = typename S::A;
   using B = typename Num<F32>::B;
-  __shared__ unsigned long long s_key[kWarps];
-  // compacted sweeps: tier-0 tiles of the compacted affected items (32 items of a round),
-  // double-buffered per warp, and their barriers
-  __shared__ __align__(128) uint4 s_items[CMP ? kWarps : 1][2][32];
-  __shared__ __align__(8) unsigned long long s_ibar[CMP ? kWarps : 1][2];
   RankCtl *ctl = a.ctl;
   const uint32_t tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
-  if (CMP && lane == 0) {
-    mbar_init1(smem_addr(&s_ibar[wib][0]));
-    mbar_init1(smem_addr(&s_ibar[wib][1]));
-  }
-  __syncwarp();
-  const uint32_t nwarps = (gridDim.x * kRankBlock) >> 5, gwarp = (blockIdx.x * kRankBlock + tid) >> 5;
-  const uint32_t it = __ldcg(&ctl->it_cur);
+  const uint32_t it = io.it, hot = a.hot, sbase = io.sbase;
   const int par = it & 1;
   const R *Rin = par ? a.R1 : a.R0;
   const C *Cin = par ? a.C1 : a.C0;
   R *Rout = par ? a.R0 : a.R1;
   C *Cout = par ? a.C0 : a.C1;
   const uint4 *T = CMP ? a.items_cmp : a.items;
-  const uint32_t *cnts = CMP ? ctl->cmp_cur : ctl->sw_all;
-  const uint32_t n0 = __ldcg(cnts), n1 = __ldcg(cnts + 1), n2 = __ldcg(cnts + 2);
-  const uint32_t off1 = __ldcg(&ctl->sw_off[0]), off2 = __ldcg(&ctl->sw_off[1]);
-  const bool expand = DF && __ldcg(&ctl->dexpand) != 0;
-  const bool pulling = ALL && __ldcg(&ctl->pull_check) != 0;
-  const bool erec = ALL && __ldcg(&ctl->erec) != 0;
-  uint32_t cap_end = 0;
-  if (ALL) {
-    const uint32_t x0 = __ldcg(&ctl->xdone), xc = __ldcg(&ctl->xcap);
-    cap_end = xc > 0xFFFFFFFFu - x0 ? 0xFFFFFFFFu : x0 + xc;
-  }
+  const uint32_t n0 = io.n0, n1 = io.n1, n2 = io.n2, off1 = io.off1, off2 = io.off2;
+  const bool expand = io.expand, pulling = io.pulling, erec = io.erec;
+  const uint32_t cap_end = io.cap_end;
   bool xfull = false;
   uint32_t xloc = 0, jloc = 0;
   const uint8_t *Eprev = a.emap + (size_t)((it - 1) & 1) * a.n;  // read only when pulling (it > 0)
@@ -324,24 +414,33 @@ __global__ void __launch_bounds__(kRankBlock, MODE == 1 ? kDfMinBlocks : kSweepM
     atomicOr(a.bitmap + (v >> 5), 1u << (v & 31));
     jloc++;
   };
-  // Dynamic Frontier bookkeeping after v's change dr: change flag (iterations that record
-  // them), first-expansion test; true where v's out-row is to be marked from for the first
-  // time.  st = v's stamp as read and xw its word of the bitmap of out-rows the marking
-  // launch scanned (all-item iterations; a joined vertex's stamp is it and it never
-  // expanded); cache = the compacted item's bit (ci = its index), the word read only where
-  // no cache decides
-  auto book = [&](uint32_t v, B dr, uint16_t st, bool joined, uint32_t xw, uint32_t cache, uint32_t ci) -> bool {
+  // All-item iterations, after v's change dr: change flag (iterations that record them),
+  // first-expansion test; true where v's out-row is to be marked from for the first time.
+  // st = v's stamp as read and xw its word of the bitmap of out-rows the marking launch
+  // scanned (a joined vertex's stamp is it and it never expanded)
+  auto book = [&](uint32_t v, B dr, uint16_t st, bool joined, uint32_t xw) -> bool {
     if (!expand) return false;
     const bool big = dr > a.ftol;
     if (erec) Ecur[v] = big ? 1 : 0;
-    if (!big) return false;
-    if (ALL) {
-      if (st & kStampExp) return false;
-      const bool was = !joined && ((xw >> (v & 31)) & 1u);
-      a.stamp[v] = (uint16_t)(st | kStampExp);
-      return !was;
-    }
-    return false;  // compacted iterations: expand_cmp
+    if (!big || (st & kStampExp)) return false;
+    const bool was = !joined && ((xw >> (v & 31)) & 1u);
+    a.stamp[v] = (uint16_t)(st | kStampExp);
+    return !was;
+  };
+  // A tier's rounds (32 items, 4 items, 1 chunk) are dealt to the blocks in turn, starting after
+  // the block that took the last round of the tier before (with few rounds no block gets one
+  // more of every tier); a block's warps take its rounds as they get free, one ahead of the
+  // round they work on, so that the next round's items are on their way.  (Dealt to the warps
+  // beforehand, they waited 13% of an iteration for the slowest: 0.303 ms against 0.238.)
+  const uint32_t nblk = gridDim.x;
+  const uint32_t r0 = (uint32_t)(((uint64_t)n0 + 31) >> 5), r1 = (uint32_t)(((uint64_t)n1 + 3) >> 2);
+  const uint32_t d1 = r0 % nblk, d2 = (uint32_t)(((uint64_t)r0 + r1) % nblk);
+  const uint32_t f1 = blockIdx.x >= d1 ? blockIdx.x - d1 : blockIdx.x + nblk - d1;
+  const uint32_t f2 = blockIdx.x >= d2 ? blockIdx.x - d2 : blockIdx.x + nblk - d2;
+  auto take = [&](int t, uint32_t first) -> uint32_t {  // the warp's next round of tier t
+    uint32_t k = 0;
+    if (lane == 0) k = atomicAdd(io.next + t, 1u);
+    return first + __shfl_sync(kFull, k, 0) * nblk;
   };
 
   // tier 0: one thread per vertex, 32 consecutive items per warp.  In all-item iterations
@@ -351,114 +450,90 @@ __global__ void __launch_bounds__(kRankBlock, MODE == 1 ? kDfMinBlocks : kSweepM
   // vertex's own self-loop.
   //
   // Every tier has the items of its next round on the way while it works on the current
-  // one, so a round's row loads wait for no item: the next round's items are loaded into
-  // registers, except in tier 0 of a compacted sweep, which stages each round's 32
-  // compacted items (512 contiguous bytes) into the warp's shared-memory slot with one
-  // bulk copy issued a round ahead (two slots per warp; round r uses slot r & 1 for the
-  // (r >> 1)-th time, hence that phase parity).
+  // one, so a round's row loads wait for no item.
   const uint4 zero4 = make_uint4(0, 0, 0, 0);
-  const uint32_t sbar = smem_addr(&s_ibar[CMP ? wib : 0][0]), sbuf = smem_addr(&s_items[CMP ? wib : 0][0][0]);
-  uint32_t rr = 0;
-  auto stage = [&](uint32_t first, uint32_t cnt, uint32_t slot) {
-    if (lane == 0) bulk_stage(sbuf + slot * 512u, T + first, cnt * 16u, sbar + slot * 8u);
-  };
-  // wait for round rr's items; on a copy that never lands, record the error, wait once
-  // more (bounded) for the copies in flight and tell the tier to stop
-  auto landed = [&](bool next_staged) -> bool {
-    const uint32_t slot = rr & 1u;
-    if (mbar_wait(sbar + slot * 8u, (rr >> 1) & 1u, kStageTimeoutNs)) return true;
-    if (lane == 0) atomicOr(&ctl->err, 2u);
-    mbar_wait(sbar + slot * 8u, (rr >> 1) & 1u, kStageTimeoutNs);
-    if (next_staged) mbar_wait(sbar + (slot ^ 1u) * 8u, ((rr + 1) >> 1) & 1u, kStageTimeoutNs);
-    return false;
-  };
   auto tier0 = [&]() {
-  uint4 item_nx = zero4;
-  if constexpr (CMP) {
-    if ((uint64_t)gwarp * 32 < n0) stage(gwarp * 32, min(32u, n0 - gwarp * 32), rr & 1u);
-  } else {
-    if ((uint64_t)gwarp * 32 + lane < n0) item_nx = ldcg(T + gwarp * 32 + lane);
-  }
-  for (uint32_t b0 = gwarp * 32; b0 < n0; b0 += nwarps * 32, rr++) {
-    const uint32_t i = b0 + lane;
-    bool act = false, join = false, push = false;
-    uint4 item;
-    if constexpr (CMP) {
-      const uint32_t slot = rr & 1u;
-      __syncwarp();  // the other slot was read by every lane in the previous round
-      const bool nx = (uint64_t)b0 + nwarps * 32 < n0;
-      if (nx) stage(b0 + nwarps * 32, min(32u, n0 - b0 - nwarps * 32), slot ^ 1u);
-      if (!landed(nx)) break;
-      item = i < n0 ? s_items[wib][slot][lane] : zero4;
-    } else {
-      item = item_nx;
-      if ((uint64_t)i + nwarps * 32 < n0) item_nx = ldcg(T + i + nwarps * 32);
-    }
-    uint16_t st = 0;
-    uint32_t xw = 0;
-    R rold = (R)0;
-    A ad = (A)0;
-    uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0;
-    if (i < n0) {
-      const uint32_t v = item.x;
-      if (ALL) {
-        st = ldcg(a.stamp + v);
-        if (expand) xw = __ldcg(a.xbits + (v >> 5));
-      }
-      rold = ldcg(Rin + v);
-      ad = __ldg(a.adeg + v);
-      if (item.z > 1 && item.z <= 8) {  // a one-entry row is v's self-loop: no column needed
-        q0 = ld_cols(a.in_col + item.y, pol_cols);
-        if (item.z > 4) q1 = ld_cols(a.in_col + item.y + 4, pol_cols);
-      }
-      act = !ALL || (st & kStampIt) <= itk;
-      if (ALL && !act && pulling && item.z > 1) {
-        if (item.z <= 8) {
-          const uint32_t w[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
-          uint32_t any = 0;  // every flag load issued at once (no chain of dependent loads)
-#pragma unroll
-          for (uint32_t j = 0; j < 8; j++) any |= j < item.z ? (uint32_t)__ldcg(Eprev + w[j]) : 0u;
-          join = any != 0;
-        } else {
-          for (uint32_t j = 0; j < item.z && !join; j++) join = __ldcg(Eprev + __ldg(a.in_col + item.y + j)) != 0;
+    uint32_t k = take(0, blockIdx.x);
+    uint4 item_nx = k < r0 && k * 32 + lane < n0 ? ldcg(T + k * 32 + lane) : zero4;
+    while (k < r0) {
+      const uint32_t i = k * 32 + lane;
+      bool act = false, join = false, push = false;
+      const uint4 item = item_nx;
+      k = take(0, blockIdx.x);
+      if (k < r0 && k * 32 + lane < n0) item_nx = ldcg(T + k * 32 + lane);
+      uint16_t st = 0;
+      uint32_t xw = 0;
+      R rold = (R)0;
+      A ad = (A)0;
+      uint4 q[2] = {zero4, zero4};
+      if (i < n0) {
+        const uint32_t v = item.x;
+        if (ALL) {
+          st = ldcg(a.stamp + v);
+          if (expand) xw = __ldcg(a.xbits + (v >> 5));
         }
-        if (join) join_now(v);
+        rold = ldcg(Rin + v);
+        ad = __ldg(a.adeg + v);
+        if (item.z > 1) {  // a one-entry row is v's self-loop: no column needed
+          q[0] = ld_cols(a.in_col + item.y, pol_cols);
+          if (item.z > 4) q[1] = ld_cols(a.in_col + item.y + 4, pol_cols);
+        }
+        act = !ALL || (st & kStampIt) <= itk;
+        if (ALL && !act && pulling && item.z > 1) {
+          if (item.z <= 8) {
+            const uint32_t w[8] = {q[0].x, q[0].y, q[0].z, q[0].w, q[1].x, q[1].y, q[1].z, q[1].w};
+            uint32_t any = 0;  // every flag load issued at once (no chain of dependent loads)
+#pragma unroll
+            for (uint32_t j = 0; j < 8; j++) any |= j < item.z ? (uint32_t)__ldcg(Eprev + w[j]) : 0u;
+            join = any != 0;
+          } else {
+            for (uint32_t j = 0; j < item.z && !join; j++) join = __ldcg(Eprev + __ldg(a.in_col + item.y + j)) != 0;
+          }
+          if (join) join_now(v);
+        }
       }
+      if (act || join) {
+        const uint32_t v = item.x;
+        C sum = (C)0;
+        if (item.z == 1) {
+          // self-loop mode: the row is v's self-loop, and C[v] is contrib(R[v], A[v]) (stored
+          // that way by the previous iteration), so it is recomputed from the values in hand
+          sum += S::contrib(rold, ad);
+        } else {
+          // runs of eight columns, the first one in hand
+          for (uint32_t j0 = 0;;) {
+            sum = gather_runs<2>(sum, Cin, q, item.z, j0, 4u, sbase, hot, pol_c);
+            if (item.z <= 8) break;
+            if ((j0 += 8) >= item.z) break;
+            q[0] = ld_cols(a.in_col + item.y + j0, pol_cols);
+            if (item.z - j0 > 4) q[1] = ld_cols(a.in_col + item.y + j0 + 4, pol_cols);
+          }
+        }
+        const B dr = finish(v, sum, rold, ad);
+        if constexpr (ALL) push = book(v, dr, join ? itk : st, join, xw);
+        if constexpr (CMP) {
+          if (expand && dr > a.ftol && !item.w)
+            expand_cmp(ctl, a.stamp, a.xbits, a.xlist, a.items_cmp, a.out_rd, v, i, true, it);
+        }
+        if constexpr (ALL) {
+          my_v++;
+          my_e += item.z;
+        }
+      }
+      if constexpr (ALL) note_expansion(ctl, a.xlist, push, item.x, lane, cap_end, xfull, xloc);
     }
-    if (act || join) {
-      const uint32_t v = item.x;
-      C sum;
-      if (item.z == 1) {
-        // self-loop mode: the row is v's self-loop, and C[v] is contrib(R[v], A[v]) (stored
-        // that way by the previous iteration), so it is recomputed from the values in hand
-        sum = (C)0 + S::contrib(rold, ad);
-      } else if (item.z <= 8) {  // the first round of row_sum_thread, from the columns in hand
-        sum = (C)0;
-        sum += gather4(Cin, q0, min(4u, item.z), pol_c);
-        if (item.z > 4) sum += gather4(Cin, q1, min(4u, item.z - 4), pol_c);
-      } else {
-        sum = row_sum_thread(Cin, a.in_col + item.y, item.z, pol_cols, pol_c);
-      }
-      const B dr = finish(v, sum, rold, ad);
-      if constexpr (ALL) push = book(v, dr, join ? itk : st, join, xw, item.w, i);
-      if constexpr (CMP) {
-        if (expand && dr > a.ftol && !item.w) expand_cmp(ctl, a.stamp, a.xbits, a.xlist, a.items_cmp, a.out_rd, v, i, true);
-      }
-      if constexpr (!CMP) my_v++;
-      if constexpr (!CMP) my_e += item.z;
-    }
-    if constexpr (ALL) note_expansion(ctl, a.xlist, push, item.x, lane, cap_end, xfull, xloc);
-  }
   };
 
   // tier 1: rows of lo < len <= group_max (<= kGroupMax) by 8-lane groups, four vertices per warp
   auto tier1 = [&]() {
-      const uint32_t grp = lane >> 3, gl = lane & 7;
-    uint4 item_nx = (uint64_t)gwarp * 4 + grp < n1 ? ldcg(T + off1 + gwarp * 4 + grp) : zero4;
-    for (uint32_t b0 = gwarp * 4; b0 < n1; b0 += nwarps * 4) {
-      const uint32_t i = b0 + grp;
+    const uint32_t grp = lane >> 3, gl = lane & 7;
+    uint32_t k = take(1, f1);
+    uint4 item_nx = k < r1 && k * 4 + grp < n1 ? ldcg(T + off1 + k * 4 + grp) : zero4;
+    while (k < r1) {
+      const uint32_t i = k * 4 + grp;
       const uint4 item = item_nx;
-      if ((uint64_t)i + nwarps * 4 < n1) item_nx = ldcg(T + off1 + i + nwarps * 4);
+      k = take(1, f1);
+      if (k < r1 && k * 4 + grp < n1) item_nx = ldcg(T + off1 + k * 4 + grp);
       bool act = false, join = false;
       uint16_t st = 0;
       uint32_t xw = 0;
@@ -494,25 +569,21 @@ __global__ void __launch_bounds__(kRankBlock, MODE == 1 ? kDfMinBlocks : kSweepM
         if (join && gl == 0) join_now(item.x);
       }
       C sum = (C)0;
-      if (act || join) {
-#pragma unroll
-        for (int r = 0; r < 2; r++) {
-          const uint32_t j = 4 * (gl + 8 * r);
-          if (j < item.z) sum += gather4(Cin, q[r], min(4u, item.z - j), pol_c);
-        }
-      }
+      if (act || join) sum = gather_runs<2>(sum, Cin, q, item.z, 4 * gl, 32u, sbase, hot, pol_c);
 #pragma unroll
       for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
       bool push = false;
       if ((act || join) && gl == 0) {
         const B dr = finish(item.x, sum, rold, ad);
-        if constexpr (ALL) push = book(item.x, dr, join ? itk : st, join, xw, item.w, off1 + i);
+        if constexpr (ALL) push = book(item.x, dr, join ? itk : st, join, xw);
         if constexpr (CMP) {
           if (expand && dr > a.ftol && !item.w)
-            expand_cmp(ctl, a.stamp, a.xbits, a.xlist, a.items_cmp, a.out_rd, item.x, off1 + i, true);
+            expand_cmp(ctl, a.stamp, a.xbits, a.xlist, a.items_cmp, a.out_rd, item.x, off1 + i, true, it);
         }
-        if constexpr (!CMP) my_v++;
-        if constexpr (!CMP) my_e += item.z;
+        if constexpr (ALL) {
+          my_v++;
+          my_e += item.z;
+        }
       }
       if constexpr (ALL) note_expansion(ctl, a.xlist, push, item.x, lane, cap_end, xfull, xloc);
     }
@@ -523,89 +594,82 @@ __global__ void __launch_bounds__(kRankBlock, MODE == 1 ? kDfMinBlocks : kSweepM
   // chunk order
   C *part = a.partials;
   auto tier2 = [&]() {
-  uint4 item_nx = gwarp < n2 ? ldcg(T + off2 + gwarp) : zero4;
-  for (uint32_t k = gwarp; k < n2; k += nwarps) {
-    const uint4 ch = item_nx;
-    if ((uint64_t)k + nwarps < n2) item_nx = ldcg(T + off2 + k + nwarps);
-    const uint32_t v = ch.x;
-    uint16_t st = 0;
-    if (ALL) st = ldcg(a.stamp + v);
-    const uint32_t len = ch.z & 0x3FFu;
-    const bool several = (ch.z >> 31) != 0;
-    R rold = (R)0;
-    A ad = (A)0;
-    uint32_t deg = len, xw = 0;
-    if (lane == 0) {
-      rold = ldcg(Rin + v);
-      ad = __ldg(a.adeg + v);
-      if (several) deg = __ldg(&a.in_rd[v]).y;
-      if (ALL && expand) xw = __ldcg(a.xbits + (v >> 5));
-      if (CMP && expand) st = ldcg(a.stamp + v);
-    }
-    const uint32_t *cols = a.in_col + ch.y;
-    uint4 q[4];
-#pragma unroll
-    for (int r = 0; r < 4; r++) {
-      const uint32_t j = 4 * (lane + 32 * r);
-      if (j < len) q[r] = ld_cols(cols + j, pol_cols);
-    }
-    if (ALL && (st & kStampIt) > itk) continue;  // warp-uniform: not affected
-    C sum = (C)0;
-#pragma unroll
-    for (int r = 0; r < 4; r++) {
-      const uint32_t j = 4 * (lane + 32 * r);
-      if (j < len) sum += gather4(Cin, q[r], min(4u, len - j), pol_c);
-    }
-    sum = warp_sum(sum);
-    bool fin = true;
-    if (several) {
-      const uint32_t nch = (__shfl_sync(kFull, deg, 0) + a.chunk - 1) / a.chunk;
-      uint32_t old = 0;
+    uint32_t k = take(2, f2);
+    uint4 item_nx = k < n2 ? ldcg(T + off2 + k) : zero4;
+    while (k < n2) {
+      const uint4 ch = item_nx;
+      k = take(2, f2);
+      if (k < n2) item_nx = ldcg(T + off2 + k);
+      const uint32_t v = ch.x;
+      uint16_t st = 0;
+      if (ALL) st = ldcg(a.stamp + v);
+      const uint32_t len = ch.z & 0x3FFu;
+      const bool several = (ch.z >> 31) != 0;
+      R rold = (R)0;
+      A ad = (A)0;
+      uint32_t deg = len, xw = 0;
       if (lane == 0) {
-        part[ch.w] = sum;
-        __threadfence();
-        old = atomicAdd(&a.chunk_done[v], 1u);
+        rold = ldcg(Rin + v);
+        ad = __ldg(a.adeg + v);
+        if (several) deg = __ldg(&a.in_rd[v]).y;
+        if (ALL && expand) xw = __ldcg(a.xbits + (v >> 5));
+        if (CMP && expand) st = ldcg(a.stamp + v);
       }
-      old = __shfl_sync(kFull, old, 0);
-      fin = old == nch - 1;
-      if (fin) {
-        __threadfence();
-        const uint32_t first = ch.w - ((ch.z >> 10) & 0x1FFFFFu);
-        C tot = (C)0;
-        for (uint32_t c = lane; c < nch; c += 32) tot += ldcg(part + first + c);
-        sum = warp_sum(tot);
-        if (lane == 0) a.chunk_done[v] = 0;
+      const uint32_t *cols = a.in_col + ch.y;
+      uint4 q[4] = {zero4, zero4, zero4, zero4};
+#pragma unroll
+      for (int r = 0; r < 4; r++) {
+        const uint32_t j = 4 * (lane + 32 * r);
+        if (j < len) q[r] = ld_cols(cols + j, pol_cols);
       }
-    }
-    bool push = false;
-    if (fin && lane == 0) {
-      const B dr = finish(v, sum, rold, ad);
-      if constexpr (ALL) {
-        // chunks have no cache bit: the stamp and the word read with the row decide
-        if (expand) {
-          const bool big = dr > a.ftol;
-          if (erec) Ecur[v] = big ? 1 : 0;
-          if (big && !(st & kStampExp)) {
-            push = !((xw >> (v & 31)) & 1u);
-            a.stamp[v] = (uint16_t)(st | kStampExp);
-          }
+      if (ALL && (st & kStampIt) > itk) continue;  // warp-uniform: not affected
+      // two runs at a time: all four in flight together need 16 more registers (0.238 ms a full
+      // sweep of scale 22 against 0.235)
+      C sum = gather_runs<2>((C)0, Cin, q, len, 4 * lane, 128u, sbase, hot, pol_c);
+      if (len > 256) sum = gather_runs<2>(sum, Cin, q + 2, len, 4 * lane + 256, 128u, sbase, hot, pol_c);
+      sum = warp_sum(sum);
+      bool fin = true;
+      if (several) {
+        const uint32_t nch = (__shfl_sync(kFull, deg, 0) + a.chunk - 1) / a.chunk;
+        uint32_t old = 0;
+        if (lane == 0) {
+          part[ch.w] = sum;
+          __threadfence();
+          old = atomicAdd(&a.chunk_done[v], 1u);
+        }
+        old = __shfl_sync(kFull, old, 0);
+        fin = old == nch - 1;
+        if (fin) {
+          __threadfence();
+          const uint32_t first = ch.w - ((ch.z >> 10) & 0x1FFFFFu);
+          C tot = (C)0;
+          for (uint32_t c = lane; c < nch; c += 32) tot += ldcg(part + first + c);
+          sum = warp_sum(tot);
+          if (lane == 0) a.chunk_done[v] = 0;
         }
       }
-      if constexpr (CMP) {
-        if (expand && dr > a.ftol && !(st & kStampExp))
-          expand_cmp(ctl, a.stamp, a.xbits, a.xlist, a.items_cmp, a.out_rd, v, 0, false);
+      bool push = false;
+      if (fin && lane == 0) {
+        const B dr = finish(v, sum, rold, ad);
+        // chunks have no cache bit: the stamp and the word read with the row decide
+        if constexpr (ALL) push = book(v, dr, st, false, xw);
+        if constexpr (CMP) {
+          if (expand && dr > a.ftol && !(st & kStampExp))
+            expand_cmp(ctl, a.stamp, a.xbits, a.xlist, a.items_cmp, a.out_rd, v, 0, false, it);
+        }
+        if constexpr (ALL) {
+          my_v++;
+          my_e += deg;
+        }
       }
-      if constexpr (!CMP) my_v++;
-      if constexpr (!CMP) my_e += deg;
+      if constexpr (ALL) note_expansion(ctl, a.xlist, push, v, lane, cap_end, xfull, xloc);
     }
-    if constexpr (ALL) note_expansion(ctl, a.xlist, push, v, lane, cap_end, xfull, xloc);
-  }
   };
 
-  // Odd warps take the long rows first: their gathers, bound by the rate of random loads,
-  // then overlap the latency-bound short rows of the even warps (6% less time per full
-  // sweep of R-MAT scale 22 than one order for all warps)
-  if (gwarp & 1) {
+  // Three warps of four take the long rows first: their gathers, bound by the rate of random
+  // loads, then overlap the latency-bound short rows of the fourth.  Full sweep of scale 22:
+  // 0.223 ms; one warp of two 0.228, one of four 0.234, all 0.238, none 0.244.
+  if (wib & 3) {
     tier2();
     tier0();
     tier1();
@@ -614,39 +678,267 @@ __global__ void __launch_bounds__(kRankBlock, MODE == 1 ? kDfMinBlocks : kSweepM
     tier1();
     tier2();
   }
+  io.my_max = my_max;
+  io.my_v = my_v;
+  io.my_e = my_e;
+  io.xloc = xloc;
+  io.jloc = jloc;
+}
 
-  // L-inf of the iteration, counters, and the last block's decision
+// The L-inf change of an iteration from the threads' maxima: one atomic per block.  Called
+// by the whole block; s_key is free after the next block barrier.
+template <bool F32>
+__device__ __forceinline__ void block_max(typename Num<F32>::B my_max, unsigned long long *dR,
+                                          unsigned long long *s_key) {
   unsigned long long m = Num<F32>::key(my_max);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(kFull, m, o));
-  if (lane == 0) s_key[wib] = m;
-  if constexpr (DF) {
-    const unsigned long long vs = warp_sum((unsigned long long)my_v), es = warp_sum((unsigned long long)my_e);
-    const uint32_t js = warp_sum(jloc);
-    if (lane == 0) {
-      if (vs) {
-        atomicAdd(&ctl->vproc, vs);
-        atomicAdd(&ctl->eproc, es);
-      }
-      if (xloc) atomicAdd(&ctl->xcnt, xloc);  // the same in every lane
-      if (js) atomicAdd(&ctl->tail[it][3], js);
-    }
+  if ((threadIdx.x & 31) == 0) s_key[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    m = threadIdx.x < kSweepWarps ? s_key[threadIdx.x] : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(kFull, m, o));
+    if (threadIdx.x == 0 && m) atomicMax(dR, m);
+  }
+}
+
+// A wait for the block's hot contributions that ran out ends the call (error 2); the copies
+// in flight are waited for once more, bounded, before the block gives up its shared memory.
+__device__ __forceinline__ bool hot_landed(RankCtl *ctl, uint32_t bar, uint32_t parity) {
+  if (__all_sync(kFull, mbar_wait(bar, parity, kStageTimeoutNs))) return true;  // the same in the whole warp
+  atomicOr(&ctl->err, 2u);
+  mbar_wait(bar, parity, kStageTimeoutNs);
+  return false;
+}
+
+// One iteration: over every item of a dense Dynamic Frontier call (MODE 1), or over every
+// vertex (MODE 0).  The last block to finish decides how the call goes on.
+template <bool F32, int MODE>
+__global__ void __launch_bounds__(kSweepBlock, 1) k_sweep(const SweepArgs<F32> a) {
+  using C = typename Store<F32>::C;
+  __shared__ unsigned long long s_key[kSweepWarps];
+  __shared__ __align__(8) unsigned long long s_bar;
+  __shared__ uint32_t s_next[3];
+  extern __shared__ __align__(128) unsigned char s_hot[];
+  RankCtl *ctl = a.ctl;
+  const uint32_t tid = threadIdx.x, lane = tid & 31;
+  const uint32_t it = __ldcg(&ctl->it_cur), bar = smem_addr(&s_bar), bytes = a.hot * (uint32_t)sizeof(C);
+  Pass<F32> io{};
+  io.sbase = smem_addr(s_hot);
+  io.next = s_next;
+  if (tid < 3) s_next[tid] = 0;
+  if (bytes && tid == 0) {
+    mbar_init1(bar);
+    stage_hot(it & 1 ? a.C1 : a.C0, bytes, io.sbase, bar);
   }
   __syncthreads();
+  io.it = it;
+  io.n0 = __ldcg(&ctl->sw_all[0]);
+  io.n1 = __ldcg(&ctl->sw_all[1]);
+  io.n2 = __ldcg(&ctl->sw_all[2]);
+  io.off1 = __ldcg(&ctl->sw_off[0]);
+  io.off2 = __ldcg(&ctl->sw_off[1]);
+  io.expand = __ldcg(&ctl->dexpand) != 0;
+  io.pulling = __ldcg(&ctl->pull_check) != 0;
+  io.erec = __ldcg(&ctl->erec) != 0;
+  const uint32_t x0 = __ldcg(&ctl->xdone), xc = __ldcg(&ctl->xcap);
+  io.cap_end = xc > 0xFFFFFFFFu - x0 ? 0xFFFFFFFFu : x0 + xc;
+  if (!bytes || hot_landed(ctl, bar, 0)) sweep_pass<F32, MODE>(a, io);
+  if constexpr (MODE == 0) {
+    block_max<F32>(io.my_max, &ctl->dR_bits[it], s_key);
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      if (atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1) {
+        __threadfence();
+        sweep_decide_every<F32>(a, it);
+      }
+    }
+    return;
+  }
+  const unsigned long long vs = warp_sum((unsigned long long)io.my_v), es = warp_sum((unsigned long long)io.my_e);
+  const uint32_t js = warp_sum(io.jloc);
+  if (lane == 0) {
+    if (vs) {
+      atomicAdd(&ctl->vproc, vs);
+      atomicAdd(&ctl->eproc, es);
+    }
+    if (io.xloc) atomicAdd(&ctl->xcnt, io.xloc);  // the same in every lane
+    if (js) atomicAdd(&ctl->tail[it][3], js);
+  }
+  block_max<F32>(io.my_max, &ctl->dR_bits[it], s_key);
+  __syncthreads();
   if (tid == 0) {
-    unsigned long long bm = 0;
-    for (int w = 0; w < kWarps; w++) bm = max(bm, s_key[w]);
-    if (bm) atomicMax(&ctl->dR_bits[it], bm);
     __threadfence();
     const uint32_t t = atomicAdd(&ctl->ticket, 1u);
     if (t == gridDim.x - 1) {
       __threadfence();
-      sweep_decide<F32, DF>(a, it, ALL);
+      sweep_decide<F32>(a, it, it, true);
     }
   }
 }
 
-// Before the first full-sweep iteration: Static starts from 1/n (both parities); the
+// A run of iterations in one persistent cooperative launch, one grid barrier apart: all
+// iterations of Static and Naive-dynamic (every vertex, from the first to the stop), or
+// compacted Dynamic Frontier iterations until the stop or until a vertex expands for the
+// first time.  One launch per iteration cost about 20 us beside the sweep itself (conditional
+// node, launch, one thread's decision after the last block): 26 us a compacted iteration of
+// an R-MAT graph of 16,384 vertices and 136,000 edges, 7.2 us in a run.
+template <bool F32>
+struct LoopArgs {
+  SweepArgs<F32> a;
+  // every-vertex runs: sizes and start
+  uint32_t n0, n1, n2, m, is_static;
+  typename Store<F32>::R init;
+};
+
+template <bool F32, bool CMP>
+__global__ void __launch_bounds__(kSweepBlock, 1) k_loop(const LoopArgs<F32> p) {
+  using S = Store<F32>;
+  using R = typename S::R;
+  using C = typename S::C;
+  __shared__ unsigned long long s_key[kSweepWarps], s_dR;
+  __shared__ __align__(8) unsigned long long s_bar;
+  __shared__ uint32_t s_x, s_err, s_next[3];
+  extern __shared__ __align__(128) unsigned char s_hot[];
+  const SweepArgs<F32> &a = p.a;
+  RankCtl *ctl = a.ctl;
+  const uint32_t tid = threadIdx.x;
+  const uint32_t gtid = blockIdx.x * kSweepBlock + tid, nthreads = gridDim.x * kSweepBlock;
+  const uint32_t bar = smem_addr(&s_bar), bytes = a.hot * (uint32_t)sizeof(C);
+  if (bytes && tid == 0) mbar_init1(bar);
+  Pass<F32> io{};
+  io.sbase = smem_addr(s_hot);
+  io.next = s_next;
+  if (tid < 3) s_next[tid] = 0;
+  uint32_t it = 0, epoch = 0;
+  // Grid barrier with a bounded wait; false in every thread of the block once the call has an
+  // error.  Thread 0 also reads what the iteration left (slot k): its L-inf change and first
+  // expansions.
+  auto barrier = [&](uint32_t k) -> bool {
+    __syncthreads();
+    epoch++;
+    if (tid == 0) {
+      asm volatile("fence.proxy.async;" ::: "memory");  // the next hot copies read what was written
+      __threadfence();
+      red_release_add_u32(&ctl->lbar, 1u);
+      const uint32_t target = epoch * gridDim.x;
+      const unsigned long long lim = *(volatile unsigned long long *)&ctl->bar_limit_ns;
+      const uint32_t every = lim ? 0u : 127u;
+      unsigned long long t0 = 0;
+      for (uint32_t spins = 1; ld_acquire_u32(&ctl->lbar) < target; spins++) {
+        if (*(volatile uint32_t *)&ctl->err) break;
+        if ((spins & every) == 0) {
+          const unsigned long long t = globaltimer_ns();
+          if (t0 == 0) {
+            t0 = t;
+          } else if (t - t0 > (lim ? lim : kBarrierTimeoutNs)) {
+            atomicExch(&ctl->err_where, epoch);
+            atomicOr(&ctl->err, 1u);
+            break;
+          }
+        }
+      }
+      s_err = *(volatile uint32_t *)&ctl->err;
+      s_dR = __ldcg(&ctl->dR_bits[k]);
+      s_x = CMP ? __ldcg(&ctl->xit[k]) : 0u;
+    }
+    __syncthreads();
+    return s_err == 0;
+  };
+  // an error ends the device-side loop: nothing else would
+  auto give_up = [&]() {
+    if (CMP && tid == 0) {
+      cudaGraphSetConditional(a.h_pro, 0u);
+      cudaGraphSetConditional(a.h_fin, 0u);
+      cudaGraphSetConditional(a.h_loop, 0u);
+    }
+  };
+  if constexpr (CMP) {
+    it = __ldcg(&ctl->it_cur);
+    io.n0 = __ldcg(&ctl->cmp_cur[0]);
+    io.n1 = __ldcg(&ctl->cmp_cur[1]);
+    io.n2 = __ldcg(&ctl->cmp_cur[2]);
+    io.off1 = __ldcg(&ctl->sw_off[0]);
+    io.off2 = __ldcg(&ctl->sw_off[1]);
+    io.expand = __ldcg(&ctl->dexpand) != 0;
+  } else {
+    if (gtid == 0 && ctl->t_ns[0] == 0) ctl->t_ns[0] = globaltimer_ns();  // unless a marking launch ran first
+    io.n0 = p.n0;
+    io.n1 = p.n1;
+    io.n2 = p.n2;
+    io.off1 = p.n0;
+    io.off2 = p.n0 + p.n1;
+    if (p.is_static) {  // ranks restart at 1/n, in both parities
+      for (uint32_t v = gtid; v < a.n; v += nthreads) {
+        const C c = S::contrib(p.init, __ldg(a.adeg + v));
+        a.R0[v] = p.init;
+        a.R1[v] = p.init;
+        a.C0[v] = c;
+        a.C1[v] = c;
+      }
+      if (!barrier(0)) return;
+    }
+    if (gtid == 0) {
+      ctl->t_ns[1] = globaltimer_ns();
+      ctl->status = kStatusDone;
+    }
+    if (a.max_iter <= 0) return;
+  }
+  const uint32_t it_first = it;
+  for (;; it++) {
+    __syncthreads();  // s_next is zero, the block's mbarrier initialised
+    if (bytes && tid == 0) stage_hot(it & 1 ? a.C1 : a.C0, bytes, io.sbase, bar);
+    io.it = it;
+    if (!bytes || hot_landed(ctl, bar, (it - it_first) & 1u)) sweep_pass<F32, CMP ? 2 : 0>(a, io);
+    block_max<F32>(io.my_max, &ctl->dR_bits[it], s_key);  // (a block barrier: every warp has taken its last round)
+    if (tid < 3) s_next[tid] = 0;
+    if (!barrier(it)) {
+      give_up();
+      return;
+    }
+    if (gtid == 0) {
+      ctl->t_ns[it + 2] = globaltimer_ns();
+      if (!CMP) {
+        ctl->it_aff[it] = a.n;
+        ctl->it_kind[it] = 3;
+      }
+    }
+    if (s_dR <= a.tol_key || (int)it + 1 >= a.max_iter || s_x) break;
+  }
+  if constexpr (CMP) {
+    if (tid == 0) {
+      __threadfence();
+      if (atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1) {
+        __threadfence();
+        sweep_decide<F32>(a, it_first, it, false);
+      }
+    }
+  } else {
+    // both parities take the final values
+    const uint32_t k = it + 1;
+    const bool fp = k & 1;
+    const R *Rf = fp ? a.R1 : a.R0;
+    const C *Cf = fp ? a.C1 : a.C0;
+    R *Ro = fp ? a.R0 : a.R1;
+    C *Co = fp ? a.C0 : a.C1;
+    for (uint32_t v = gtid; v < a.n; v += nthreads) {
+      Ro[v] = ldcg(Rf + v);
+      Co[v] = ldcg(Cf + v);
+    }
+    if (gtid == 0) {
+      ctl->iterations = k;
+      ctl->converged = s_dR <= a.tol_key ? 1u : 0u;
+      ctl->last_key = s_dR;
+      ctl->vproc += (unsigned long long)k * a.n;
+      ctl->eproc += (unsigned long long)k * p.m;
+    }
+  }
+}
+
+// Handles tuned with df_split = 0 keep one launch per iteration for Static and Naive-dynamic
+// (k_sweep<F32, 0> between these two).  Before the first iteration: Static starts from 1/n (both parities); the
 // per-call sizes go to the control block, and the loop runs if max_iter > 0.
 template <bool F32>
 struct FullInit {
@@ -719,7 +1011,7 @@ struct DenseInit {
   uint32_t n, m;
   uint32_t traversal;
   int max_iter;
-  cudaGraphConditionalHandle h_loop, h_pro, h_mode, h_fin, h_inner;
+  cudaGraphConditionalHandle h_loop, h_pro, h_mode, h_fin;
 };
 
 __global__ void k_dense_init(const DenseInit p) {
@@ -743,6 +1035,7 @@ __global__ void k_dense_init(const DenseInit p) {
   ctl->it_cur = it0;
   ctl->ticket = 0;
   ctl->bar = 0;
+  ctl->lbar = 0;
   for (int t = 0; t < 3; t++) {
     ctl->sw_all[t] = p.sw_all[t];
     ctl->dcnt[t] = ctl->save_cnt[t];
@@ -771,7 +1064,6 @@ __global__ void k_dense_init(const DenseInit p) {
   ctl->status = kStatusDone;
   cudaGraphSetConditional(p.h_pro, 0u);
   cudaGraphSetConditional(p.h_mode, 1u);
-  cudaGraphSetConditional(p.h_inner, 0u);
   if (ctl->fin_only) {
     // the marking launch ran the last iteration (recording its change flags): only its
     // marks remain, by a pull over every tier
@@ -1048,7 +1340,7 @@ struct LoopGraph {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaGraphNode_t init = nullptr;
-  cudaGraphConditionalHandle h_loop = 0, h_pro = 0, h_mode = 0, h_fin = 0, h_inner = 0;
+  cudaGraphConditionalHandle h_loop = 0, h_pro = 0, h_mode = 0, h_fin = 0;
   std::vector<unsigned char> key;
   void release() {
     if (exec) cudaGraphExecDestroy(exec);
@@ -1061,7 +1353,7 @@ struct LoopGraph {
 };
 
 struct Loops {
-  LoopGraph full;
+  LoopGraph full;      // one launch per iteration (df_split = 0)
   LoopGraph dense[2];  // synchronous, asynchronous (aliased parities)
 };
 
@@ -1078,12 +1370,12 @@ void append_key(std::vector<unsigned char> &k, const T &x) {
   } while (0)
 
 cudaError_t add_kernel(cudaGraphNode_t *node, cudaGraph_t graph, const cudaGraphNode_t *dep, size_t ndep,
-                       const void *fn, dim3 grid, dim3 block, void **args, bool coop) {
+                       const void *fn, dim3 grid, dim3 block, void **args, bool coop, size_t smem = 0) {
   cudaKernelNodeParams kp{};
   kp.func = const_cast<void *>(fn);
   kp.gridDim = grid;
   kp.blockDim = block;
-  kp.sharedMemBytes = 0;
+  kp.sharedMemBytes = (unsigned)smem;
   kp.kernelParams = args;
   cudaError_t e = cudaGraphAddKernelNode(node, graph, dep, ndep, &kp);
   if (e == cudaSuccess && coop) {
@@ -1108,6 +1400,8 @@ cudaError_t add_conditional(cudaGraphNode_t *node, cudaGraph_t graph, const cuda
   return e;
 }
 
+size_t hot_bytes(const Graph *g) { return (size_t)g->hot * (g->f32 ? 4 : 8); }
+
 template <bool F32>
 SweepArgs<F32> sweep_args(const Graph *g, bool async) {
   using S = Store<F32>;
@@ -1131,6 +1425,7 @@ SweepArgs<F32> sweep_args(const Graph *g, bool async) {
   a.emap = g->emap;
   a.out_rd = g->out.rd;
   a.ctl = g->ctl;
+  a.hot = g->hot;
   const double n = (double)g->n;
   if constexpr (F32) {
     a.base = (float)((1.0 - g->p.alpha) / n);
@@ -1152,13 +1447,30 @@ SweepArgs<F32> sweep_args(const Graph *g, bool async) {
 
 template <bool F32>
 pr_status full_impl(Graph *g, bool from_init) {
+  LoopArgs<F32> p{};
+  p.a = sweep_args<F32>(g, false);
+  p.n0 = g->item_cnt[0];
+  p.n1 = g->item_cnt[1];
+  p.n2 = g->item_cnt[2];
+  p.m = (uint32_t)g->m;
+  p.is_static = from_init ? 1u : 0u;
+  if constexpr (F32) p.init = (float)(1.0 / (double)g->n);
+  else p.init = std::llrint(1.0 / (double)g->n * 4611686018427387904.0);
+  void *args[] = {(void *)&p};
+  CKG(cudaLaunchCooperativeKernel((const void *)k_loop<F32, false>, dim3(g->loop_grid), dim3(kSweepBlock), args,
+                                  hot_bytes(g), g->st));
+  count_launch();
+  return PR_OK;
+}
+
+template <bool F32>
+pr_status full_steps_impl(Graph *g, bool from_init) {
   using S = Store<F32>;
   Loops *L = (Loops *)g->loops;
   LoopGraph &lg = L->full;
   SweepArgs<F32> a = sweep_args<F32>(g, false);
   std::vector<unsigned char> key;
   append_key(key, a);
-  append_key(key, g->sweep_grid);
   if (lg.exec && key != lg.key) lg.release();
   FullInit<F32> ip{};
   ip.R0 = (typename S::R *)g->R[0];
@@ -1188,8 +1500,8 @@ pr_status full_impl(Graph *g, bool from_init) {
     cudaGraph_t body = nullptr;
     CKG(add_conditional(&wnode, lg.graph, &lg.init, 1, lg.h_loop, cudaGraphCondTypeWhile, &body));
     void *sargs[] = {(void *)&a};
-    CKG(add_kernel(&snode, body, nullptr, 0, (const void *)k_sweep<F32, 0>, dim3(g->sweep_grid), dim3(kRankBlock),
-                   sargs, false));
+    CKG(add_kernel(&snode, body, nullptr, 0, (const void *)k_sweep<F32, 0>, dim3(g->sm_count), dim3(kSweepBlock), sargs,
+                   false, hot_bytes(g)));
     typename S::R *R0 = ip.R0, *R1 = ip.R1;
     typename S::C *C0 = ip.C0, *C1 = ip.C1;
     uint32_t n = g->n;
@@ -1238,8 +1550,7 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
   std::vector<unsigned char> key;
   append_key(key, a);
   append_key(key, ra);
-  append_key(key, g->dfsweep_grid);
-  append_key(key, g->cmpsweep_grid);
+  append_key(key, g->loop_grid);
   append_key(key, g->pro_grid);
   if (lg.exec && key != lg.key) lg.release();
   DenseInit ip{};
@@ -1265,14 +1576,11 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
     CKG(add_conditional(&wnode, lg.graph, nullptr, 0, lg.h_loop, cudaGraphCondTypeWhile, &body));
     CKG(cudaGraphConditionalHandleCreate(&lg.h_pro, body, 0, 0));
     CKG(cudaGraphConditionalHandleCreate(&lg.h_mode, body, 1, 0));
-    CKG(cudaGraphConditionalHandleCreate(&lg.h_inner, body, 0, 0));
     ip.h_pro = lg.h_pro;
     ip.h_mode = lg.h_mode;
-    ip.h_inner = lg.h_inner;
     a.h_loop = lg.h_loop;
     a.h_pro = lg.h_pro;
     a.h_mode = lg.h_mode;
-    a.h_inner = lg.h_inner;
     // SWITCH on the prologue: 0 = none, 1 = tier-2 pull, 2 = push (and compaction), 3 = light push
     cudaGraph_t pb[4] = {nullptr, nullptr, nullptr, nullptr};
     CKG(add_conditional(&inode, body, nullptr, 0, lg.h_pro, cudaGraphCondTypeSwitch, pb, 4));
@@ -1286,21 +1594,18 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
     cudaGraphNode_t lnode = nullptr;
     CKG(add_kernel(&lnode, pb[3], nullptr, 0, (const void *)k_df_push_light<F32>, dim3(std::max(1, g->sm_count)),
                    dim3(kRankBlock), pargs, false));
-    // SWITCH on the iteration's mode: 0 = compacted items, 1 = every item
+    // SWITCH on what follows: 0 = a run of compacted iterations, 1 = one iteration over every item
     cudaGraph_t sw[2] = {nullptr, nullptr};
     cudaGraphNode_t swnode = nullptr, s0 = nullptr, s1 = nullptr;
     CKG(add_conditional(&swnode, body, &inode, 1, lg.h_mode, cudaGraphCondTypeSwitch, sw, 2));
+    LoopArgs<F32> la{};
+    la.a = a;
+    void *largs[] = {(void *)&la};
+    CKG(add_kernel(&s0, sw[0], nullptr, 0, (const void *)k_loop<F32, true>, dim3(g->loop_grid), dim3(kSweepBlock), largs,
+                   true, hot_bytes(g)));
     void *sargs[] = {(void *)&a};
-    CKG(add_kernel(&s0, sw[0], nullptr, 0, (const void *)k_sweep<F32, 2>, dim3(g->cmpsweep_grid), dim3(kRankBlock),
-                   sargs, false));
-    CKG(add_kernel(&s1, sw[1], nullptr, 0, (const void *)k_sweep<F32, 1>, dim3(g->dfsweep_grid), dim3(kRankBlock),
-                   sargs, false));
-    // then the run of plain compacted iterations that follows (WHILE on h_inner)
-    cudaGraph_t ib = nullptr;
-    cudaGraphNode_t inner = nullptr, s2 = nullptr;
-    CKG(add_conditional(&inner, body, &swnode, 1, lg.h_inner, cudaGraphCondTypeWhile, &ib));
-    CKG(add_kernel(&s2, ib, nullptr, 0, (const void *)k_sweep<F32, 2>, dim3(g->cmpsweep_grid), dim3(kRankBlock), sargs,
-                   false));
+    CKG(add_kernel(&s1, sw[1], nullptr, 0, (const void *)k_sweep<F32, 1>, dim3(g->sm_count),
+                   dim3(kSweepBlock), sargs, false, hot_bytes(g)));
     void *iargs[] = {(void *)&ip};
     CKG(add_kernel(&lg.init, lg.graph, nullptr, 0, (const void *)k_dense_init, dim3(1), dim3(32), iargs, false));
     cudaGraphEdgeData ed{};
@@ -1324,7 +1629,6 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
     ip.h_pro = lg.h_pro;
     ip.h_mode = lg.h_mode;
     ip.h_fin = lg.h_fin;
-    ip.h_inner = lg.h_inner;
     cudaKernelNodeParams kp{};
     void *iargs[] = {(void *)&ip};
     kp.func = (void *)k_dense_init;
@@ -1340,27 +1644,30 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
 
 }  // namespace
 
+uint32_t hot_limit(bool f32) { return kHotBytes / (f32 ? 4 : 8); }
+
 pr_status sweep_setup(Graph *g) {
   if (!g->emap) {
     CKG(cudaMalloc((void **)&g->emap, 2ull * g->n));
     CKG(cudaMemsetAsync(g->emap, 0, 2ull * g->n, g->st));
   }
-  const void *fns[2][3] = {{(const void *)k_sweep<false, 0>, (const void *)k_sweep<false, 1>, (const void *)k_sweep<false, 2>},
-                           {(const void *)k_sweep<true, 0>, (const void *)k_sweep<true, 1>, (const void *)k_sweep<true, 2>}};
-  int per_mode[3] = {0, 0, 0};
-  for (int k = 0; k < 3; k++) {
-    CKG(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_mode[k], fns[g->f32 ? 1 : 0][k], kRankBlock, 0));
-    per_mode[k] = std::max(1, std::min(per_mode[k], 8));
-  }
-  g->sweep_grid = per_mode[0] * g->sm_count;
-  g->dfsweep_grid = per_mode[1] * g->sm_count;
-  g->cmpsweep_grid = per_mode[2] * g->sm_count;
+  const void *fns[4] = {g->f32 ? (const void *)k_loop<true, false> : (const void *)k_loop<false, false>,
+                        g->f32 ? (const void *)k_loop<true, true> : (const void *)k_loop<false, true>,
+                        g->f32 ? (const void *)k_sweep<true, 1> : (const void *)k_sweep<false, 1>,
+                        g->f32 ? (const void *)k_sweep<true, 0> : (const void *)k_sweep<false, 0>};
+  for (const void *fn : fns) CKG(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHotBytes));
+  g->loop_grid = g->sm_count;
   int per_sm_pro = 0;
   CKG(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
       &per_sm_pro, g->f32 ? (const void *)k_df_push<true> : (const void *)k_df_push<false>, kRankBlock, 0));
-  g->pro_grid = std::max(1, std::min(per_sm_pro, 4)) * g->sm_count;
+  g->pro_grid = g->pro_grid_max = std::max(1, std::min(per_sm_pro, 4)) * g->sm_count;
   if (!g->loops) g->loops = new Loops();
   return PR_OK;
+}
+
+void sweep_share(Graph *g, int slots) {
+  g->loop_grid = std::max(1, g->sm_count / slots);
+  g->pro_grid = std::max(1, g->pro_grid_max / slots);
 }
 
 bool sweep_eligible(const Graph *g) {
@@ -1368,6 +1675,7 @@ bool sweep_eligible(const Graph *g) {
 }
 
 pr_status sweep_full(Graph *g, bool from_init) {
+  if (!g->split_df) return g->f32 ? full_steps_impl<true>(g, from_init) : full_steps_impl<false>(g, from_init);
   return g->f32 ? full_impl<true>(g, from_init) : full_impl<false>(g, from_init);
 }
 
