@@ -132,7 +132,7 @@ pr_status pr_graph_create(uint32_t n, int64_t m, const uint32_t *src, const uint
  * first_c = comp_n[0] + ... + comp_n[c-1] (each comp_n[c] >= 1).  src/dst hold the edges of
  * all graphs in global ids; an edge (or later a batch pair) joining two graphs is rejected
  * with PR_ERR_INVALID_ARG.  pr_apply_batch takes one combined batch for all graphs, and each
- * rank call runs every graph in one persistent launch: graph c uses its own (1 - alpha)/n_c
+ * rank call runs every graph in one persistent launch (after a marking launch, where it marks): graph c uses its own (1 - alpha)/n_c
  * and starting rank 1/n_c (Eq. 1 per graph) and its own convergence test, and stops
  * updating once converged, so its ranks are those of a run of graph c alone.  Self-loop
  * dead-end mode only.  Per-graph results: pr_get_component_stats. */
@@ -181,8 +181,8 @@ pr_status pr_get_tuning(const pr_graph *g, pr_tuning *t);
 pr_status pr_autotune(pr_graph *g, int32_t sweep_iters, pr_tuning *chosen);
 
 /* enable != 0: rank calls replay one CUDA graph (control-block reset + the cooperative
- * persistent kernel), captured on first use; only the kernel's arguments change between
- * replays. */
+ * persistent kernel, or for a batched handle the marking launch and the iterations), captured
+ * on first use; only the kernels' arguments change between replays. */
 pr_status pr_set_graph_launch(pr_graph *g, int32_t enable);
 
 /* Fault injection on the host, for tests of the out-of-memory path: after this call the

@@ -382,17 +382,23 @@ static pr_status create_impl(uint32_t n, int64_t m, const uint32_t *src, const u
         if (rc == PR_OK && (best < 0 || cost[k][1] < cost[best][1])) best = k;
       }
       bool keep = rc == PR_OK && best >= 0 && (p.vertex_order >= 2 || cost[best][1] * 20 < cost[best][0] * 19);
-      // single-graph self-loop handles sweep with the contributions of the first vertices in
+      // self-loop handles sweep with the contributions of each graph's first vertices in
       // shared memory; the hot vertices go first in the numbering that is kept
-      if (keep && !comp_n && !g.teleport) {
+      if (keep && !g.teleport) {
+        std::vector<uint32_t> hot;
         if (g.f32) {
           e = cudaMalloc((void **)&g.lab, 4ull * n);
           if (e == cudaSuccess) e = cudaMalloc((void **)&g.at, 4ull * n);
           if (e != cudaSuccess) rc = prdf::cuda_fail(&g0, e, "vertex numbering");
         }
-        if (rc == PR_OK) rc = prdf::hot_order(&g0, prdf::hot_limit(g.f32), cp[best], ci[best], &g.hot, g.lab, g.at);
+        if (rc == PR_OK)
+          rc = prdf::hot_order(&g0, comp_n ? *comp_n : std::vector<uint32_t>{n}, prdf::hot_limit(g.f32), cp[best],
+                               ci[best], hot, g.lab, g.at);
         keep = rc == PR_OK;
-        if (!g.hot) {
+        if (!hot.empty()) {
+          if (comp_n) g.comp_hot_h = hot;
+          else g.hot = hot[0] & ~3u;
+        } else {
           cudaFree(g.lab);
           cudaFree(g.at);
           g.lab = g.at = nullptr;
@@ -421,6 +427,8 @@ static pr_status create_impl(uint32_t n, int64_t m, const uint32_t *src, const u
         if (e != cudaSuccess) { rc = prdf::cuda_fail(&g, e, "vertex numbering"); break; }
       }
     }
+    // a small graph's contributions are copied whole, in any numbering
+    if (!comp_n && !g.teleport && n <= prdf::hot_limit(g.f32)) g.hot = n & ~3u;
     rc = prdf::graph_build(&g, (uint64_t)m, sd, dd);
     if (rc != PR_OK) break;
     if (comp_n && (rc = prdf::components_setup(&g, *comp_n)) != PR_OK) break;

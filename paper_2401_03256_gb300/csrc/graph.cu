@@ -399,6 +399,8 @@ __device__ void merge_row(uint32_t s, uint2 *rd, uint32_t *cap, uint32_t *col, c
     uint32_t db = (q - s0) - ib;
     dst[lo - db + ib] = hook.at ? hook.at[y] : y;
   }
+  // the free slots of the row's last 16 bytes say so (the sweeps read rows by 16 bytes)
+  if (tid < 4 && new_len + tid < ((new_len + 3) & ~3u)) dst[new_len + tid] = kNoCol;
   if (hook.is_out) {
     for (uint32_t q = s0 + tid; q < e; q += kMergeThreads) {
       uint64_t c = chg[q];
@@ -665,7 +667,7 @@ static pr_status build_adj(Graph *g, const uint64_t *keys, uint64_t m, Adj &A, u
   }
   A.col_cap = total + reserve;
   CK(dalloc(&A.col, A.col_cap));
-  CK(cudaMemsetAsync(A.col, 0, sizeof(uint32_t) * A.col_cap, st));
+  CK(cudaMemsetAsync(A.col, 0xFF, sizeof(uint32_t) * A.col_cap, st));  // free slots: kNoCol
   k_row_desc<<<grid_for(n), 256, 0, st>>>(tmp, off, n, A.rd); count_launch();
   k_scatter_cols<<<grid_for(m), 256, 0, st>>>(keys, m, g->b, off, A.rd, A.col, at); count_launch();
   A.used = total;
@@ -850,7 +852,7 @@ static pr_status repack_adj(Graph *g, Adj &A, uint64_t reserve) {
   }
   uint32_t *nc = nullptr;
   CK(dalloc(&nc, total + reserve));
-  CK(cudaMemsetAsync(nc, 0, sizeof(uint32_t) * (total + reserve), st));
+  CK(cudaMemsetAsync(nc, 0xFF, sizeof(uint32_t) * (total + reserve), st));
   k_repack_rows<<<grid_for((uint64_t)n * 32), 256, 0, st>>>(A.rd, n, A.col, nc, g->gen_tmp); count_launch();
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));
@@ -1136,7 +1138,7 @@ pr_status graph_refresh_ident(Graph *g) {
   g->item_cnt[1] = c01 - h[0];
   g->item_cnt[2] = total;
   g->ident_dirty = false;
-  return PR_OK;
+  return g->comp_item ? batch_items(g) : PR_OK;
 }
 
 pr_status graph_refresh_dead(Graph *g) {
@@ -1228,6 +1230,15 @@ pr_status components_setup(Graph *g, const std::vector<uint32_t> &comp_n) {
   CK(cudaMalloc(&g->comp_base, 8ull * nc));
   CK(cudaMalloc(&g->comp_init, 8ull * nc));
   CK(dalloc(&g->dRc, 3ull * nc));
+  CK(dalloc(&g->comp_x, 3ull * nc));
+  CK(dalloc(&g->comp_hot, nc));
+  CK(dalloc(&g->comp_item, 3ull * (nc + 1)));
+  // a graph's first vertices, as many as fit an SM's shared copy: numbered by out-degree where
+  // the graph is larger and the handle has an internal numbering
+  std::vector<uint32_t> hot(nc);
+  for (uint32_t c = 0; c < nc; c++)
+    hot[c] = g->comp_hot_h.empty() ? std::min(comp_n[c], hot_limit(g->f32)) : g->comp_hot_h[c];
+  CK(cudaMemcpyAsync(g->comp_hot, hot.data(), 4ull * nc, cudaMemcpyHostToDevice, st));
   CK(dalloc(&g->comp_out, 4ull * nc));
   CK(dalloc(&g->comp_last, nc));
   if (g->f32) {
@@ -1249,7 +1260,7 @@ pr_status components_setup(Graph *g, const std::vector<uint32_t> &comp_n) {
   count_launch();
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));
-  cudaFree(first_d);
+  g->comp_first_d = first_d;
   g->comp_stats.assign(nc, pr_stats{});
   return PR_OK;
 }
@@ -1278,6 +1289,10 @@ void graph_free(Graph *g) {
   cudaFree(g->comp_base);
   cudaFree(g->comp_init);
   cudaFree(g->dRc);
+  cudaFree(g->comp_x);
+  cudaFree(g->comp_first_d);
+  cudaFree(g->comp_hot);
+  cudaFree(g->comp_item);
   cudaFree(g->comp_out);
   cudaFree(g->comp_last);
   cudaFree(g->partials);

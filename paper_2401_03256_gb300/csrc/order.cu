@@ -72,16 +72,19 @@ __global__ void k_order_start(const unsigned long long *best, uint32_t *label, u
   perm[0] = s;
 }
 
-// graph of each vertex (first[c] <= v < first[c + 1]; nc <= kMaxComponents)
-__global__ void k_order_graph_of(const uint32_t *first, uint32_t nc, uint32_t n, uint32_t *gid) {
-  const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= n) return;
+// graph of vertex v (first[c] <= v < first[c + 1]; nc <= kMaxComponents)
+__device__ __forceinline__ uint32_t graph_of(const uint32_t *first, uint32_t nc, uint32_t v) {
   uint32_t lo = 0, hi = nc;  // last c with first[c] <= v
   while (hi - lo > 1) {
     const uint32_t mid = (lo + hi) >> 1;
     if (first[mid] <= v) lo = mid; else hi = mid;
   }
-  gid[v] = lo;
+  return lo;
+}
+
+__global__ void k_order_graph_of(const uint32_t *first, uint32_t nc, uint32_t n, uint32_t *gid) {
+  const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v < n) gid[v] = graph_of(first, nc, v);
 }
 
 // every graph's vertex of largest out + in degree (smallest id on ties)
@@ -235,41 +238,45 @@ __global__ void k_map_ids(const uint32_t *inv, uint32_t *a, uint64_t m) {
   if (i < m) a[i] = inv[a[i]];
 }
 
-// Out-degrees of all vertices, counted by degree (kHotBins and above together).
-constexpr uint32_t kHotBins = 8192;
-__global__ void __launch_bounds__(1024) k_hot_hist(const uint2 *out_rd, uint32_t n, uint32_t *hist) {
-  __shared__ uint32_t s[kHotBins];
-  for (uint32_t k = threadIdx.x; k < kHotBins; k += blockDim.x) s[k] = 0;
-  __syncthreads();
-  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
-    atomicAdd(&s[min(out_rd[v].y, kHotBins - 1)], 1u);
-  __syncthreads();
-  for (uint32_t k = threadIdx.x; k < kHotBins; k += blockDim.x)
-    if (s[k]) atomicAdd(&hist[k], s[k]);
+// Out-degrees by graph, counted by degree (kHotBins and above together; below kHotLeast not at
+// all: such vertices are never put first).  Graphs of at most hot_max vertices are left out.
+constexpr uint32_t kHotBins = 2048, kHotLeast = 4;
+__global__ void k_hot_hist(const uint2 *out_rd, const uint32_t *first, uint32_t nc, uint32_t hot_max, uint32_t n,
+                           uint32_t *hist) {
+  const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= n) return;
+  const uint32_t d = out_rd[v].y;
+  if (d < kHotLeast) return;
+  const uint32_t c = graph_of(first, nc, v);
+  if (first[c + 1] - first[c] > hot_max) atomicAdd(&hist[c * kHotBins + min(d, kHotBins - 1)], 1u);
 }
 
 // flags of the hot vertices by place in the numbering, and the sum of their out-degrees
-__global__ void k_hot_flags(const uint2 *out_rd, const uint32_t *perm, uint32_t n, uint32_t least, uint32_t *flags,
-                            unsigned long long *edges) {
+__global__ void k_hot_flags(const uint2 *out_rd, const uint32_t *perm, const uint32_t *first, const uint32_t *least,
+                            uint32_t nc, uint32_t n, uint32_t *flags, unsigned long long *edges) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long d = 0;
   if (i < n) {
     const uint32_t y = out_rd[perm[i]].y;
-    flags[i] = y >= least ? 1u : 0u;
-    d = y >= least ? y : 0u;
+    const bool f = y >= least[graph_of(first, nc, i)];
+    flags[i] = f ? 1u : 0u;
+    d = f ? y : 0u;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
   if ((threadIdx.x & 31) == 0 && d) atomicAdd(edges, d);
 }
 
-// the numbering with the flagged places (the first `hot` of them) in front
-__global__ void k_hot_perm(const uint32_t *flags, const uint32_t *pos, uint32_t n, uint32_t hot, const uint32_t *old,
-                           uint32_t *perm, uint32_t *inv, uint32_t *lab, uint32_t *at) {
+// the numbering with every graph's flagged places (the first hot[c] of them) at its front
+__global__ void k_hot_perm(const uint32_t *flags, const uint32_t *pos, const uint32_t *first, const uint32_t *hots,
+                           uint32_t nc, uint32_t n, const uint32_t *old, uint32_t *perm, uint32_t *inv, uint32_t *lab,
+                           uint32_t *at) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const bool f = flags[i] && pos[i] < hot;
-  const uint32_t k = f ? pos[i] : hot + (i - min(pos[i], hot));
+  const uint32_t c = graph_of(first, nc, i), b = first[c], hot = hots[c];
+  const uint32_t p = pos[i] - pos[b];  // flagged places of the graph before this one
+  const bool f = flags[i] && p < hot;
+  const uint32_t k = f ? b + p : b + hot + (i - b - min(p, hot));
   perm[k] = old[i];
   inv[old[i]] = k;
   if (lab) {
@@ -395,37 +402,49 @@ pr_status order_cost(Graph *g, const uint32_t *perm, const uint32_t *inv, uint64
   return PR_OK;
 }
 
-// The first vertices of the numbering, hot_max at most, become those of largest out-degree: the
-// sweeps keep their contributions in shared memory.  R-MAT graphs take 16,384 (64-bit) or 32,768 (FP32) of
-// them: 38% and 50% of the gathers at scale 22, 54% and 66% at scale 20, all at scale 14 (edge
-// factor 8).  Below a tenth of the out-edges (grids, chains) the numbering is left as it is:
-// a gather that can be hot costs two predicated loads.
-pr_status hot_order(Graph *g, uint32_t hot_max, uint32_t *perm, uint32_t *inv, uint32_t *hot, uint32_t *lab,
-                    uint32_t *at) {
-  *hot = 0;
-  const uint32_t n = g->n;
+// Every graph's first vertices, hot_max at most, become those of largest out-degree: the
+// sweeps keep their contributions in shared memory.  R-MAT graphs take 16 K (64-bit) or 32 K (FP32) of
+// them: 38% and 50% of the gathers at scale 22, 54% and 66% at scale 20 (edge factor 16), 70%
+// and 80% at scale 18 (edge factor 8); graphs of at most hot_max vertices are copied whole, in any order.  Where the
+// hot vertices have less than a tenth of the out-edges (grids, chains) the numbering is left
+// as it is: a gather that can be hot costs two predicated loads.
+pr_status hot_order(Graph *g, const std::vector<uint32_t> &comp_n, uint32_t hot_max, uint32_t *perm, uint32_t *inv,
+                    std::vector<uint32_t> &hot, uint32_t *lab, uint32_t *at) {
+  hot.clear();
+  const uint32_t n = g->n, nc = (uint32_t)comp_n.size();
   cudaStream_t st = g->st;
-  hot_max = std::min(hot_max, n) & ~3u;
-  if (hot_max == 0) return PR_OK;
-  pr_status rc = apply_scratch(g, std::max(n, kHotBins));
+  bool any = false;
+  for (uint32_t k : comp_n) any = any || k > hot_max;
+  if (!any) return PR_OK;
+  pr_status rc = apply_scratch(g, std::max<uint64_t>(n, (uint64_t)nc * kHotBins));
   if (rc != PR_OK) return rc;
   ApplyScratch &s = g->sc;
   uint32_t *hist = s.vals, *flags = s.flags, *pos = s.pos, *old = s.vals2;
+  uint32_t *first_d = s.seg, *least_d = s.seg + (nc + 1), *hot_d = least_d + nc;  // seg: 2 (cap + 2) words
   unsigned long long *edges = (unsigned long long *)s.tmp2;
-  CK(cudaMemsetAsync(hist, 0, 4ull * kHotBins, st));
+  std::vector<uint32_t> first(nc + 1, 0), least(nc, kHotLeast);
+  for (uint32_t c = 0; c < nc; c++) first[c + 1] = first[c] + comp_n[c];
+  CK(cudaMemcpyAsync(first_d, first.data(), 4ull * (nc + 1), cudaMemcpyHostToDevice, st));
+  CK(cudaMemsetAsync(hist, 0, 4ull * nc * kHotBins, st));
   CK(cudaMemsetAsync(edges, 0, 8, st));
-  k_hot_hist<<<std::max(1, g->sm_count), 1024, 0, st>>>(g->out.rd, n, hist);
+  k_hot_hist<<<grid_of(n), 256, 0, st>>>(g->out.rd, first_d, nc, hot_max, n, hist);
   count_launch();
-  std::vector<uint32_t> h(kHotBins);
-  CK(cudaMemcpyAsync(h.data(), hist, 4ull * kHotBins, cudaMemcpyDeviceToHost, st));
+  std::vector<uint32_t> h((size_t)nc * kHotBins);
+  CK(cudaMemcpyAsync(h.data(), hist, 4ull * h.size(), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  // the least degree of at most hot_max vertices (the bin of the largest degrees may hold
-  // more: the first of them in the numbering are taken)
-  uint32_t least = kHotBins - 1, count = h[least];
-  while (least > 0 && count + h[least - 1] <= hot_max) count += h[--least];
-  count = std::min(count, hot_max) & ~3u;
-  if (count == 0) return PR_OK;
-  k_hot_flags<<<grid_of(n), 256, 0, st>>>(g->out.rd, perm, n, least, flags, edges);
+  std::vector<uint32_t> counts(nc);
+  for (uint32_t c = 0; c < nc; c++) {
+    // the least degree of at most hot_max vertices (the bin of the largest degrees may hold
+    // more: the first of them in the numbering are taken)
+    const uint32_t *b = h.data() + (size_t)c * kHotBins;
+    uint32_t d = kHotBins - 1, k = b[d];
+    while (d > kHotLeast && k + b[d - 1] <= hot_max) k += b[--d];
+    least[c] = comp_n[c] > hot_max ? d : 0xFFFFFFFFu;
+    counts[c] = comp_n[c] > hot_max ? std::min(k, hot_max) : 0u;
+  }
+  CK(cudaMemcpyAsync(least_d, least.data(), 4ull * nc, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(hot_d, counts.data(), 4ull * nc, cudaMemcpyHostToDevice, st));
+  k_hot_flags<<<grid_of(n), 256, 0, st>>>(g->out.rd, perm, first_d, least_d, nc, n, flags, edges);
   count_launch();
   unsigned long long he = 0;
   CK(cudaMemcpyAsync(&he, edges, 8, cudaMemcpyDeviceToHost, st));
@@ -433,11 +452,11 @@ pr_status hot_order(Graph *g, uint32_t hot_max, uint32_t *perm, uint32_t *inv, u
   if (he * 10 < g->m) return PR_OK;
   exclusive_scan_u32(flags, pos, n, s.scan_tmp, st);
   CK(cudaMemcpyAsync(old, perm, 4ull * n, cudaMemcpyDeviceToDevice, st));
-  k_hot_perm<<<grid_of(n), 256, 0, st>>>(flags, pos, n, count, old, perm, inv, lab, at);
+  k_hot_perm<<<grid_of(n), 256, 0, st>>>(flags, pos, first_d, hot_d, nc, n, old, perm, inv, lab, at);
   count_launch();
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));
-  *hot = count;
+  for (uint32_t c = 0; c < nc; c++) hot.push_back(comp_n[c] > hot_max ? counts[c] : comp_n[c]);
   return PR_OK;
 }
 

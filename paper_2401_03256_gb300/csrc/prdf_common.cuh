@@ -21,6 +21,7 @@ constexpr uint32_t kSmallSort = 4096;     // largest key count sorted by one blo
 constexpr uint32_t kChunk = 512;          // entries per chunk of a long row (hub out-rows; the most a sweep chunk holds)
 constexpr uint32_t kGroupMax = 64;        // the longest row an 8-lane group of a sweep takes (two runs of 32)
 constexpr uint32_t kMaxComponents = 1024; // graphs in one batched handle
+constexpr uint32_t kNoCol = 0xFFFFFFFFu;  // free slots behind a row's entries, up to the next 16 bytes
 
 // Tier of an in-degree in the full/dense sweep order: 0 = one thread (<= lo), 1 = an
 // 8-lane group (<= max(lo, gmax), gmax <= kGroupMax), 2 = chunks of `chunk` edges taken by

@@ -83,9 +83,8 @@ struct Graph {
   bool use_graph = false;
   cudaGraph_t cg = nullptr;
   cudaGraphExec_t cg_exec = nullptr;
-  cudaGraphNode_t cg_kernel = nullptr;
-  bool cg_f32 = false;
-  bool cg_df = false;
+  cudaGraphNode_t cg_kernel = nullptr, cg_kernel2 = nullptr;
+  int cg_kind = 0;                   // what the captured graph runs (kGraph...)
   uint32_t last_list_cnt[3] = {0, 0, 0};
   bool last_full = false;
 
@@ -104,6 +103,11 @@ struct Graph {
   void *comp_base = nullptr;         // [ncomp] (1 - alpha) / n_c, rank representation
   void *comp_init = nullptr;         // [ncomp] 1 / n_c
   unsigned long long *dRc = nullptr; // [3][ncomp]
+  uint32_t *comp_x = nullptr;        // [3][ncomp] first expansions by iteration modulo 3
+  uint32_t *comp_first_d = nullptr;  // [ncomp + 1] comp_first on the device
+  uint32_t *comp_hot = nullptr;      // [ncomp] vertices of a graph, from its first on, copied to shared memory
+  uint32_t *comp_item = nullptr;     // [3][ncomp + 1] first sweep item of each graph, by tier
+  std::vector<uint32_t> comp_hot_h;  // hot vertices of each graph as numbered at creation (or empty)
   uint32_t *comp_out = nullptr;      // [ncomp][4]
   unsigned long long *comp_last = nullptr;
   std::vector<pr_stats> comp_stats;  // per graph, from the last rank call
@@ -138,13 +142,14 @@ constexpr int kOrderFromMax = 0, kOrderFromSeeds = 1, kOrderPerGraph = 2;
 pr_status vertex_order(Graph *g, int kind, uint32_t *perm, uint32_t *inv,
                        const std::vector<uint32_t> *comp_n = nullptr);
 pr_status order_cost(Graph *g, const uint32_t *perm, const uint32_t *inv, uint64_t cost[2]);  // order.cu, on a built graph
-// Puts the vertices of largest out-degree first in the numbering (perm, inv), up to hot_max of
-// them, the rest in the order they had; *hot = their number, or 0 (numbering unchanged) where
-// their out-edges are too few to matter.
-// lab and at (null, or n each) receive the order before: lab[new number] = old, at[old] = new.
-pr_status hot_order(Graph *g, uint32_t hot_max, uint32_t *perm, uint32_t *inv, uint32_t *hot, uint32_t *lab,
-                    uint32_t *at);
-uint32_t hot_limit(bool f32);  // sweep.cu: contributions a block's shared-memory copy holds
+// Puts the vertices of largest out-degree of every graph (comp_n vertices each) first in its
+// part of the numbering (perm, inv), up to hot_max of them, the rest in the order they had;
+// hot = how many of each graph's first vertices to copy, or empty (numbering unchanged) where it
+// would not matter.  lab and at (null, or n each) receive the order before: lab[new number] =
+// old, at[old] = new.
+pr_status hot_order(Graph *g, const std::vector<uint32_t> &comp_n, uint32_t hot_max, uint32_t *perm, uint32_t *inv,
+                    std::vector<uint32_t> &hot, uint32_t *lab, uint32_t *at);
+uint32_t hot_limit(bool f32);  // sweep.cu: contributions a block's shared-memory copy holds (less a few)
 void map_ids(const uint32_t *inv, uint32_t *a, uint64_t m, cudaStream_t st);
 pr_status graph_export(Graph *g, int dir, uint64_t *offs_h, uint32_t *cols_h);
 pr_status graph_refresh_ident(Graph *g);
@@ -162,6 +167,16 @@ pr_status rank_set(Graph *g, const double *in_d);
 pr_status rank_get(Graph *g, double *out_d);
 pr_status rank_dead_mass(Graph *g, double *D);
 pr_status components_setup(Graph *g, const std::vector<uint32_t> &comp_n);  // after graph_build
+
+// batch.cu: the iterations of batched handles (unless df_split is 0), one persistent launch
+// after the marking launch of marking calls.
+constexpr int kGraphWhole = 0, kGraphMarking = 1, kGraphBatchMarking = 2, kGraphBatchEvery = 3;
+bool batch_eligible(const Graph *g);
+pr_status batch_setup(Graph *g);
+pr_status batch_items(Graph *g);  // after a rebuild of the sweep items
+pr_status batch_run(Graph *g, RankMode mode, bool marking, const void *rank_args);
+const void *marking_kernel(bool f32);  // rank.cu: the marking launch of batched handles
+size_t marking_smem(const Graph *g);
 
 // sweep.cu: Static / Naive-dynamic iterations, and the dense iterations of a Dynamic
 // Frontier, Dynamic Traversal or asynchronous call, one launch per iteration inside a

@@ -331,10 +331,11 @@ __device__ __noinline__ DtOut dt_search(const RankArgs<F32> &a, uint32_t epoch, 
   return o;
 }
 
-// SPLIT: the marking launch of a split call (single graph, self-loop mode), which hands the
-// call to the per-iteration launches before its first dense iteration and before any
+// SPLIT 1: the marking launch of a split call (single graph, self-loop mode), which hands the
+// call to the sweep launches before its first dense iteration and before any
 // iteration over every vertex; its instance carries no dense or full sweep code.
-template <bool F32, bool DF, bool SPLIT = false>
+// 2: of a batched handle in self-loop mode (the iterations follow in batch.cu).
+template <bool F32, bool DF, int SPLIT = 0>
 __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const RankArgs<F32> a) {
   using S = Store<F32>;
   using R = typename S::R;
@@ -357,8 +358,8 @@ __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const
   constexpr bool df = DF;
   // per-component state (batched form), identical in every block; a split call's marking
   // launch serves one graph in self-loop mode (no components, no teleport)
-  const bool multi = !SPLIT && a.ncomp > 1;
-  const bool tele = !SPLIT && a.teleport;
+  const bool multi = SPLIT != 1 && a.ncomp > 1;
+  const bool tele = SPLIT == 0 && a.teleport;
   const uint32_t nc = a.ncomp;
   extern __shared__ unsigned long long dsm[];
   unsigned long long *s_kmax = dsm;                         // block max key / counter per component
@@ -664,7 +665,7 @@ __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const
       return big && first_expansion(a.xbits, v);
     };
 
-    if (!SPLIT && (I.full || dense)) {
+    if (SPLIT == 0 && (I.full || dense)) {
       const uint32_t off1 = a.it_c0, off2 = a.it_c0 + a.it_c1;
       const uint4 *T = a.items;
       uint32_t n0 = a.it_c0, n1 = a.it_c1, n2 = a.it_c2;
@@ -1064,6 +1065,12 @@ static cudaError_t grid_blocks(int sm_count, size_t smem, int *blocks) {
   return cudaSuccess;
 }
 
+const void *marking_kernel(bool f32) {
+  return f32 ? (const void *)k_rank<true, true, 2> : (const void *)k_rank<false, true, 2>;
+}
+
+size_t marking_smem(const Graph *g) { return rank_smem(g->ncomp); }
+
 pr_status rank_setup(Graph *g) {
   int blocks = 0;
   const size_t smem = rank_smem(g->ncomp);
@@ -1075,7 +1082,9 @@ pr_status rank_setup(Graph *g) {
   CK(cudaMalloc((void **)&g->dpart, sizeof(DeadPart) * 2 * (size_t)blocks));
   CK(cudaEventCreate(&g->ev0));
   CK(cudaEventCreate(&g->ev1));
-  return sweep_setup(g);
+  pr_status rc = sweep_setup(g);
+  if (rc == PR_OK && g->ncomp > 1) rc = batch_setup(g);
+  return rc;
 }
 
 // The full-sweep instance in Naive-dynamic mode on the arguments of a marking call whose
@@ -1176,8 +1185,8 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
   a.emap = g->emap;
   a.item_pos = g->item_pos;
   const bool marking = mode == kModeDF || mode == kModeDT || async;
-  const bool loops = sweep_eligible(g);
-  a.split = marking && loops && g->split_df && !start_full;
+  const bool loops = sweep_eligible(g), batch = batch_eligible(g);
+  a.split = marking && (loops || batch) && g->split_df && !start_full;
   // expected marks of a set of k vertices: k * m / n; deferring to a pull pays once they
   // would make the next set dense (more than n / dense_div) several times over: a pull
   // reads the in-rows of every vertex not yet affected, so below that a push is cheaper
@@ -1192,6 +1201,7 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
     }
     return PR_OK;
   };
+  if (batch) return batch_run(g, mode, a.split != 0, &a);
   if (loops && (!marking || start_full)) {
     // every vertex every iteration (Static; Naive-dynamic, also for a marking call whose
     // affected set is all of V): per-iteration launches in a device-side loop
@@ -1204,7 +1214,7 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
     CK(launch_full_sweep<F32>(g, a));
     return copy_async_parity();
   }
-  const void *fn = marking ? (a.split && !g->use_graph ? (const void *)k_rank<F32, true, true> : (const void *)k_rank<F32, true>)
+  const void *fn = marking ? (a.split && !g->use_graph ? (const void *)k_rank<F32, true, 1> : (const void *)k_rank<F32, true>)
                            : (const void *)k_rank<F32, false>;
   if (!g->use_graph) {
     CK(cudaLaunchCooperativeKernel(fn, dim3(g->rank_grid), dim3(kRankBlock), args,
@@ -1232,10 +1242,12 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
   kp.blockDim = dim3(kRankBlock);
   kp.sharedMemBytes = (unsigned)rank_smem(g->ncomp);
   kp.kernelParams = args;
-  if (g->cg_exec && (g->cg_f32 != F32 || g->cg_df != marking)) {
+  const int kind = marking ? kGraphMarking : kGraphWhole;
+  if (g->cg_exec && g->cg_kind != kind) {
     cudaGraphExecDestroy(g->cg_exec);
     cudaGraphDestroy(g->cg);
     g->cg_exec = nullptr;
+    g->cg = nullptr;
   }
   if (!g->cg_exec) {
     cudaGraph_t graph = nullptr;
@@ -1256,8 +1268,7 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
     CK(cudaGraphInstantiate(&g->cg_exec, graph, 0));
     g->cg = graph;
     g->cg_kernel = kern;
-    g->cg_f32 = F32;
-    g->cg_df = marking;
+    g->cg_kind = kind;
   } else {
     CK(cudaGraphExecKernelNodeSetParams(g->cg_exec, g->cg_kernel, &kp));
   }
@@ -1287,6 +1298,7 @@ pr_status rank_run(Graph *g, RankMode mode, pr_stats *stats) {
   }
   if (g->ncomp > 1) {
     CK(cudaMemsetAsync(g->dRc, 0, 3ull * g->ncomp * sizeof(unsigned long long), g->st));
+    CK(cudaMemsetAsync(g->comp_x, 0, 12ull * g->ncomp, g->st));
     CK(cudaMemsetAsync(g->comp_out, 0, 16ull * g->ncomp, g->st));
     CK(cudaMemsetAsync(g->comp_last, 0, 8ull * g->ncomp, g->st));
   }
