@@ -362,6 +362,7 @@ static pr_status create_impl(uint32_t n, int64_t m, const uint32_t *src, const u
       g0.p = p;
       g0.f32 = g.f32;
       g0.teleport = g.teleport;
+      g0.transient = true;
       g0.st = g.st;
       g0.device = g.device;
       g0.sm_count = g.sm_count;

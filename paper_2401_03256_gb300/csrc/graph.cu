@@ -744,7 +744,9 @@ pr_status graph_build(Graph *g, uint64_t m_in, const uint32_t *src_d, const uint
     k_transpose_keys<<<grid_for(m), 256, 0, st>>>(other, m, g->b, g->lab, sorted);
     count_launch();
   }
-    uint64_t *tsorted = sort_u64(sorted, other, m, 2 * g->b, hist, stmp, st);
+    // the keys are in (u, v) order: a stable sort by v alone puts them in (v, u) order, unless
+    // the in-rows are ordered by another key than u
+    uint64_t *tsorted = sort_u64(sorted, other, m, 2 * g->b, hist, stmp, st, g->lab ? 0 : g->b);
     rc = build_adj(g, tsorted, m, g->in, flags, pos, stmp, g->at);
     if (rc != PR_OK) break;
     e = cudaStreamSynchronize(st);
@@ -753,6 +755,12 @@ pr_status graph_build(Graph *g, uint64_t m_in, const uint32_t *src_d, const uint
   if (e != cudaSuccess) return cuda_fail(g, e, "graph build");
   if (rc != PR_OK) return rc;
 
+  // what the vertex numbering needs of a transient build
+  CK(dalloc(&g->gen_tmp, (uint64_t)n + 8));  // also the sweep-item rebuild's 4 ceil(n / 4096) + 2 tile counts
+  CK(dalloc(&g->gen_tmp2, (uint64_t)n + 8));
+  CK(dalloc(&g->scan_tmp, scan_tmp_words((uint64_t)n + 8) + 1));
+  CK(dalloc(&g->actl, 1));
+  if (g->transient) return PR_OK;
   // rank state
   const size_t es = g->f32 ? 4 : 8;
   for (int i = 0; i < 2; i++) {
@@ -775,14 +783,9 @@ pr_status graph_build(Graph *g, uint64_t m_in, const uint32_t *src_d, const uint
   for (int i = 0; i < 3; i++) CK(dalloc(&g->list[i], n));
   CK(dalloc(&g->xlist, n));
   CK(dalloc(&g->dead, n));
-  // (n + 8 words: also the sweep-item rebuild's 4 ceil(n / 4096) + 2 tile counts)
-  CK(dalloc(&g->gen_tmp, (uint64_t)n + 8));
-  CK(dalloc(&g->gen_tmp2, (uint64_t)n + 8));
-  CK(dalloc(&g->scan_tmp, scan_tmp_words((uint64_t)n + 8) + 1));
   g->pend_cap = std::max<uint32_t>(1u << 16, std::min<uint32_t>(n, 1u << 22));
   CK(dalloc(&g->pend_src, g->pend_cap));
   CK(dalloc(&g->pend_tgt, g->pend_cap));
-  CK(dalloc(&g->actl, 1));
   CK(cudaMallocHost((void **)&g->actl_h, sizeof(ApplyCtl)));
   if (g->f32) {
     using S = Store<true>;
@@ -909,7 +912,7 @@ pr_status graph_apply(Graph *g, uint64_t nd, const uint32_t *ds, const uint32_t 
   // the change list is already in (u, v) order (one entry per key); only the transposed
   // copy needs a sort
   uint64_t *co = s.chg;
-  uint64_t *ci = sort_u64(s.chg_t, s.tmp2, K, kbits, s.radix_hist, s.scan_tmp, st);
+  uint64_t *ci = sort_u64(s.chg_t, s.tmp2, K, kbits, s.radix_hist, s.scan_tmp, st, g->lab ? 1 : b + 1);
   uint32_t *seg_o = s.seg, *seg_i = s.seg + (s.cap + 2);
   uint32_t *tp_o = s.tagpref, *tp_i = s.tagpref + (s.cap + 2);
   ApplyCtl *dctl = g->actl;

@@ -135,24 +135,72 @@ __global__ void k_order_seeds(uint32_t k, uint32_t step, uint32_t *label, uint32
 
 // One level: every vertex of the frontier (perm[lo, hi), numbered lo..hi-1) offers its
 // number to its unnumbered neighbours (out- and in-rows, one warp per frontier vertex); a
-// neighbour keeps the smallest offer, and its first offer lists it.
+// neighbour keeps the smallest offer, and its first offer lists it (the warp's new ones with
+// one atomic).  Rows longer than kOrderRow are queued (long_v: 2 k + direction; long_base: first
+// segment) for a second launch: with a warp to every row, two levels of an R-MAT graph of scale
+// 20 took 9 ms (now 1.8 ms in all).
+constexpr uint32_t kOrderRow = 1024, kOrderSeg = 256;
+__device__ __forceinline__ void order_offer(const uint32_t *col, uint32_t len, uint32_t k, uint32_t lane,
+                                            const uint32_t *label, uint32_t *cand, uint32_t *next, uint32_t *cnt) {
+  for (uint32_t j0 = 0; j0 < len; j0 += 32) {  // the same rounds for the whole warp
+    const uint32_t j = j0 + lane;
+    uint32_t w = 0;
+    bool fresh = false;
+    if (j < len) {
+      w = col[j];
+      // an earlier offer seen here or one that arrives later: the smallest stays either way
+      if (label[w] == kUnset && *(volatile uint32_t *)&cand[w] > k) fresh = atomicMin(&cand[w], k) == kUnset;
+    }
+    const uint32_t mask = __ballot_sync(0xffffffffu, fresh);
+    if (mask) {
+      const uint32_t leader = __ffs(mask) - 1, me = threadIdx.x & 31;
+      uint32_t base = 0;
+      if (me == leader) base = atomicAdd(cnt, (uint32_t)__popc(mask));
+      base = __shfl_sync(0xffffffffu, base, leader);
+      if (fresh) next[base + __popc(mask & ((1u << me) - 1u))] = w;
+    }
+  }
+}
+
 __global__ void k_order_expand(const uint2 *out_rd, const uint32_t *out_col, const uint2 *in_rd,
                                const uint32_t *in_col, const uint32_t *perm, uint32_t lo, uint32_t hi,
-                               const uint32_t *label, uint32_t *cand, uint32_t *next, uint32_t *cnt) {
+                               const uint32_t *label, uint32_t *cand, uint32_t *next, uint32_t *cnt,
+                               unsigned long long *queue, uint32_t *long_v, uint32_t *long_base) {
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
   for (uint32_t k = lo + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5); k < hi; k += nwarps) {
     const uint32_t u = perm[k];
-    for (int dir = 0; dir < 2; dir++) {
+    for (uint32_t dir = 0; dir < 2; dir++) {
       const uint2 d = dir ? in_rd[u] : out_rd[u];
-      const uint32_t *col = (dir ? in_col : out_col) + d.x;
-      for (uint32_t j = lane; j < d.y; j += 32) {
-        const uint32_t w = col[j];
-        if (label[w] != kUnset) continue;
-        const uint32_t old = atomicMin(&cand[w], k);
-        if (old == kUnset) next[atomicAdd(cnt, 1u)] = w;
+      if (d.y > kOrderRow) {
+        if (lane == 0) {  // entry and first segment from one atomic, so bases ascend
+          const unsigned long long old = atomicAdd(queue, (1ull << 32) | ((d.y + kOrderSeg - 1) / kOrderSeg));
+          long_v[old >> 32] = 2 * (k - lo) + dir;
+          long_base[old >> 32] = (uint32_t)old;
+        }
+        continue;
       }
+      order_offer((dir ? in_col : out_col) + d.x, d.y, k, lane, label, cand, next, cnt);
     }
+  }
+}
+
+// The long rows of a level, in segments dealt to the warps of the grid.
+__global__ void k_order_expand_long(const uint2 *out_rd, const uint32_t *out_col, const uint2 *in_rd,
+                                    const uint32_t *in_col, const uint32_t *perm, uint32_t lo, const uint32_t *label,
+                                    uint32_t *cand, uint32_t *next, uint32_t *cnt, const unsigned long long *queue,
+                                    const uint32_t *long_v, const uint32_t *long_base) {
+  const uint32_t lane = threadIdx.x & 31, nwarps = (gridDim.x * blockDim.x) >> 5;
+  const uint32_t n_long = (uint32_t)(*queue >> 32), n_seg = (uint32_t)*queue;
+  for (uint32_t s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < n_seg; s += nwarps) {
+    uint32_t a = 0, b = n_long;  // the row: last with long_base <= s
+    while (b - a > 1) {
+      const uint32_t mid = (a + b) >> 1;
+      if (long_base[mid] <= s) a = mid; else b = mid;
+    }
+    const uint32_t x = long_v[a], k = lo + (x >> 1), u = perm[k], at = (s - long_base[a]) * kOrderSeg;
+    const uint2 d = (x & 1) ? in_rd[u] : out_rd[u];
+    order_offer(((x & 1) ? in_col : out_col) + d.x + at, min(kOrderSeg, d.y - at), k, lane, label, cand, next, cnt);
   }
 }
 
@@ -296,6 +344,8 @@ pr_status vertex_order(Graph *g, int kind, uint32_t *perm, uint32_t *inv, const 
   if (rc != PR_OK) return rc;
   ApplyScratch &s = g->sc;
   uint32_t *cand = s.flags, *next = s.pos, *cnt = (uint32_t *)&g->actl->n_seg_out;
+  uint32_t *long_v = s.seg, *long_base = s.tagpref;  // 2 (cap + 2) words: both rows of every vertex
+  unsigned long long *queue = &g->actl->reloc_out;
   unsigned long long *keys = (unsigned long long *)s.kd;
   k_order_init<<<grid_of(n), 256, 0, st>>>(n, inv, cand);
   count_launch();
@@ -342,12 +392,22 @@ pr_status vertex_order(Graph *g, int kind, uint32_t *perm, uint32_t *inv, const 
   const unsigned egrid = (unsigned)std::max(1, g->sm_count * 8);
   for (int level = 0; hi > lo && level < kMaxLevels; level++) {
     CK(cudaMemsetAsync(cnt, 0, 4, st));
+    CK(cudaMemsetAsync(queue, 0, 8, st));
     k_order_expand<<<egrid, 256, 0, st>>>(g->out.rd, g->out.col, g->in.rd, g->in.col, perm, lo, hi, inv, cand,
-                                          next, cnt);
+                                          next, cnt, queue, long_v, long_base);
     count_launch();
     uint32_t c = 0;
+    unsigned long long q = 0;
     CK(cudaMemcpyAsync(&c, cnt, 4, cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(&q, queue, 8, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    if (q) {
+      k_order_expand_long<<<egrid, 256, 0, st>>>(g->out.rd, g->out.col, g->in.rd, g->in.col, perm, lo, inv, cand,
+                                                 next, cnt, queue, long_v, long_base);
+      count_launch();
+      CK(cudaMemcpyAsync(&c, cnt, 4, cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));
+    }
     if (c) {
       k_order_keys<<<grid_of(c), 256, 0, st>>>(next, c, cand, keys);
       count_launch();

@@ -234,10 +234,12 @@ size_t scan_tmp_words(uint64_t n);
 void exclusive_scan_u32(const uint32_t *in, uint32_t *out, uint64_t n, uint32_t *tmp, cudaStream_t st);
 
 // Sort n 64-bit keys on their low `bits` bits (stable LSD radix; one block when
-// n <= kSmallSort).  keys and alt are both n long; the result is returned (one of them).
+// n <= kSmallSort).  keys and alt are both n long; the result is returned (one of them).  first:
+// keys with equal bits [first, bits) are already in the order of their bits below first, so
+// the passes over those are left out.
 size_t radix_hist_words(uint64_t n);
 uint64_t *sort_u64(uint64_t *keys, uint64_t *alt, uint64_t n, int bits, uint32_t *hist,
-                   uint32_t *scan_tmp, cudaStream_t st);
+                   uint32_t *scan_tmp, cudaStream_t st, int first = 0);
 
 // Stable sort of n (key, value) pairs by the key's low `bits` bits; *keys / *vals point at
 // the result afterwards (the inputs or the alternates).

@@ -30,6 +30,7 @@ struct Graph {
   pr_params p{};
   bool f32 = false;
   bool teleport = false;
+  bool transient = false;  // built for the vertex numbering alone: no rank state
 
   Adj out, in;
   void *R[2] = {nullptr, nullptr};   // ranks, both parities equal between calls
