@@ -1,19 +1,8 @@
-// graph.cu - device graph store: build from pairs, batch update, repack, export.
+// graph.cu - device graph store: build from pairs, repack, export (batch updates: apply.cu).
 //
 // Section 3.2 of the paper defines a batch update as E^t = (E^{t-1} \ D) U I with
 // effective deletions Delta^- = E^{t-1} \ E^t and insertions Delta^+ = E^t \ E^{t-1};
 // Section 3.1 / 5.1.4 add a self-loop to every vertex (kept fixed across updates).
-//
-// Update pipeline (all on the handle's stream):
-//   keys (u << b | v) of the requested pairs in sequence order -> stable sort -> the last
-//   request on each edge decides its state, and the edges whose state changes are the
-//   effective changes (self pairs, duplicates, deletions of absent edges, deletions that
-//   are re-inserted and insertions of present edges drop out) -> tagged change list in
-//   (u, v) order and a transposed copy sorted by (v, u) -> segments = touched rows -> one block
-//   per touched row merges the row with its changes, in place if the row's slots
-//   suffice, else into freshly allocated tail slots.  The out-row merge also refreshes
-//   the row's contribution alpha R[u] / |out(u)| and records the pending marks
-//   (sources and deleted targets) for the next Dynamic Frontier call.
 #include <algorithm>
 #include <vector>
 
@@ -44,14 +33,6 @@ static inline unsigned grid_for(uint64_t n, int threads = 256) {
   uint64_t g = (n + threads - 1) / threads;
   return (unsigned)std::max<uint64_t>(1, g);
 }
-
-constexpr int kMergeThreads = 256;
-constexpr int kMergeThreadsLong = 1024;
-constexpr uint32_t kSmemRow = 2048;   // rows up to this length are staged in shared memory
-#ifndef PRDF_LONG_ROW
-#define PRDF_LONG_ROW 8192
-#endif
-constexpr uint32_t kLongRow = PRDF_LONG_ROW;  // longer rows are merged by blocks of kMergeThreadsLong
 
 // ------------------------------------------------------------------- kernels ----
 
@@ -145,349 +126,6 @@ __global__ void k_init_rank(const uint2 *out_rd, uint32_t n, double alpha, typen
   R1[v] = r;
   C0[v] = c;
   C1[v] = c;
-}
-
-// ---- batch update ----
-
-// Chunk items of the tier-2 rows; chunk c of a row covers edges [c chunk, (c+1) chunk).
-__device__ __forceinline__ uint4 chunk_item(uint32_t v, uint2 d, uint32_t c, uint32_t nch, uint32_t number,
-                                            uint32_t chunk) {
-  uint32_t len = min(chunk, d.y - c * chunk);
-  return make_uint4(v, d.x + c * chunk, len | (c << 10) | (nch > 1 ? 0x80000000u : 0u), number);
-}
-
-
-__device__ __forceinline__ bool row_has(const uint2 *rd, const uint32_t *col, uint32_t u, uint32_t v) {
-  uint2 d = rd[u];
-  const uint32_t *c = col + d.x;
-  uint32_t lo = 0, hi = d.y;
-  while (lo < hi) {
-    uint32_t mid = (lo + hi) >> 1;
-    if (c[mid] < v) lo = mid + 1; else hi = mid;
-  }
-  return lo < d.y && c[lo] == v;
-}
-
-__device__ __forceinline__ bool sorted_has(const uint64_t *a, uint64_t n, uint64_t x) {
-  uint64_t lo = 0, hi = n;
-  while (lo < hi) {
-    uint64_t mid = (lo + hi) >> 1;
-    if (a[mid] < x) lo = mid + 1; else hi = mid;
-  }
-  return lo < n && a[lo] == x;
-}
-
-// Batch k of a sequence holding op x of one kind: the last k with off[k] <= x.
-__device__ __forceinline__ uint32_t batch_of(const uint32_t *off, int nb, uint64_t x) {
-  uint32_t lo = 0, hi = (uint32_t)nb;  // off[0] = 0 <= x
-  while (hi - lo > 1) {
-    uint32_t mid = (lo + hi) >> 1;
-    if (off[mid] <= x) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
-// Keys (u << b | v) of a sequence of batches, each request written at its place in the
-// order D_0, I_0, D_1, I_1, ... (deletions before insertions inside a batch, Section 3.2),
-// with the payload (place << 1) | is_insertion.  off = [del offsets (nb + 1), ins offsets
-// (nb + 1)], or null for a single batch.
-__global__ void k_seq_keys(const uint32_t *ds, const uint32_t *dd, uint64_t nd, const uint32_t *is,
-                           const uint32_t *id, uint64_t ni, int nb, const uint32_t *off, uint32_t n, int b,
-                           uint64_t *keys, uint32_t *vals, const uint16_t *comp, const uint32_t *inv,
-                           ApplyCtl *actl) {
-  uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nd + ni) return;
-  uint64_t u, v, at;
-  uint32_t kind;
-  if (i < nd) {
-    u = ds[i];
-    v = dd[i];
-    kind = 0;
-    at = off ? off[nb + 1 + batch_of(off, nb, i)] + i : i;
-  } else {
-    const uint64_t j = i - nd;
-    u = is[j];
-    v = id[j];
-    kind = 1;
-    at = off ? off[batch_of(off + nb + 1, nb, j) + 1] + j : nd + j;
-  }
-  uint64_t key;
-  if (u >= n || v >= n) {
-    atomicOr(&actl->bad_id, 1u);
-    key = kSentinel;
-  } else if (comp && comp[u] != comp[v]) {
-    atomicOr(&actl->bad_comp, 1u);
-    key = kSentinel;
-  } else {
-    if (inv) {  // the handle's internal numbering
-      u = inv[u];
-      v = inv[v];
-    }
-    key = u == v ? kSentinel : ((u << b) | v);
-  }
-  keys[at] = key;
-  vals[at] = (uint32_t)(at << 1) | kind;
-}
-
-// After the stable sort every key's requests sit together in sequence order, so the last
-// one fixes the edge's final state; flags[i] = 1 where that state differs from the graph's
-// (an effective deletion or insertion).  Self pairs and repeated requests never count.
-__global__ void k_last_op(const uint64_t *keys, const uint32_t *vals, uint64_t N, const uint2 *rd,
-                          const uint32_t *col, int b, uint32_t *flags) {
-  uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  const uint64_t k = keys[i];
-  uint32_t keep = 0;
-  if (k != kSentinel && (i + 1 == N || keys[i + 1] != k)) {
-    const bool fin = vals[i] & 1u;
-    const bool was = row_has(rd, col, (uint32_t)(k >> b), (uint32_t)(k & ((1ull << b) - 1)));
-    keep = fin != was;
-  }
-  flags[i] = keep;
-}
-
-// Tagged change keys: (key << 1) | is_insertion, in row-major (u, v) order and a
-// transposed (v, u) copy.
-__global__ void k_emit_changes(const uint64_t *keys, const uint32_t *vals, uint64_t N, const uint32_t *flags,
-                               const uint32_t *pos, int b, const uint32_t *lab, uint64_t *chg, uint64_t *chg_t,
-                               ApplyCtl *actl) {
-  uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  if (flags[i]) {
-    const uint64_t k = keys[i];
-    const uint64_t tag = vals[i] & 1u;
-    const uint64_t mask = (1ull << b) - 1;
-    const uint64_t kt = ((k & mask) << b) | (lab ? (uint64_t)lab[k >> b] : k >> b);
-    chg[pos[i]] = (k << 1) | tag;
-    chg_t[pos[i]] = (kt << 1) | tag;
-    if (!tag) atomicAdd(&actl->n_eff_del, 1u);
-  }
-  if (i == N - 1) actl->n_eff = pos[i] + flags[i];
-}
-
-__device__ __forceinline__ uint32_t chg_row(uint64_t c, int b) { return (uint32_t)((c >> 1) >> b); }
-__device__ __forceinline__ uint32_t chg_col(uint64_t c, int b) { return (uint32_t)((c >> 1) & ((1ull << b) - 1)); }
-
-// flags[j] = start of a row segment; tags[j] = is_insertion; tags[K] = 0.
-__global__ void k_seg_flags(const uint64_t *chg, uint32_t K, int b, uint32_t *flags, uint32_t *tags) {
-  uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < K) {
-    flags[j] = (j == 0 || chg_row(chg[j], b) != chg_row(chg[j - 1], b)) ? 1u : 0u;
-    tags[j] = (uint32_t)(chg[j] & 1);
-  } else if (j == K) {
-    tags[j] = 0;
-  }
-}
-
-__global__ void k_seg_emit(const uint32_t *flags, const uint32_t *pos, uint32_t K, uint32_t *seg, uint32_t *nseg) {
-  uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= K) return;
-  if (flags[j]) seg[pos[j]] = j;
-  if (j == K - 1) {
-    uint32_t c = pos[j] + flags[j];
-    seg[c] = K;
-    *nseg = c;
-  }
-}
-
-// Words the moved rows need, and the long rows' staging words.
-__global__ void k_plan(const uint2 *rd, const uint32_t *cap, const uint64_t *chg, uint32_t K, int b,
-                       const uint32_t *seg, const uint32_t *nseg, const uint32_t *tagpref,
-                       unsigned long long *reloc, unsigned long long *big_need) {
-  uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= *nseg) return;
-  uint32_t s0 = seg[s], e = seg[s + 1];
-  uint32_t r = chg_row(chg[s0], b);
-  uint32_t nI = tagpref[e] - tagpref[s0], nD = (e - s0) - nI;
-  uint32_t len = rd[r].y;
-  uint32_t new_len = len - nD + nI;
-  if (new_len > cap[r]) atomicAdd(reloc, (unsigned long long)move_cap(new_len));
-  if (len > kSmemRow) atomicAdd(big_need, (unsigned long long)len);
-}
-
-// Extra work done by the merge of a row.  Out-rows (source u): contribution refresh and
-// pending marks.  In-rows: note an in-degree that crosses a bin threshold.
-template <bool F32>
-struct RowHook {
-  bool is_out;
-  double alpha;
-  typename Store<F32>::A *adeg;
-  typename Store<F32>::R *R0;
-  typename Store<F32>::C *C0, *C1;
-  uint32_t *pend_src, *pend_tgt;
-  uint32_t pend_cap;
-  uint32_t bin_lo, bin_hi;
-  uint32_t gmax, chunk;       // sweep tiers of the handle (sweep_tier)
-  uint4 *items;               // in-rows: sweep items to patch (tier and chunk count unchanged)
-  const uint32_t *item_pos;
-  const uint32_t *lab, *at;   // in-rows ordered by another key than the id (see the graph handle), or null
-};
-
-__device__ __forceinline__ int degree_bin(uint32_t d, uint32_t lo, uint32_t hi) {
-  return d <= lo ? 0 : (d <= hi ? 1 : 2);
-}
-
-// Merges one touched row (segment s of the sorted changes) with its changes; called by a
-// whole block.
-template <bool F32, int THREADS>
-__device__ void merge_row(uint32_t s, uint2 *rd, uint32_t *cap, uint32_t *col, const uint64_t *chg, int b,
-                          const uint32_t *seg, const uint32_t *tagpref, unsigned long long *tail,
-                          unsigned long long *garbage, uint32_t *big, unsigned long long *big_cursor,
-                          uint64_t col_cap, uint64_t big_cap, ApplyCtl *actl, const RowHook<F32> &hook) {
-  constexpr int kMergeThreads = THREADS;
-  __shared__ uint32_t srow[kSmemRow];
-  __shared__ uint32_t s_dest, s_big;
-  const uint32_t tid = threadIdx.x;
-  const uint32_t s0 = seg[s], e = seg[s + 1];
-  const uint32_t r = chg_row(chg[s0], b);
-  const uint2 d = rd[r];
-  const uint32_t len = d.y, cap_r = cap[r];
-  const uint32_t nI = tagpref[e] - tagpref[s0], nD = (e - s0) - nI;
-  const uint32_t new_len = len - nD + nI;
-  const bool moves = new_len > cap_r;
-  uint32_t *src_row = srow;
-  __shared__ int s_ok;
-  if (tid == 0) {
-    unsigned long long dest = moves ? atomicAdd(tail, (unsigned long long)move_cap(new_len)) : d.x;
-    unsigned long long bg = len > kSmemRow ? atomicAdd(big_cursor, (unsigned long long)len) : 0ull;
-    s_ok = (!moves || dest + move_cap(new_len) <= col_cap) && (len <= kSmemRow || bg + len <= big_cap);
-    if (!s_ok) atomicOr(&actl->overflow, 1u);
-    s_dest = (uint32_t)dest;
-    s_big = (uint32_t)bg;
-  }
-  __syncthreads();
-  if (!s_ok) return;  // no room: the row is left as it was and the host reports the failure
-  if (len > kSmemRow) src_row = big + s_big;
-  for (uint32_t j = tid; j < len; j += kMergeThreads) {
-    const uint32_t x = col[d.x + j];
-    src_row[j] = hook.lab ? hook.lab[x] : x;
-  }
-  __syncthreads();
-  uint32_t *dst = col + s_dest;
-  // A thread's entries ascend, so the first change with column >= x lies at or after the
-  // one found for its previous entry: a galloping search from there (a hub row's entries
-  // are each a few changes apart, not a whole binary search over them).
-  uint32_t lo_prev = s0;
-  for (uint32_t j = tid; j < len; j += kMergeThreads) {
-    uint32_t x = src_row[j];
-    uint32_t lo = lo_prev, hi = lo_prev, step = 1;  // changes before lo have columns < x
-    while (hi < e && chg_col(chg[hi], b) < x) {
-      lo = hi + 1;
-      hi = e - hi > step ? hi + step : e;
-      step <<= 1;
-    }
-    while (lo < hi) {  // first change with column >= x, in [lo, hi]
-      uint32_t mid = (lo + hi) >> 1;
-      if (chg_col(chg[mid], b) < x) lo = mid + 1; else hi = mid;
-    }
-    lo_prev = lo;
-    if (lo < e && chg_col(chg[lo], b) == x) continue;  // deleted
-    uint32_t ib = tagpref[lo] - tagpref[s0];
-    uint32_t db = (lo - s0) - ib;
-    dst[j - db + ib] = hook.at ? hook.at[x] : x;
-  }
-  for (uint32_t q = s0 + tid; q < e; q += kMergeThreads) {
-    uint64_t c = chg[q];
-    if (!(c & 1)) continue;
-    uint32_t y = chg_col(c, b);
-    uint32_t lo = 0, hi = len;  // old entries below y
-    while (lo < hi) {
-      uint32_t mid = (lo + hi) >> 1;
-      if (src_row[mid] < y) lo = mid + 1; else hi = mid;
-    }
-    uint32_t ib = tagpref[q] - tagpref[s0];
-    uint32_t db = (q - s0) - ib;
-    dst[lo - db + ib] = hook.at ? hook.at[y] : y;
-  }
-  // the free slots of the row's last 16 bytes say so (the sweeps read rows by 16 bytes)
-  if (tid < 4 && new_len + tid < ((new_len + 3) & ~3u)) dst[new_len + tid] = kNoCol;
-  if (hook.is_out) {
-    for (uint32_t q = s0 + tid; q < e; q += kMergeThreads) {
-      uint64_t c = chg[q];
-      if (c & 1) continue;
-      uint32_t p = atomicAdd(&actl->n_pend_tgt, 1u);
-      if (p < hook.pend_cap) hook.pend_tgt[p] = chg_col(c, b);
-    }
-  }
-  __syncthreads();
-  if (tid == 0) {
-    rd[r] = make_uint2(s_dest, new_len);
-    if (moves) {
-      cap[r] = move_cap(new_len);
-      atomicAdd(garbage, (unsigned long long)cap_r);
-    }
-    if (!hook.is_out && (sweep_tier(len, hook.bin_lo, hook.gmax) != sweep_tier(new_len, hook.bin_lo, hook.gmax) ||
-                         (sweep_tier(new_len, hook.bin_lo, hook.gmax) == 2 &&
-                          (len + hook.chunk - 1) / hook.chunk != (new_len + hook.chunk - 1) / hook.chunk))) {
-      actl->bins_changed = 1;
-      s_ok = 0;  // the sweep items are rebuilt after this update; nothing to patch
-    }
-    if (hook.is_out) {
-      using S = Store<F32>;
-      typename S::A a = S::factor(hook.alpha, new_len);
-      hook.adeg[r] = a;
-      typename S::C c = S::contrib(hook.R0[r], a);
-      hook.C0[r] = c;
-      hook.C1[r] = c;
-      if ((len == 0) != (new_len == 0)) actl->dead_changed = 1;
-      uint32_t p = atomicAdd(&actl->n_pend_src, 1u);
-      if (p < hook.pend_cap) hook.pend_src[p] = r;
-    }
-  }
-  if (!hook.is_out) {
-    // keep the sweep items of this in-row current (start and length)
-    __syncthreads();
-    if (s_ok) {
-      const uint2 nd = make_uint2(s_dest, new_len);
-      const uint32_t pos = hook.item_pos[r];
-      if (sweep_tier(new_len, hook.bin_lo, hook.gmax) < 2) {
-        if (tid == 0) hook.items[pos] = make_uint4(r, nd.x, nd.y, 0u);
-      } else {
-        const uint32_t nch = (new_len + hook.chunk - 1) / hook.chunk;
-        const uint32_t number0 = hook.items[pos].w;
-        for (uint32_t c = tid; c < nch; c += kMergeThreads)
-          hook.items[pos + c] = chunk_item(r, nd, c, nch, number0 + c, hook.chunk);
-      }
-    }
-  }
-}
-
-// One block per touched row of at most kLongRow entries; the longer rows are listed (their
-// segments in long_seg) for k_merge_long, whose blocks of kMergeThreadsLong take them in
-// turn: a hub row's entries are four times as many threads' work, and only as many blocks
-// as the GPU holds are launched for them.
-template <bool F32>
-__global__ void __launch_bounds__(kMergeThreads) k_merge(uint2 *rd, uint32_t *cap, uint32_t *col, const uint64_t *chg,
-                                                         int b, const uint32_t *seg, const uint32_t *nseg,
-                                                         const uint32_t *tagpref, unsigned long long *tail,
-                                                         unsigned long long *garbage, uint32_t *big,
-                                                         unsigned long long *big_cursor, uint64_t col_cap,
-                                                         uint64_t big_cap, ApplyCtl *actl, RowHook<F32> hook,
-                                                         uint32_t *long_seg) {
-  const uint32_t s = blockIdx.x;
-  if (s >= *nseg) return;
-  if (rd[chg_row(chg[seg[s]], b)].y > kLongRow) {
-    if (threadIdx.x == 0) long_seg[atomicAdd(&actl->n_long, 1u)] = s;
-    return;
-  }
-  merge_row<F32, kMergeThreads>(s, rd, cap, col, chg, b, seg, tagpref, tail, garbage, big, big_cursor, col_cap,
-                                big_cap, actl, hook);
-}
-
-template <bool F32>
-__global__ void __launch_bounds__(kMergeThreadsLong) k_merge_long(uint2 *rd, uint32_t *cap, uint32_t *col,
-                                                                  const uint64_t *chg, int b, const uint32_t *seg,
-                                                                  const uint32_t *tagpref, unsigned long long *tail,
-                                                                  unsigned long long *garbage, uint32_t *big,
-                                                                  unsigned long long *big_cursor, uint64_t col_cap,
-                                                                  uint64_t big_cap, ApplyCtl *actl,
-                                                                  RowHook<F32> hook, const uint32_t *long_seg) {
-  const uint32_t n_long = *(volatile uint32_t *)&actl->n_long;
-  for (uint32_t k = blockIdx.x; k < n_long; k += gridDim.x) {
-    merge_row<F32, kMergeThreadsLong>(long_seg[k], rd, cap, col, chg, b, seg, tagpref, tail, garbage, big, big_cursor,
-                                      col_cap, big_cap, actl, hook);
-    __syncthreads();  // the block's shared staging is reused by its next row
-  }
 }
 
 // ---- repack / export / bins ----
@@ -828,7 +466,8 @@ pr_status apply_scratch(Graph *g, uint64_t N) {
   CK(dalloc(&s.pos, cap + 2));
   CK(dalloc(&s.seg, 2 * (cap + 2)));
   CK(dalloc(&s.tagpref, 2 * (cap + 2)));
-  s.radix_hist_cap = radix_hist_words(cap) + 256;
+  // (the plan of an update in one launch keeps 256 + 8 words a block there)
+  s.radix_hist_cap = std::max<uint64_t>(radix_hist_words(cap) + 256, 264ull * g->sm_count);
   CK(dalloc(&s.radix_hist, s.radix_hist_cap));
   s.scan_tmp_cap = scan_tmp_words(std::max<uint64_t>(cap + 2, s.radix_hist_cap)) + 1;
   CK(dalloc(&s.scan_tmp, s.scan_tmp_cap));
@@ -837,7 +476,7 @@ pr_status apply_scratch(Graph *g, uint64_t N) {
 }
 
 // Rebuilds adjacency A with fresh slack and at least `reserve` free tail words.
-static pr_status repack_adj(Graph *g, Adj &A, uint64_t reserve) {
+pr_status repack_adj(Graph *g, Adj &A, uint64_t reserve) {
   const uint32_t n = g->n;
   cudaStream_t st = g->st;
   k_len_caps<<<grid_for(n), 256, 0, st>>>(A.rd, n, A.cap); count_launch();
@@ -865,198 +504,6 @@ static pr_status repack_adj(Graph *g, Adj &A, uint64_t reserve) {
   A.used = total;
   A.garbage = 0;
   return PR_OK;
-}
-
-pr_status graph_apply(Graph *g, uint64_t nd, const uint32_t *ds, const uint32_t *dd, uint64_t ni, const uint32_t *is,
-                      const uint32_t *id, int nb, const uint32_t *off) {
-  const uint64_t N = nd + ni;
-  if (N == 0) return PR_OK;
-  cudaStream_t st = g->st;
-  pr_status rc = apply_scratch(g, N);
-  if (rc != PR_OK) return rc;
-  ApplyScratch &s = g->sc;
-  const int b = g->b;
-  const int kbits = 2 * b + 1;
-
-  ApplyCtl &h = *g->actl_h;
-  memset(&h, 0, sizeof(ApplyCtl));
-  h.n_pend_src = g->n_pend_src;
-  h.n_pend_tgt = g->n_pend_tgt;
-  h.tail_out = g->out.used;
-  h.tail_in = g->in.used;
-  CK(cudaMemcpyAsync(g->actl, &h, sizeof(ApplyCtl), cudaMemcpyHostToDevice, st));
-
-  k_seq_keys<<<grid_for(N), 256, 0, st>>>(ds, dd, nd, is, id, ni, nb, off, g->n, b, s.kd, s.vals, g->comp,
-                                          g->inv, g->actl); count_launch();
-  uint64_t *keys = s.kd;
-  uint32_t *vals = s.vals;
-  sort_u64_kv(&keys, &vals, s.tmp, s.vals2, N, 2 * b, s.radix_hist, s.scan_tmp, st);
-  k_last_op<<<grid_for(N), 256, 0, st>>>(keys, vals, N, g->out.rd, g->out.col, b, s.flags); count_launch();
-  exclusive_scan_u32(s.flags, s.pos, N, s.scan_tmp, st);
-  k_emit_changes<<<grid_for(N), 256, 0, st>>>(keys, vals, N, s.flags, s.pos, b, g->lab, s.chg, s.chg_t, g->actl); count_launch();
-  CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(&h, g->actl, sizeof(ApplyCtl), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  if (h.bad_id) {
-    g->err = "vertex id out of range";
-    return PR_ERR_VERTEX_RANGE;
-  }
-  if (h.bad_comp) {
-    g->err = "a pair joins two different graphs of a batched handle";
-    return PR_ERR_INVALID_ARG;
-  }
-  const uint32_t K = h.n_eff;
-  const uint32_t K_del = h.n_eff_del;
-  if (K == 0) return PR_OK;
-
-  // the change list is already in (u, v) order (one entry per key); only the transposed
-  // copy needs a sort
-  uint64_t *co = s.chg;
-  uint64_t *ci = sort_u64(s.chg_t, s.tmp2, K, kbits, s.radix_hist, s.scan_tmp, st, g->lab ? 1 : b + 1);
-  uint32_t *seg_o = s.seg, *seg_i = s.seg + (s.cap + 2);
-  uint32_t *tp_o = s.tagpref, *tp_i = s.tagpref + (s.cap + 2);
-  ApplyCtl *dctl = g->actl;
-  // segments of the out-row changes
-  k_seg_flags<<<grid_for(K + 1), 256, 0, st>>>(co, K, b, s.flags, tp_o); count_launch();
-  exclusive_scan_u32(s.flags, s.pos, K, s.scan_tmp, st);
-  exclusive_scan_u32(tp_o, tp_o, K + 1, s.scan_tmp, st);
-  k_seg_emit<<<grid_for(K), 256, 0, st>>>(s.flags, s.pos, K, seg_o, &dctl->n_seg_out); count_launch();
-  k_plan<<<grid_for(K), 256, 0, st>>>(g->out.rd, g->out.cap, co, K, b, seg_o, &dctl->n_seg_out, tp_o,
-                                      &dctl->reloc_out, &dctl->big_cursor); count_launch();
-  // segments of the in-row changes
-  k_seg_flags<<<grid_for(K + 1), 256, 0, st>>>(ci, K, b, s.flags, tp_i); count_launch();
-  exclusive_scan_u32(s.flags, s.pos, K, s.scan_tmp, st);
-  exclusive_scan_u32(tp_i, tp_i, K + 1, s.scan_tmp, st);
-  k_seg_emit<<<grid_for(K), 256, 0, st>>>(s.flags, s.pos, K, seg_i, &dctl->n_seg_in); count_launch();
-  k_plan<<<grid_for(K), 256, 0, st>>>(g->in.rd, g->in.cap, ci, K, b, seg_i, &dctl->n_seg_in, tp_i,
-                                      &dctl->reloc_in, &dctl->big_cursor); count_launch();
-  CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(&h, g->actl, sizeof(ApplyCtl), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-
-  // room for moved rows and staging of long rows; a repack gives rows fresh (possibly
-  // smaller) slack, so the plan is redone after one
-  for (int round = 0; round < 4; round++) {
-    bool again = false;
-    if (g->out.used + h.reloc_out > g->out.col_cap) {
-      rc = repack_adj(g, g->out, 2 * h.reloc_out);
-      if (rc != PR_OK) return rc;
-      again = true;
-    }
-    if (g->in.used + h.reloc_in > g->in.col_cap) {
-      rc = repack_adj(g, g->in, 2 * h.reloc_in);
-      if (rc != PR_OK) return rc;
-      again = true;
-    }
-    if (!again) break;
-    CK(cudaMemsetAsync(&dctl->reloc_out, 0, 16, st));  // reloc_out, reloc_in
-    CK(cudaMemsetAsync(&dctl->big_cursor, 0, 8, st));
-    k_plan<<<grid_for(K), 256, 0, st>>>(g->out.rd, g->out.cap, co, K, b, seg_o, &dctl->n_seg_out, tp_o,
-                                        &dctl->reloc_out, &dctl->big_cursor); count_launch();
-    k_plan<<<grid_for(K), 256, 0, st>>>(g->in.rd, g->in.cap, ci, K, b, seg_i, &dctl->n_seg_in, tp_i,
-                                        &dctl->reloc_in, &dctl->big_cursor); count_launch();
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(&h, g->actl, sizeof(ApplyCtl), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-  }
-  if (h.big_cursor > g->big_cap) {
-    cudaFree(g->big);
-    g->big = nullptr;
-    g->big_cap = 0;
-    uint64_t c = std::max<uint64_t>(h.big_cursor * 2, 1u << 20);
-    CK(dalloc(&g->big, c));
-    g->big_cap = c;
-  }
-  h.tail_out = g->out.used;
-  h.tail_in = g->in.used;
-  h.big_cursor = 0;
-  CK(cudaMemcpyAsync(&dctl->tail_out, &h.tail_out, 16, cudaMemcpyHostToDevice, st));  // tail_out, tail_in
-  CK(cudaMemsetAsync(&dctl->big_cursor, 0, 8, st));
-
-  const uint32_t lo = (uint32_t)g->p.bin_lo, hi_b = (uint32_t)g->p.bin_hi;
-  const unsigned long_grid = (unsigned)std::max(1, 2 * g->sm_count);
-  if (g->f32) {
-    using S = Store<true>;
-    RowHook<true> ho{true, g->p.alpha, (S::A *)g->adeg, (S::R *)g->R[0], (S::C *)g->C[0], (S::C *)g->C[1],
-                     g->pend_src, g->pend_tgt, g->pend_cap, lo, hi_b, g->group_max, g->chunk_len, nullptr, nullptr,
-                     nullptr, nullptr};
-    RowHook<true> hin{false,   g->p.alpha,   nullptr,      nullptr,       nullptr, nullptr, nullptr,
-                      nullptr, 0,            lo,           hi_b,          g->group_max, g->chunk_len,
-                      g->items, g->item_pos, g->lab,       g->at};
-    CK(cudaMemsetAsync(&dctl->n_long, 0, 4, st));
-    k_merge<true><<<K, kMergeThreads, 0, st>>>(g->out.rd, g->out.cap, g->out.col, co, b, seg_o, &dctl->n_seg_out,
-                                               tp_o, &dctl->tail_out, &dctl->garbage_out, g->big, &dctl->big_cursor,
-                                               g->out.col_cap, g->big_cap, dctl, ho, s.flags);
-    count_launch();
-    k_merge_long<true><<<long_grid, kMergeThreadsLong, 0, st>>>(g->out.rd, g->out.cap, g->out.col, co, b, seg_o,
-                                               tp_o, &dctl->tail_out, &dctl->garbage_out, g->big, &dctl->big_cursor,
-                                               g->out.col_cap, g->big_cap, dctl, ho, s.flags);
-    count_launch();
-    CK(cudaMemsetAsync(&dctl->n_long, 0, 4, st));
-    k_merge<true><<<K, kMergeThreads, 0, st>>>(g->in.rd, g->in.cap, g->in.col, ci, b, seg_i, &dctl->n_seg_in, tp_i,
-                                               &dctl->tail_in, &dctl->garbage_in, g->big, &dctl->big_cursor,
-                                               g->in.col_cap, g->big_cap, dctl, hin, s.flags);
-    count_launch();
-    k_merge_long<true><<<long_grid, kMergeThreadsLong, 0, st>>>(g->in.rd, g->in.cap, g->in.col, ci, b, seg_i, tp_i,
-                                               &dctl->tail_in, &dctl->garbage_in, g->big, &dctl->big_cursor,
-                                               g->in.col_cap, g->big_cap, dctl, hin, s.flags);
-    count_launch();
-  } else {
-    using S = Store<false>;
-    RowHook<false> ho{true, g->p.alpha, (S::A *)g->adeg, (S::R *)g->R[0], (S::C *)g->C[0], (S::C *)g->C[1],
-                      g->pend_src, g->pend_tgt, g->pend_cap, lo, hi_b, g->group_max, g->chunk_len, nullptr, nullptr,
-                     nullptr, nullptr};
-    RowHook<false> hin{false,   g->p.alpha,   nullptr,      nullptr,       nullptr, nullptr, nullptr,
-                       nullptr, 0,            lo,           hi_b,          g->group_max, g->chunk_len,
-                       g->items, g->item_pos, nullptr,      nullptr};
-    CK(cudaMemsetAsync(&dctl->n_long, 0, 4, st));
-    k_merge<false><<<K, kMergeThreads, 0, st>>>(g->out.rd, g->out.cap, g->out.col, co, b, seg_o, &dctl->n_seg_out,
-                                                tp_o, &dctl->tail_out, &dctl->garbage_out, g->big, &dctl->big_cursor,
-                                                g->out.col_cap, g->big_cap, dctl, ho, s.flags);
-    count_launch();
-    k_merge_long<false><<<long_grid, kMergeThreadsLong, 0, st>>>(g->out.rd, g->out.cap, g->out.col, co, b, seg_o,
-                                                tp_o, &dctl->tail_out, &dctl->garbage_out, g->big, &dctl->big_cursor,
-                                                g->out.col_cap, g->big_cap, dctl, ho, s.flags);
-    count_launch();
-    CK(cudaMemsetAsync(&dctl->n_long, 0, 4, st));
-    k_merge<false><<<K, kMergeThreads, 0, st>>>(g->in.rd, g->in.cap, g->in.col, ci, b, seg_i, &dctl->n_seg_in, tp_i,
-                                                &dctl->tail_in, &dctl->garbage_in, g->big, &dctl->big_cursor,
-                                                g->in.col_cap, g->big_cap, dctl, hin, s.flags);
-    count_launch();
-    k_merge_long<false><<<long_grid, kMergeThreadsLong, 0, st>>>(g->in.rd, g->in.cap, g->in.col, ci, b, seg_i, tp_i,
-                                                &dctl->tail_in, &dctl->garbage_in, g->big, &dctl->big_cursor,
-                                                g->in.col_cap, g->big_cap, dctl, hin, s.flags);
-    count_launch();
-  }
-  CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(&h, g->actl, sizeof(ApplyCtl), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  if (h.overflow) {
-    g->err = "internal error: no room for a moved row (graph rows partly updated)";
-    return PR_ERR_CUDA;
-  }
-
-  g->m = g->m + (uint64_t)(K - K_del) - (uint64_t)K_del;
-  g->out.used = h.tail_out;
-  g->in.used = h.tail_in;
-  g->out.garbage += h.garbage_out;
-  g->in.garbage += h.garbage_in;
-  g->n_pend_src = std::min(h.n_pend_src, g->pend_cap);
-  g->n_pend_tgt = std::min(h.n_pend_tgt, g->pend_cap);
-  if (h.n_pend_src > g->pend_cap || h.n_pend_tgt > g->pend_cap) g->pend_all = true;
-  if (h.dead_changed) g->dead_dirty = true;
-  if (h.bins_changed) g->ident_dirty = true;
-  // give abandoned slots back once they dominate
-  if (g->out.garbage > g->out.used / 2 && g->out.garbage > 1024) {
-    rc = repack_adj(g, g->out, 0);
-    if (rc != PR_OK) return rc;
-  }
-  if (g->in.garbage > g->in.used / 2 && g->in.garbage > 1024) {
-    rc = repack_adj(g, g->in, 0);
-    if (rc != PR_OK) return rc;
-  }
-  // the degree-binned vertex order used by full and dense sweeps follows the graph
-  return graph_refresh_ident(g);
 }
 
 pr_status graph_export(Graph *g, int dir, uint64_t *offs_h, uint32_t *cols_h) {
@@ -1316,6 +763,7 @@ void graph_free(Graph *g) {
   cudaFree(g->actl);
   if (g->actl_h) cudaFreeHost(g->actl_h);
   cudaFree(g->big);
+  cudaFree(g->longs);
   cudaFree(g->gen_tmp);
   cudaFree(g->gen_tmp2);
   cudaFree(g->perm);

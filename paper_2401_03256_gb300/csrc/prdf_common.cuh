@@ -214,15 +214,15 @@ struct ApplyCtl {
   unsigned long long reloc_out, reloc_in;   // words needed by rows that must move
   unsigned long long tail_out, tail_in;     // running allocation cursors (device)
   unsigned long long garbage_out, garbage_in;
-  uint32_t n_pend_src, n_pend_tgt;          // pending marks after this update
-  uint32_t pend_overflow;
   uint32_t dead_changed;
   uint32_t n_eff_del;                       // effective deletions among n_eff
   uint32_t overflow;                        // a merge found no room (graph left unchanged rows)
   uint32_t bins_changed;                    // an in-degree crossed a bin threshold
   uint32_t bad_comp;                        // a pair joins two graphs of a batched handle
-  unsigned long long big_cursor;            // global scratch cursor for long rows
-  uint32_t n_long;                          // rows left by the merge for its long-row pass
+  unsigned long long big_need, big_cursor;  // staging words of the long rows: in all, given out
+  unsigned long long longq;                 // long rows queued by the merge (high word) and their slices (low)
+  uint32_t n_long;                          // long rows among the touched ones
+  uint32_t bar, err;                        // grid barrier of the plan; a wait of it ran out
 };
 
 // ------------------------------------------------------------------- primitives ---
@@ -240,11 +240,6 @@ void exclusive_scan_u32(const uint32_t *in, uint32_t *out, uint64_t n, uint32_t 
 size_t radix_hist_words(uint64_t n);
 uint64_t *sort_u64(uint64_t *keys, uint64_t *alt, uint64_t n, int bits, uint32_t *hist,
                    uint32_t *scan_tmp, cudaStream_t st, int first = 0);
-
-// Stable sort of n (key, value) pairs by the key's low `bits` bits; *keys / *vals point at
-// the result afterwards (the inputs or the alternates).
-void sort_u64_kv(uint64_t **keys, uint32_t **vals, uint64_t *alt_k, uint32_t *alt_v, uint64_t n, int bits,
-                 uint32_t *hist, uint32_t *scan_tmp, cudaStream_t st);
 
 int bits_for(uint32_t n);  // bits needed for ids in [0, n), at least 1
 

@@ -91,8 +91,10 @@ struct Graph {
 
   ApplyScratch sc;
   ApplyCtl *actl = nullptr, *actl_h = nullptr;
-  uint32_t *big = nullptr;           // scratch for rows longer than shared memory
+  uint32_t *big = nullptr;           // updates: staging of the long rows' entries
   uint64_t big_cap = 0;
+  void *longs = nullptr;             // updates: long rows' merge entries
+  uint32_t long_cap = 0;
   uint32_t *gen_tmp = nullptr;       // general scratch (scans, flags) sized n + 8
   uint32_t *gen_tmp2 = nullptr;
   uint32_t *scan_tmp = nullptr;      // block sums of scans over n
@@ -139,6 +141,7 @@ pr_status graph_build(Graph *g, uint64_t m_in, const uint32_t *src_d, const uint
 pr_status graph_apply(Graph *g, uint64_t nd, const uint32_t *ds_d, const uint32_t *dd_d, uint64_t ni,
                       const uint32_t *is_d, const uint32_t *id_d, int nb, const uint32_t *off_d);
 pr_status apply_scratch(Graph *g, uint64_t N);
+pr_status repack_adj(Graph *g, Adj &A, uint64_t reserve);
 constexpr int kOrderFromMax = 0, kOrderFromSeeds = 1, kOrderPerGraph = 2;
 pr_status vertex_order(Graph *g, int kind, uint32_t *perm, uint32_t *inv,
                        const std::vector<uint32_t> *comp_n = nullptr);

@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(1024) k_block_sort(uint64_t *keys, uint32_t n)
 
 // A block sorts a tile of ITEMS keys per thread: 16 (4096 keys) for large sorts, 4 (1024
 // keys) below kSmallTileKeys, where 4096-key tiles leave most SMs idle and every pass is
-// bound by one block's serial work (the sorts of a graph update are of this size).
+// bound by one block's serial work.
 constexpr int kRadixThreads = 256;
 constexpr int kRadixWarps = kRadixThreads / 32;
 constexpr int kRadixItemsSmall = 4, kRadixItemsLarge = 16;
@@ -136,19 +136,17 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const uint64_t *ke
   hist[(uint64_t)threadIdx.x * nblocks + blockIdx.x] = cnt[threadIdx.x];
 }
 
-// Stable scatter of a tile (and its values).  Warp w ranks its 32 * ITEMS consecutive keys round
+// Stable scatter of a tile.  Warp w ranks its 32 * ITEMS consecutive keys round
 // by round with __match_any_sync; per-warp digit counts are then offset across warps (warp
 // order = index order).  The keys meet in shared memory in digit order and leave for their
 // places from there: neighbouring lanes write neighbouring words of a digit's run (a tile of
 // 4096 keys has 16 a digit), where writing them straight from registers took 2 to 3 times as
 // long (18 M keys, 8 bits: 0.23 to 0.27 ms a pass, now 0.10 to 0.14).
-template <int ITEMS, bool KV>
-__global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(const uint64_t *keys, const uint32_t *vals,
-                                                                 uint64_t *out, uint32_t *vout, uint64_t n,
+template <int ITEMS>
+__global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(const uint64_t *keys, uint64_t *out, uint64_t n,
                                                                  int shift, const uint32_t *hist, uint32_t nblocks) {
   constexpr int kRadixItems = ITEMS, kRadixTile = kRadixThreads * ITEMS, kWarpKeys = kRadixTile / kRadixWarps;
   __shared__ uint64_t skey[kRadixTile];
-  __shared__ uint32_t sval[KV ? kRadixTile : 1];
   __shared__ uint32_t wcnt[kRadixWarps][256];
   __shared__ uint32_t gofs[256];  // place of a digit's first key, less its place in the tile
   __shared__ uint32_t wsum[kRadixWarps];
@@ -158,13 +156,11 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(const uint64_t 
   __syncthreads();
   const uint64_t tile = (uint64_t)blockIdx.x * kRadixTile, base = tile + (uint64_t)warp * kWarpKeys;
   uint64_t k[kRadixItems];
-  uint32_t v[KV ? kRadixItems : 1];
   uint16_t local[kRadixItems];
 #pragma unroll
   for (int r = 0; r < kRadixItems; r++) {
     uint64_t idx = base + (uint64_t)r * 32 + lane;
     k[r] = idx < n ? keys[idx] : 0ull;
-    if constexpr (KV) v[r] = idx < n ? vals[idx] : 0u;
   }
 #pragma unroll
   for (int r = 0; r < kRadixItems; r++) {
@@ -206,87 +202,14 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(const uint64_t 
     if (base + (uint64_t)r * 32 + lane < n) {
       const uint32_t at = wcnt[warp][(k[r] >> shift) & 0xFF] + local[r];
       skey[at] = k[r];
-      if constexpr (KV) sval[at] = v[r];
     }
   }
   __syncthreads();
   const uint32_t have = (uint32_t)(n - tile < (uint64_t)kRadixTile ? n - tile : (uint64_t)kRadixTile);
   for (uint32_t i = threadIdx.x; i < have; i += kRadixThreads) {
     const uint64_t key = skey[i];
-    const uint32_t at = gofs[(key >> shift) & 0xFF] + i;
-    out[at] = key;
-    if constexpr (KV) vout[at] = sval[i];
+    out[gofs[(key >> shift) & 0xFF] + i] = key;
   }
-}
-
-// Key-value variants: equal keys keep the order of their values (the values enter in
-// ascending order), so a stable sort by key is also a sort by (key, value).
-__global__ void __launch_bounds__(1024) k_block_sort_kv(uint64_t *keys, uint32_t *vals, uint32_t n) {
-  __shared__ uint64_t sk[kSmallSort / 2];
-  __shared__ uint32_t sv[kSmallSort / 2];
-  uint32_t p = 2;
-  while (p < n) p <<= 1;
-  for (uint32_t i = threadIdx.x; i < p; i += blockDim.x) {
-    sk[i] = i < n ? keys[i] : kSentinel;
-    sv[i] = i < n ? vals[i] : 0xFFFFFFFFu;
-  }
-  __syncthreads();
-  for (uint32_t k = 2; k <= p; k <<= 1) {
-    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-      for (uint32_t i = threadIdx.x; i < p; i += blockDim.x) {
-        uint32_t l = i ^ j;
-        if (l > i) {
-          uint64_t a = sk[i], b = sk[l];
-          uint32_t va = sv[i], vb = sv[l];
-          bool gt = a > b || (a == b && va > vb);
-          bool up = (i & k) == 0;
-          if (gt == up) {
-            sk[i] = b;
-            sk[l] = a;
-            sv[i] = vb;
-            sv[l] = va;
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
-  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-    keys[i] = sk[i];
-    vals[i] = sv[i];
-  }
-}
-
-template <int ITEMS>
-void radix_kv(uint64_t **keys, uint32_t **vals, uint64_t *alt_k, uint32_t *alt_v, uint64_t n, int bits,
-              uint32_t *hist, uint32_t *scan_tmp, cudaStream_t st) {
-  constexpr int kRadixTile = kRadixThreads * ITEMS;
-  const uint32_t nblocks = (uint32_t)((n + kRadixTile - 1) / kRadixTile);
-  uint64_t *sk = *keys, *dk = alt_k;
-  uint32_t *sv = *vals, *dv = alt_v;
-  for (int shift = 0; shift < bits; shift += 8) {
-    k_radix_hist<ITEMS><<<nblocks, kRadixThreads, 0, st>>>(sk, n, shift, hist, nblocks);
-    count_launch();
-    exclusive_scan_u32(hist, hist, (uint64_t)256 * nblocks, scan_tmp, st);
-    k_radix_scatter<ITEMS, true><<<nblocks, kRadixThreads, 0, st>>>(sk, sv, dk, dv, n, shift, hist, nblocks);
-    count_launch();
-    std::swap(sk, dk);
-    std::swap(sv, dv);
-  }
-  *keys = sk;
-  *vals = sv;
-}
-
-void sort_u64_kv(uint64_t **keys, uint32_t **vals, uint64_t *alt_k, uint32_t *alt_v, uint64_t n, int bits,
-                 uint32_t *hist, uint32_t *scan_tmp, cudaStream_t st) {
-  if (n < 2) return;
-  if (n <= kSmallSort / 2) {
-    k_block_sort_kv<<<1, 1024, 0, st>>>(*keys, *vals, (uint32_t)n);
-    count_launch();
-    return;
-  }
-  if (n < kSmallTileKeys) radix_kv<kRadixItemsSmall>(keys, vals, alt_k, alt_v, n, bits, hist, scan_tmp, st);
-  else radix_kv<kRadixItemsLarge>(keys, vals, alt_k, alt_v, n, bits, hist, scan_tmp, st);
 }
 
 size_t radix_hist_words(uint64_t n) {
@@ -312,9 +235,7 @@ uint64_t *radix_keys(uint64_t *keys, uint64_t *alt, uint64_t n, int first, int b
   for (int shift = first; shift < bits; shift += 8) {
     k_radix_hist<ITEMS><<<nblocks, kRadixThreads, 0, st>>>(src, n, shift, hist, nblocks); count_launch();
     exclusive_scan_u32(hist, hist, (uint64_t)256 * nblocks, scan_tmp, st);
-    k_radix_scatter<ITEMS, false><<<nblocks, kRadixThreads, 0, st>>>(src, nullptr, dst, nullptr, n, shift, hist,
-                                                                     nblocks);
-    count_launch();
+    k_radix_scatter<ITEMS><<<nblocks, kRadixThreads, 0, st>>>(src, dst, n, shift, hist, nblocks); count_launch();
     uint64_t *t = src;
     src = dst;
     dst = t;
