@@ -335,8 +335,10 @@ __device__ __noinline__ DtOut dt_search(const RankArgs<F32> &a, uint32_t epoch, 
 // call to the sweep launches before its first dense iteration and before any
 // iteration over every vertex; its instance carries no dense or full sweep code.
 // 2: of a batched handle in self-loop mode (the iterations follow in batch.cu).
+// 3: as 1, for calls that mark much at once (kFewMarks).
 template <bool F32, bool DF, int SPLIT = 0>
-__global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const RankArgs<F32> a) {
+__global__ void __launch_bounds__(kRankBlock, SPLIT == 1 ? kFewMarksBlocks : PRDF_RANK_MIN_BLOCKS)
+    k_rank(const RankArgs<F32> a) {
   using S = Store<F32>;
   using R = typename S::R;
   using C = typename S::C;
@@ -358,7 +360,7 @@ __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const
   constexpr bool df = DF;
   // per-component state (batched form), identical in every block; a split call's marking
   // launch serves one graph in self-loop mode (no components, no teleport)
-  const bool multi = SPLIT != 1 && a.ncomp > 1;
+  const bool multi = SPLIT != 1 && SPLIT != 3 && a.ncomp > 1;
   const bool tele = SPLIT == 0 && a.teleport;
   const uint32_t nc = a.ncomp;
   extern __shared__ unsigned long long dsm[];
@@ -473,7 +475,7 @@ __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const
     for (uint32_t k = gtid; k < a.n_dead; k += nthreads) dacc.add(ldcg(a.R0 + __ldg(a.dead + k)));
   }
   const uint32_t zero_cnt[3] = {0, 0, 0};
-  WarpBuf wb{s_mbuf[wib], {0u, 0u, 0u, 0u}, false, 0u};
+  WarpBuf wb{s_mbuf[wib], {0u, 0u, 0u, 0u}, false, 0u, false};
   // expansion-list entries already scanned; read before any barrier of this launch, since
   // the sweeps append to the list once the first barrier is passed
   uint32_t xdone = 0;
@@ -654,16 +656,18 @@ __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const
     };
     // sparse iterations: whether v's out-row is marked now; a deferred iteration records
     // the change flag instead (the out-row is then marked by the next iteration's pull)
-    auto sparse_push = [&](uint32_t v, B dr) -> int {
+    auto sparse_push = [&](uint32_t v, B dr, uint32_t xw) -> int {
       if (!expand) return 0;
       const bool big = dr > a.ftol;
       if (defer) {
         a.emap[(size_t)(it & 1) * a.n + v] = big ? 1 : 0;
-        if (big) first_expansion(a.xbits, v);
+        if (big) first_expansion_pre(a.xbits, v, xw);
         return 0;
       }
-      return big && first_expansion(a.xbits, v);
+      return big && first_expansion_pre(a.xbits, v, xw);
     };
+    // v's word of the expansion bits, read with its row
+    auto push_word = [&](uint32_t v) -> uint32_t { return expand ? __ldcg(a.xbits + (v >> 5)) : ~0u; };
 
     if (SPLIT == 0 && (I.full || dense)) {
       const uint32_t off1 = a.it_c0, off2 = a.it_c0 + a.it_c1;
@@ -750,16 +754,21 @@ __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const
         const uint32_t i = b0 + lane;
         int push = 0;
         uint32_t v = 0;
-        if (i < cnt[0] && live(ldcg(a.list0 + i))) {
+        bool mine = i < cnt[0];
+        if (mine) {
           v = ldcg(a.list0 + i);
+          mine = live(v);
+        }
+        if (mine) {
           const R rold = ldcg(Rin + v);
           const typename S::A ad = __ldg(a.adeg + v);
           const uint2 d = __ldg(&a.in_rd[v]);
+          const uint32_t xw = push_word(v);
           C sum = row_sum_thread(Cin, a.in_col + d.x, d.y, pol_cols, pol_c);
           B dr = finish_at(v, sum, rold, ad);
           my_v++;
           my_e += d.y;
-          push = sparse_push(v, dr);
+          push = sparse_push(v, dr, xw);
         }
         if (expand) expand_if(push, v);
       }
@@ -768,20 +777,28 @@ __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const
       for (uint32_t i = gwarp; i < cnt[1]; i += nwarps) {
         const uint32_t v = ldcg(a.list1 + i);
         if (!live(v)) continue;
+        const R rold = ldcg(Rin + v);
+        const typename S::A ad = __ldg(a.adeg + v);
         const uint2 d = __ldg(&a.in_rd[v]);
+        const uint32_t xw = push_word(v);
         const uint32_t *cols = a.in_col + d.x;
         C sum = (C)0;
-        for (uint32_t j = lane * 4; j < d.y; j += 128) {
-          uint4 q = ld_cols(cols + j, pol_cols);
-          sum += gather4(Cin, q, min(4u, d.y - j), pol_c);
+        for (uint32_t j0 = lane * 4; j0 < d.y; j0 += 256) {
+          uint4 q[2];
+#pragma unroll
+          for (int r = 0; r < 2; r++)
+            if (j0 + r * 128 < d.y) q[r] = ld_cols(cols + j0 + r * 128, pol_cols);
+#pragma unroll
+          for (int r = 0; r < 2; r++)
+            if (j0 + r * 128 < d.y) sum += gather4(Cin, q[r], min(4u, d.y - j0 - r * 128), pol_c);
         }
         sum = warp_sum(sum);
         int exp_now = 0;
         if (lane == 0) {
-          B dr = finish_at(v, sum, ldcg(Rin + v), __ldg(a.adeg + v));
+          B dr = finish_at(v, sum, rold, ad);
           my_v++;
           my_e += d.y;
-          exp_now = sparse_push(v, dr);
+          exp_now = sparse_push(v, dr, xw);
         }
         exp_now = __shfl_sync(kFull, exp_now, 0);
         if (exp_now) {
@@ -793,7 +810,7 @@ __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const
       }
 
       // sparse: block bin, one block per vertex, taken dynamically
-      for (;;) {
+      while (cnt[2] != 0) {
         if (tid == 0) s_idx = atomicAdd(&ctl->blk_next[it], 1u);
         __syncthreads();
         const uint32_t idx = s_idx;
@@ -826,7 +843,7 @@ __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const
           B dr = finish_at(v, tot, ldcg(Rin + v), __ldg(a.adeg + v));
           my_v++;
           my_e += d.y;
-          s_expand = sparse_push(v, dr);
+          s_expand = sparse_push(v, dr, push_word(v));
         }
         __syncthreads();
         if (s_expand) {
@@ -870,31 +887,42 @@ __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const
     }
     if (tele) block_dead_partial((it + 1) & 1);
     if (!grid_sync(ctl, epoch, &s_err)) return;
+    // what the iteration left, read together: each of these in turn was a round trip to L2
+    uint32_t xi = 0, tl[3] = {0, 0, 0};
+    unsigned long long hub = 0, dR = __ldcg(&ctl->dR_bits[it]);
     if (expand) {
+      xi = ldcg(&ctl->xit[slot]);
+      hub = __ldcg(&ctl->hubq[slot]);
+#pragma unroll
+      for (int bb = 0; bb < 3; bb++) tl[bb] = ldcg(&ctl->tail[slot][bb]);
+    }
+    if (xi) {
       // out-rows of the vertices this iteration's sweep queued, 32 per warp round, one
       // vertex per lane; rows longer than 128 go to the hub queue
-      const uint32_t xend = xdone + ldcg(&ctl->xit[slot]);
-      if (xend > xdone) {
-        for (uint32_t k0 = xdone + gwarp * 32; k0 < xend; k0 += nwarps * 32) {
-          const bool p = k0 + lane < xend;
-          const uint32_t x = p ? ldcg(a.xlist + k0 + lane) : 0u;
-          const ExpandOut o = expand_lanes(a, p ? 1 : 0, x, slot, cnt[0], cnt[1], cnt[2], &wb);
-          my_app += o.app;
-          my_xv += o.xv;
-          my_xe += o.xe;
-        }
-        xdone = xend;
-        flush_marks(a, slot, cnt, lane, wb);
-        if (!grid_sync(ctl, epoch, &s_err)) return;
+      const uint32_t xend = xdone + xi;
+      for (uint32_t k0 = xdone + gwarp * 32; k0 < xend; k0 += nwarps * 32) {
+        const bool p = k0 + lane < xend;
+        const uint32_t x = p ? ldcg(a.xlist + k0 + lane) : 0u;
+        const ExpandOut o = expand_lanes(a, p ? 1 : 0, x, slot, cnt[0], cnt[1], cnt[2], &wb);
+        my_app += o.app;
+        my_xv += o.xv;
+        my_xe += o.xe;
       }
+      xdone = xend;
+      flush_marks(a, slot, cnt, lane, wb);
+      if (!grid_sync(ctl, epoch, &s_err)) return;
+      hub = __ldcg(&ctl->hubq[slot]);
     }
-    if (expand && __ldcg(&ctl->hubq[slot]) != 0) {
+    if (hub) {
       my_app += hub_pass(a, slot, cnt, lane, gwarp, nwarps, wb);
       flush_marks(a, slot, cnt, lane, wb);
       if (!grid_sync(ctl, epoch, &s_err)) return;
     }
+    if (xi || hub) {
+#pragma unroll
+      for (int bb = 0; bb < 3; bb++) tl[bb] = ldcg(&ctl->tail[slot][bb]);
+    }
 
-    unsigned long long dR = __ldcg(&ctl->dR_bits[it]);
     int any_active = 1;
     if (multi) {
       // every block applies the same per-component convergence decisions
@@ -930,7 +958,7 @@ __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const
     }
     if (expand) {
 #pragma unroll
-      for (int bb = 0; bb < 3; bb++) cnt[bb] += ldcg(&ctl->tail[slot][bb]);
+      for (int bb = 0; bb < 3; bb++) cnt[bb] += tl[bb];
     }
     if (tele) {
       double pd = 0.0;
@@ -1047,6 +1075,7 @@ __global__ void __launch_bounds__(kRankBlock, PRDF_RANK_MIN_BLOCKS) k_rank(const
   } while (0)
 
 static constexpr double kOne62 = 4611686018427387904.0;  // 2^62
+static constexpr double kFewMarks = 32768.0;
 
 // Dynamic shared memory of k_rank: per-component max key, base, iteration count, active flag.
 static size_t rank_smem(uint32_t ncomp) { return ((size_t)ncomp * 19 + 15) & ~(size_t)15; }
@@ -1077,6 +1106,10 @@ pr_status rank_setup(Graph *g) {
   CK(g->f32 ? grid_blocks<true>(g->sm_count, smem, &blocks) : grid_blocks<false>(g->sm_count, smem, &blocks));
   g->rank_grid = blocks;
   g->rank_grid_max = blocks;
+  int per_sm = 0;
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &per_sm, g->f32 ? (const void *)k_rank<true, true, 1> : (const void *)k_rank<false, true, 1>, kRankBlock, smem));
+  g->few_grid_max = std::max(1, std::min(per_sm, kFewMarksBlocks)) * g->sm_count;
   CK(cudaMalloc((void **)&g->ctl, sizeof(RankCtl)));
   CK(cudaMallocHost((void **)&g->ctl_h, sizeof(RankCtl)));
   CK(cudaMalloc((void **)&g->dpart, sizeof(DeadPart) * 2 * (size_t)blocks));
@@ -1214,11 +1247,24 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
     CK(launch_full_sweep<F32>(g, a));
     return copy_async_parity();
   }
-  const void *fn = marking ? (a.split && !g->use_graph ? (const void *)k_rank<F32, true, 1> : (const void *)k_rank<F32, true>)
-                           : (const void *)k_rank<F32, false>;
+  // Split calls with few marks: with 2 blocks an SM instead of 4 the kernel spills a third of
+  // the bytes and its barriers wait for half the blocks, and what follows is bound by
+  // latency (sparse iterations of 4200 pairs on a graph of 20 M vertices of degree 2: 24 us
+  // instead of 29, the call 3.87 to 3.63 ms).  Many marks at once want the warps (60,000
+  // sources with 17 M marks: 0.95 ms with 4 blocks, 1.22 with 2).  Few is judged by the marks
+  // expected when the first ones have expanded, sources times the mean degree squared: at 26,000
+  // (the graph above) 2 blocks are ahead, at 48,000 (650 sources, R-MAT, 4.2 M vertices) the
+  // first iteration takes 254 us with 4 and 290 with 2.
+  const bool split = marking && a.split && !g->use_graph;
+  const double degree = (double)g->m / (double)g->n;
+  const bool few = split && (double)g->n_pend_src * degree * degree <= kFewMarks;
+  const void *fn = few      ? (const void *)k_rank<F32, true, 1>
+                   : split   ? (const void *)k_rank<F32, true, 3>
+                   : marking ? (const void *)k_rank<F32, true>
+                             : (const void *)k_rank<F32, false>;
   if (!g->use_graph) {
-    CK(cudaLaunchCooperativeKernel(fn, dim3(g->rank_grid), dim3(kRankBlock), args,
-                                   rank_smem(g->ncomp), g->st));
+    CK(cudaLaunchCooperativeKernel(fn, dim3(few ? std::min(g->rank_grid, g->few_grid_max) : g->rank_grid),
+                                   dim3(kRankBlock), args, rank_smem(g->ncomp), g->st));
     count_launch();
     if (a.split) {
       // the marking launch stops once the affected set is dense (or, for Dynamic

@@ -29,6 +29,7 @@ constexpr uint32_t kInlineOut = 128;  // longer out-rows are marked by the whole
 #ifndef PRDF_RANK_MIN_BLOCKS
 #define PRDF_RANK_MIN_BLOCKS 4  // resident blocks per SM the register budget must allow
 #endif
+constexpr int kFewMarksBlocks = 2;  // ... of the marking launch of split calls with few marks
 
 // Per-mode arithmetic of the kernel.  Rank changes are compared as "delta bits"
 // (non-negative values that order like unsigned integers) and reduced to an L-inf key
@@ -244,37 +245,40 @@ __device__ __forceinline__ uint16_t ldcg(const uint16_t *p) {
   return __ldcg(reinterpret_cast<const unsigned short *>(p));
 }
 
-// Grid-wide barrier with a bounded wait.  Returns false (in every thread of the block)
-// if the device control block holds an error.
+// Arrival at a grid barrier and the bounded wait, by one thread of the block after a block
+// barrier (the release covers the block's writes, the acquire the other blocks').  An error
+// sets kBarErr in the counter itself, so it is known with the count: no load of ctl->err beside
+// every poll and none after the wait (two of the four round trips to L2 of a barrier).
+constexpr uint32_t kBarErr = 0x80000000u;
+__device__ __forceinline__ bool bar_wait(RankCtl *ctl, uint32_t *bar, uint32_t epoch) {
+  red_release_add_u32(bar, 1u);
+  const uint32_t target = epoch * gridDim.x;
+  // the default limit is checked every 128 spins; a short limit set for tests, every spin
+  const unsigned long long lim = *(volatile unsigned long long *)&ctl->bar_limit_ns;
+  const uint32_t every = lim ? 0u : 127u;
+  unsigned long long t0 = 0;
+  uint32_t x;
+  for (uint32_t spins = 1; (x = ld_acquire_u32(bar)) < target; spins++) {
+    if ((spins & every) == 0) {
+      const unsigned long long t = globaltimer_ns();
+      if (t0 == 0) {
+        t0 = t;
+      } else if (t - t0 > (lim ? lim : kBarrierTimeoutNs)) {
+        atomicExch(&ctl->err_where, epoch);
+        atomicOr(&ctl->err, 1u);
+        atomicOr(bar, kBarErr);
+        return false;
+      }
+    }
+  }
+  return x < kBarErr;
+}
+
+// Grid-wide barrier; false in every thread of the block once a wait of this launch ran out.
 __device__ __forceinline__ bool grid_sync(RankCtl *ctl, uint32_t &epoch, uint32_t *s_err) {
   __syncthreads();
   epoch++;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    red_release_add_u32(&ctl->bar, 1u);
-    const uint32_t target = epoch * gridDim.x;
-    uint64_t t0 = 0;
-    uint32_t spins = 0;
-    // the default limit is checked every 128 spins; a short limit set for tests, every spin
-    const unsigned long long lim = *(volatile unsigned long long *)&ctl->bar_limit_ns;
-    const uint32_t every = lim ? 0u : 127u;
-    while (ld_acquire_u32(&ctl->bar) < target) {
-      if (*(volatile uint32_t *)&ctl->err) break;
-      __nanosleep(32);
-      if ((++spins & every) == 0) {
-        uint64_t t = globaltimer_ns();
-        if (t0 == 0) {
-          t0 = t;
-        } else if (t - t0 > (lim ? lim : kBarrierTimeoutNs)) {
-          atomicExch(&ctl->err_where, epoch);
-          atomicOr(&ctl->err, 1u);
-          break;
-        }
-      }
-    }
-    __threadfence();
-    *s_err = *(volatile uint32_t *)&ctl->err;
-  }
+  if (threadIdx.x == 0) *s_err = bar_wait(ctl, &ctl->bar, epoch) ? 0u : 1u;
   __syncthreads();
   return *s_err == 0;
 }
@@ -390,20 +394,42 @@ __device__ __forceinline__ void queue_expansion(const RankArgs<F32> &a, bool pus
   }
 }
 
+// All runs at once: lane b reserves run b's place, so the atomics' round trips overlap.
 template <bool F32>
 __device__ __forceinline__ void flush_marks(const RankArgs<F32> &a, uint32_t slot, const uint32_t cnt[3],
                                             uint32_t lane, WarpBuf &wb) {
+  if ((wb.n[0] | wb.n[1] | wb.n[2] | wb.n[3]) == 0) return;
+  __syncwarp();
+  const uint32_t mine = lane == 0 ? wb.n[0] : lane == 1 ? wb.n[1] : lane == 2 ? wb.n[2] : lane == 3 ? wb.n[3] : 0u;
+  uint32_t base = 0;
+  if (mine) {
+    base = atomicAdd(lane < 3 ? &a.ctl->tail[slot][lane] : &a.ctl->xcnt, mine);
+    if (lane == 3) atomicAdd(&a.ctl->xit[wb.slot], mine);
+  }
+  uint32_t *lists[3] = {a.list0, a.list1, a.list2};
 #pragma unroll
-  for (int bb = 0; bb < 3; bb++) flush_bin(a, bb, slot, cnt, lane, wb);
-  flush_expansions(a, lane, wb);
+  for (int bb = 0; bb < 4; bb++) {
+    const uint32_t k = wb.n[bb];
+    if (k == 0) continue;
+    const uint32_t b0 = __shfl_sync(kFull, base, bb);
+    uint32_t *to = bb < 3 ? lists[bb] + cnt[bb] + b0 : a.xlist + b0;
+    for (uint32_t i = lane; i < k; i += 32) to[i] = wb.buf[bb * kMarkBuf + i];
+    if (bb < 3 && wb.items) append_items(a, wb.buf + bb * kMarkBuf, k, lane);
+    wb.n[bb] = 0;
+  }
+  __syncwarp();
 }
 
-// Appends w where fresh to its bin's run in the warp's buffer.  Called by a whole warp.
+// The bin of a newly marked vertex.
 template <bool F32>
-__device__ __forceinline__ void append_mark(const RankArgs<F32> &a, bool fresh, uint32_t w, uint32_t slot,
+__device__ __forceinline__ int mark_bin(const RankArgs<F32> &a, uint32_t w, const WarpBuf &wb) {
+  return wb.dense ? 0 : bin_of(__ldg(&a.in_rd[w]).y, a.bin_lo, a.bin_hi);
+}
+
+// Appends w to its bin's run in the warp's buffer (bin < 0: nothing).  Called by a whole warp.
+template <bool F32>
+__device__ __forceinline__ void append_mark(const RankArgs<F32> &a, int bin, uint32_t w, uint32_t slot,
                                             const uint32_t cnt[3], uint32_t lane, WarpBuf &wb) {
-  int bin = -1;
-  if (fresh) bin = wb.dense ? 0 : bin_of(__ldg(&a.in_rd[w]).y, a.bin_lo, a.bin_hi);
   const int nb = wb.dense ? 1 : 3;
   for (int bb = 0; bb < nb; bb++) {
     const uint32_t mask = __ballot_sync(kFull, bin == bb);
@@ -415,41 +441,57 @@ __device__ __forceinline__ void append_mark(const RankArgs<F32> &a, bool fresh, 
   }
 }
 
-// Marks w (where valid) for iteration `slot`: a plain read of the bitmap first, then the
-// atomic; a newly marked vertex is stamped and appended through the warp's buffer.  Called
-// by a whole warp; returns 1 where this lane marked a new vertex.
-template <bool F32>
-__device__ __forceinline__ uint32_t mark_one(const RankArgs<F32> &a, bool valid, uint32_t w, uint32_t slot,
-                                             const uint32_t cnt[3], uint32_t lane, WarpBuf &wb) {
-  bool fresh = false;
-  if (valid) {
-    uint32_t bit = 1u << (w & 31);
-    uint32_t *word = a.bitmap + (w >> 5);
-    if (!(ldcg(word) & bit)) {
-      uint32_t old = atomicOr(word, bit);
-      if (!(old & bit)) {
-        fresh = true;
-        a.stamp[w] = (uint16_t)slot;
-      }
+// Marks w[0 .. K) of every lane (where ok has its bit) for iteration `slot`: a plain read of
+// the bitmap first, then the atomic for a clear bit; a newly marked vertex is stamped and
+// appended through the warp's buffer.  Each step is a dependent round trip, so the K entries
+// take it together (the marks of 60,000 sources with 17 M out-edges by 2 blocks an SM: 1.47 ms
+// one entry at a time, 1.22 four).  Called by a whole warp; returns how many this lane marked.
+template <bool F32, int K>
+__device__ __forceinline__ uint32_t mark_entries(const RankArgs<F32> &a, const uint32_t (&w)[K], uint32_t ok,
+                                                 uint32_t slot, const uint32_t cnt[3], uint32_t lane, WarpBuf &wb) {
+  uint32_t word[K];
+#pragma unroll
+  for (int k = 0; k < K; k++) word[k] = (ok >> k) & 1u ? ldcg(a.bitmap + (w[k] >> 5)) : ~0u;
+  uint32_t fresh = 0;  // bit k: entry k newly marked by this lane
+#pragma unroll
+  for (int k = 0; k < K; k++) {
+    const uint32_t bit = 1u << (w[k] & 31);
+    if (!(word[k] & bit) && !(atomicOr(a.bitmap + (w[k] >> 5), bit) & bit)) fresh |= 1u << k;
+  }
+  if (!__any_sync(kFull, fresh)) return 0;
+  int bin[K];
+#pragma unroll
+  for (int k = 0; k < K; k++) {
+    bin[k] = -1;
+    if ((fresh >> k) & 1u) {
+      a.stamp[w[k]] = (uint16_t)slot;
+      bin[k] = mark_bin(a, w[k], wb);
     }
   }
-  append_mark(a, fresh, w, slot, cnt, lane, wb);
-  return fresh ? 1u : 0u;
+#pragma unroll
+  for (int k = 0; k < K; k++)
+    if (__any_sync(kFull, bin[k] >= 0)) append_mark(a, bin[k], w[k], slot, cnt, lane, wb);
+  return __popc(fresh);
 }
 
-// Marks cols[first + 32 k + lane] (k = 0, 1, ...; stride `stride`), stamping newly marked
-// vertices with `slot` (the iteration they join).  Called by a whole warp.
+// Marks cols[first + stride k + lane] (k = 0, 1, ...), stamping newly marked vertices with
+// `slot` (the iteration they join); four entries a lane at a time.  Called by a whole warp.
 template <bool F32>
 __device__ __forceinline__ uint32_t warp_mark_range(const RankArgs<F32> &a, const uint32_t *cols, uint32_t len,
                                                     uint32_t first, uint32_t stride, uint32_t slot,
                                                     const uint32_t cnt[3], uint32_t lane, WarpBuf &wb) {
-  uint32_t newly_total = 0;
-  for (uint32_t j0 = first; j0 < len; j0 += stride) {
-    const uint32_t j = j0 + lane;
-    const bool valid = j < len;
-    newly_total += mark_one(a, valid, valid ? __ldg(cols + j) : 0u, slot, cnt, lane, wb);
+  uint32_t newly = 0;
+  for (uint32_t j0 = first; j0 < len; j0 += 4 * stride) {
+    uint32_t w[4], ok = 0;
+#pragma unroll
+    for (uint32_t k = 0; k < 4; k++) {
+      const uint32_t j = j0 + k * stride + lane;
+      w[k] = j < len ? __ldg(cols + j) : 0u;
+      ok |= j < len ? 1u << k : 0u;
+    }
+    newly += mark_entries<F32, 4>(a, w, ok, slot, cnt, lane, wb);
   }
-  return newly_total;
+  return newly;
 }
 
 // Short out-rows (at most kThreadOut entries; a row starts 16-byte aligned and its slots
@@ -462,43 +504,16 @@ template <bool F32>
 __device__ __forceinline__ uint32_t lane_mark_rows(const RankArgs<F32> &a, bool mine, uint2 od, uint32_t slot,
                                                    const uint32_t cnt[3], uint32_t lane, WarpBuf &wb) {
   const uint32_t len = mine ? od.y : 0u;
-  const uint32_t rounds = __reduce_max_sync(kFull, len);
   uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0;
   if (len > 0) q0 = __ldg(reinterpret_cast<const uint4 *>(a.out_col + od.x));
   if (len > 4) q1 = __ldg(reinterpret_cast<const uint4 *>(a.out_col + od.x + 4));
   const uint32_t w[kThreadOut] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
-  uint32_t word[kThreadOut];
-#pragma unroll
-  for (uint32_t k = 0; k < kThreadOut; k++) word[k] = k < len ? ldcg(a.bitmap + (w[k] >> 5)) : ~0u;
-  uint32_t fresh = 0;  // bit k: entry k newly marked by this lane
-#pragma unroll
-  for (uint32_t k = 0; k < kThreadOut; k++) {
-    const uint32_t bit = 1u << (w[k] & 31);
-    if (!(word[k] & bit) && !(atomicOr(a.bitmap + (w[k] >> 5), bit) & bit)) fresh |= 1u << k;
-  }
-  uint32_t newly = 0;
-#pragma unroll
-  for (uint32_t k = 0; k < kThreadOut; k++) {
-    if (k < rounds) {
-      const bool f = (fresh >> k) & 1u;
-      if (f) a.stamp[w[k]] = (uint16_t)slot;
-      append_mark(a, f, w[k], slot, cnt, lane, wb);
-      newly += f ? 1u : 0u;
-    }
-  }
-  return newly;
+  return mark_entries<F32, kThreadOut>(a, w, (1u << len) - 1u, slot, cnt, lane, wb);
 }
 
-// True the first time v asks (per call): its out-row is then scanned by the caller.  A
-// plain read first, so a vertex that keeps changing costs one load per iteration, not an
-// atomic.
-__device__ __forceinline__ bool first_expansion(uint32_t *xbits, uint32_t v) {
-  uint32_t bit = 1u << (v & 31);
-  if (__ldcg(xbits + (v >> 5)) & bit) return false;
-  return !(atomicOr(xbits + (v >> 5), bit) & bit);
-}
-// The same with the word read beforehand (issued with the row's loads, so the test adds no
-// round trip); the atomic still decides, so a stale word only costs an atomic.
+// True the first time v asks (per call): its out-row is then scanned by the caller.  `word`
+// is v's word of the bits, read beforehand (with the row's loads, so the test adds no round
+// trip); the atomic decides, so a stale word only costs an atomic.
 __device__ __forceinline__ bool first_expansion_pre(uint32_t *xbits, uint32_t v, uint32_t word) {
   uint32_t bit = 1u << (v & 31);
   if (word & bit) return false;
@@ -653,8 +668,7 @@ __device__ __noinline__ ExpandOut expand_lanes(const RankArgs<F32> &a, int push,
   const uint32_t total = __shfl_sync(kFull, incl, 31);
   const uint32_t excl = incl - mlen;
   for (uint32_t e0 = 0; e0 < total; e0 += 128) {
-    uint32_t w[4], word[4];
-    bool valid[4];
+    uint32_t w[4], ok = 0;
 #pragma unroll
     for (int k = 0; k < 4; k++) {
       const uint32_t e = e0 + 32u * k + lane;
@@ -667,24 +681,10 @@ __device__ __noinline__ ExpandOut expand_lanes(const RankArgs<F32> &a, int push,
       }
       const uint32_t base = __shfl_sync(kFull, od.x, owner & 31u);
       const uint32_t first = __shfl_sync(kFull, excl, owner & 31u);
-      valid[k] = e < total;
-      w[k] = valid[k] ? __ldg(a.out_col + base + (e - first)) : 0u;
+      w[k] = e < total ? __ldg(a.out_col + base + (e - first)) : 0u;
+      ok |= e < total ? 1u << k : 0u;
     }
-#pragma unroll
-    for (int k = 0; k < 4; k++) word[k] = valid[k] ? ldcg(a.bitmap + (w[k] >> 5)) : ~0u;
-    uint32_t fresh = 0;
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-      const uint32_t bit = 1u << (w[k] & 31);
-      if (!(word[k] & bit) && !(atomicOr(a.bitmap + (w[k] >> 5), bit) & bit)) fresh |= 1u << k;
-    }
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-      const bool f = (fresh >> k) & 1u;
-      if (f) a.stamp[w[k]] = (uint16_t)slot;
-      append_mark(a, f, w[k], slot, cnt, lane, wb);
-      o.app += f ? 1u : 0u;
-    }
+    o.app += mark_entries<F32, 4>(a, w, ok, slot, cnt, lane, wb);
   }
   if (mine || med) {
     o.xv++;

@@ -644,6 +644,7 @@ __device__ __forceinline__ void block_max(typename Num<F32>::B my_max, unsigned 
 __device__ __forceinline__ bool hot_landed(RankCtl *ctl, uint32_t bar, uint32_t parity) {
   if (__all_sync(kFull, mbar_wait(bar, parity, kStageTimeoutNs))) return true;  // the same in the whole warp
   atomicOr(&ctl->err, 2u);
+  atomicOr(&ctl->lbar, kBarErr);  // a run's barriers end too
   mbar_wait(bar, parity, kStageTimeoutNs);
   return false;
 }
@@ -656,27 +657,9 @@ __device__ __forceinline__ bool run_barrier(RankCtl *ctl, uint32_t &epoch, uint3
   epoch++;
   if (threadIdx.x == 0) {
     asm volatile("fence.proxy.async;" ::: "memory");  // the next hot copies read what was written
-    __threadfence();
-    red_release_add_u32(&ctl->lbar, 1u);
-    const uint32_t target = epoch * gridDim.x;
-    const unsigned long long lim = *(volatile unsigned long long *)&ctl->bar_limit_ns;
-    const uint32_t every = lim ? 0u : 127u;
-    unsigned long long t0 = 0;
-    for (uint32_t spins = 1; ld_acquire_u32(&ctl->lbar) < target; spins++) {
-      if (*(volatile uint32_t *)&ctl->err) break;
-      if ((spins & every) == 0) {
-        const unsigned long long t = globaltimer_ns();
-        if (t0 == 0) {
-          t0 = t;
-        } else if (t - t0 > (lim ? lim : kBarrierTimeoutNs)) {
-          atomicExch(&ctl->err_where, epoch);
-          atomicOr(&ctl->err, 1u);
-          break;
-        }
-      }
-    }
-    *s_err = *(volatile uint32_t *)&ctl->err;
+    const bool ok = bar_wait(ctl, &ctl->lbar, epoch);
     read();
+    *s_err = ok ? 0u : 1u;
   }
   __syncthreads();
   return *s_err == 0;
