@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_batch(const BatchArgs<F32> p
       a.C0[v] = c;
       a.C1[v] = c;
     }
-    if (!run_barrier(ctl, epoch, &s_err, [] {})) return;
+    if (!run_barrier(ctl, epoch, &s_err)) return;
   }
   if (gtid == 0 && !p.marking) ctl->t_ns[1] = globaltimer_ns();
 
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_batch(const BatchArgs<F32> p
         pull_long(it);
         __syncthreads();
       });
-      if (!run_barrier(ctl, epoch, &s_err, [] {})) return;
+      if (!run_barrier(ctl, epoch, &s_err)) return;
     }
     pre_pulled = false;
     const C *Cin = it & 1 ? a.C1 : a.C0;
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_batch(const BatchArgs<F32> p
       joined = 0;
       if (lane == 0 && j) atomicAdd(&ctl->jtotal, j);
     }
-    if (!run_barrier(ctl, epoch, &s_err, [] {})) return;
+    if (!run_barrier(ctl, epoch, &s_err)) return;
     if (!live) break;  // only the last marks were left
     // every block takes the same decisions
     int changed = 0;

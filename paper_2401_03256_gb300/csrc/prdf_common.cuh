@@ -42,6 +42,16 @@ __device__ __forceinline__ void red_release_add_u32(uint32_t *p, uint32_t v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void red_release_add_u64(unsigned long long *p, unsigned long long v) {
+  asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
 __device__ __forceinline__ uint64_t globaltimer_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -147,7 +157,8 @@ struct RankCtl {
   uint32_t xneed[kMaxIterLimit + 2];                  // continuation: a recorded expansion would mark
   // per-iteration sweep launches (sweep.cu): what one launch leaves for the next
   uint32_t ticket;        // blocks of the current sweep launch that have finished
-  uint32_t lbar;          // grid barrier arrivals of the current run of iterations (k_loop)
+  uint32_t lbar;          // grid barrier arrivals of the current run of iterations (k_batch)
+  unsigned long long tally[2];  // the same of k_loop, with what the iteration left (sweep_dev.cuh)
   uint32_t it_cur;        // iteration the next sweep launch computes
   uint32_t sw_all[3];     // sweep items per tier (all vertices)
   uint32_t sw_off[2];     // first item of tiers 1 and 2 (in the item and compacted arrays)

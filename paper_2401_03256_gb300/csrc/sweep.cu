@@ -56,7 +56,7 @@ __device__ void sweep_decide(const SweepArgs<F32> &a, uint32_t it_first, uint32_
   ctl->it_cur = iters;
   ctl->ticket = 0;
   ctl->bar = 0;  // a prologue's grid barriers count from zero, and so do a run's
-  ctl->lbar = 0;
+  ctl->tally[0] = ctl->tally[1] = 0;
   ctl->launches += 1;
   uint32_t total = 0;
   for (int b = 0; b < 3; b++) {  // only the first iteration of a run has marks of its own
@@ -259,9 +259,9 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_loop(const LoopArgs<F32> p) 
   using S = Store<F32>;
   using R = typename S::R;
   using C = typename S::C;
-  __shared__ unsigned long long s_key[kSweepWarps], s_dR;
+  __shared__ unsigned long long s_key[kSweepWarps];
   __shared__ __align__(8) unsigned long long s_bar;
-  __shared__ uint32_t s_x, s_err;
+  __shared__ uint32_t s_left, s_err;
   __shared__ Rounds s_rounds;
   extern __shared__ __align__(128) unsigned char s_hot[];
   const SweepArgs<F32> &a = p.a;
@@ -274,13 +274,7 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_loop(const LoopArgs<F32> p) 
   io.sbase = smem_addr(s_hot);
   io.r = &s_rounds;
   uint32_t it = 0, epoch = 0;
-  // Thread 0 also reads what the iteration left (slot k): its L-inf change and first expansions.
-  auto barrier = [&](uint32_t k) -> bool {
-    return run_barrier(ctl, epoch, &s_err, [&] {
-      s_dR = __ldcg(&ctl->dR_bits[k]);
-      s_x = CMP ? __ldcg(&ctl->xit[k]) : 0u;
-    });
-  };
+  unsigned long long seen[2] = {0, 0};
   // an error ends the device-side loop: nothing else would
   auto give_up = [&]() {
     if (CMP && tid == 0) {
@@ -306,7 +300,7 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_loop(const LoopArgs<F32> p) 
         a.C0[v] = c;
         a.C1[v] = c;
       }
-      if (!barrier(0)) return;
+      if (!run_tally(ctl, epoch, &s_err, &s_left, false, false, seen)) return;
     }
     if (gtid == 0) {
       ctl->t_ns[1] = globaltimer_ns();
@@ -315,14 +309,19 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_loop(const LoopArgs<F32> p) 
     if (a.max_iter <= 0) return;
   }
   const uint32_t it_first = it;
+  __syncthreads();  // the rounds are set, the block's mbarrier initialised
   for (;; it++) {
-    __syncthreads();  // the rounds are set, the block's mbarrier initialised
     if (bytes && tid == 0) stage_hot(it & 1 ? a.C1 : a.C0, bytes, io.sbase, bar);
     io.it = it;
     if (!bytes || hot_landed(ctl, bar, (it - it_first) & 1u)) sweep_pass<F32, CMP ? 2 : 0>(a, io);
-    block_max<F32>(io.my_max, &ctl->dR_bits[it], s_key);  // (a block barrier: every warp has taken its last round)
-    if (tid < 3) s_rounds.next[tid] = 0;
-    if (!barrier(it)) {
+    // (a block barrier: every warp has taken its last round)
+    const unsigned long long key = block_max<F32>(io.my_max, &ctl->dR_bits[it], s_key);
+    bool grew = false;
+    if (tid == 0) {
+      grew = CMP && s_rounds.grew;
+      s_rounds.next[0] = s_rounds.next[1] = s_rounds.next[2] = s_rounds.grew = 0;
+    }
+    if (!run_tally(ctl, epoch, &s_err, &s_left, key > a.tol_key, grew, seen)) {
       give_up();
       return;
     }
@@ -333,7 +332,7 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_loop(const LoopArgs<F32> p) 
         ctl->it_kind[it] = 3;
       }
     }
-    if (s_dR <= a.tol_key || (int)it + 1 >= a.max_iter || s_x) break;
+    if (s_left != 1u || (int)it + 1 >= a.max_iter) break;  // (nothing above the tolerance, or first expansions)
   }
   if constexpr (CMP) {
     if (tid == 0) {
@@ -357,8 +356,9 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_loop(const LoopArgs<F32> p) 
     }
     if (gtid == 0) {
       ctl->iterations = k;
-      ctl->converged = s_dR <= a.tol_key ? 1u : 0u;
-      ctl->last_key = s_dR;
+      const unsigned long long dR = __ldcg(&ctl->dR_bits[it]);
+      ctl->converged = dR <= a.tol_key ? 1u : 0u;
+      ctl->last_key = dR;
       ctl->vproc += (unsigned long long)k * a.n;
       ctl->eproc += (unsigned long long)k * p.m;
     }
@@ -463,7 +463,7 @@ __global__ void k_dense_init(const DenseInit p) {
   ctl->it_cur = it0;
   ctl->ticket = 0;
   ctl->bar = 0;
-  ctl->lbar = 0;
+  ctl->tally[0] = ctl->tally[1] = 0;
   for (int t = 0; t < 3; t++) {
     ctl->sw_all[t] = p.sw_all[t];
     ctl->dcnt[t] = ctl->save_cnt[t];
