@@ -79,7 +79,7 @@ struct Graph {
   DeadPart *dpart = nullptr;         // [2][rank_grid]
   int rank_grid = 0;                 // cooperative grid of the rank kernel
   int rank_grid_max = 0;             // most blocks that can be co-resident
-  int few_grid_max = 0;              // the same of a split call's marking launch with few marks
+  int few_grid_max = 0;              // the same of a split call's marking launch with few marks (0: not used)
   // CUDA-graph launch of rank calls (pr_set_graph_launch): captured once, kernel arguments
   // updated in place before every replay
   bool use_graph = false;

@@ -1257,7 +1257,7 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
   // first iteration takes 254 us with 4 and 290 with 2.
   const bool split = marking && a.split && !g->use_graph;
   const double degree = (double)g->m / (double)g->n;
-  const bool few = split && (double)g->n_pend_src * degree * degree <= kFewMarks;
+  const bool few = split && g->few_grid_max && (double)g->n_pend_src * degree * degree <= kFewMarks;
   const void *fn = few      ? (const void *)k_rank<F32, true, 1>
                    : split   ? (const void *)k_rank<F32, true, 3>
                    : marking ? (const void *)k_rank<F32, true>
