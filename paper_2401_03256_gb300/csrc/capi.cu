@@ -375,8 +375,7 @@ static pr_status create_impl(uint32_t n, int64_t m, const uint32_t *src, const u
       int best = -1;
       for (int k = 0; k < 2 && rc == PR_OK; k++) {
         if ((p.vertex_order >= 2 && p.vertex_order - 2 != k) || (comp_n && k == 1)) continue;
-        e = cudaMalloc((void **)&cp[k], 4ull * n);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&ci[k], 4ull * n);
+        e = prdf::alloc_pieces({prdf::piece(&cp[k], n), prdf::piece(&ci[k], n)});
         if (e != cudaSuccess) { rc = prdf::cuda_fail(&g0, e, "vertex numbering"); break; }
         rc = prdf::vertex_order(&g0, kinds[k], cp[k], ci[k], comp_n);
         if (rc == PR_OK && p.vertex_order == 0) rc = prdf::order_cost(&g0, cp[k], ci[k], cost[k]);
@@ -388,8 +387,7 @@ static pr_status create_impl(uint32_t n, int64_t m, const uint32_t *src, const u
       if (keep && !g.teleport) {
         std::vector<uint32_t> hot;
         if (g.f32) {
-          e = cudaMalloc((void **)&g.lab, 4ull * n);
-          if (e == cudaSuccess) e = cudaMalloc((void **)&g.at, 4ull * n);
+          e = prdf::alloc_pieces({prdf::piece(&g.lab, n), prdf::piece(&g.at, n)});
           if (e != cudaSuccess) rc = prdf::cuda_fail(&g0, e, "vertex numbering");
         }
         if (rc == PR_OK)
@@ -401,7 +399,6 @@ static pr_status create_impl(uint32_t n, int64_t m, const uint32_t *src, const u
           else g.hot = hot[0] & ~3u;
         } else {
           cudaFree(g.lab);
-          cudaFree(g.at);
           g.lab = g.at = nullptr;
         }
       }
@@ -411,7 +408,6 @@ static pr_status create_impl(uint32_t n, int64_t m, const uint32_t *src, const u
           g.inv = ci[k];
         } else {
           cudaFree(cp[k]);
-          cudaFree(ci[k]);
         }
       }
       // no room for the numbering's transient build: the caller's numbering (vertex_order 0)
@@ -420,13 +416,7 @@ static pr_status create_impl(uint32_t n, int64_t m, const uint32_t *src, const u
       prdf::graph_free(&g0);
       if (fallback) rc = PR_OK;
       if (rc != PR_OK) break;
-      if (keep) {
-        prdf::map_ids(g.inv, tmp, 2ull * (uint64_t)m, g.st);
-        g.perm_h.resize(n);
-        e = cudaMemcpyAsync(g.perm_h.data(), g.perm, 4ull * n, cudaMemcpyDeviceToHost, g.st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(g.st);
-        if (e != cudaSuccess) { rc = prdf::cuda_fail(&g, e, "vertex numbering"); break; }
-      }
+      if (keep) prdf::map_ids(g.inv, tmp, 2ull * (uint64_t)m, g.st);
     }
     // a small graph's contributions are copied whole, in any numbering
     if (!comp_n && !g.teleport && n <= prdf::hot_limit(g.f32)) g.hot = n & ~3u;
@@ -641,15 +631,18 @@ pr_status pr_get_affected(pr_graph *h, uint32_t *out, int64_t cap, int64_t *coun
     int64_t c = g.last_list_cnt[b];
     int64_t take = std::max<int64_t>(0, std::min<int64_t>(c, cap - total));
     if (take > 0) {
-      cudaError_t e = cudaMemcpyAsync(out + total, g.list[b], 4ull * take, cudaMemcpyDeviceToHost, g.st);
+      const uint32_t *ids = g.list[b];
+      if (g.perm) {  // back to the caller's numbering (the three lists hold at most n ids)
+        prdf::gather_ids(g.perm, ids, g.gen_tmp + total, (uint64_t)take, g.st);
+        ids = g.gen_tmp + total;
+      }
+      cudaError_t e = cudaMemcpyAsync(out + total, ids, 4ull * take, cudaMemcpyDeviceToHost, g.st);
       if (e != cudaSuccess) return prdf::cuda_fail(&g, e, "get affected");
     }
     total += c;
   }
   cudaError_t e = cudaStreamSynchronize(g.st);
   if (e != cudaSuccess) return prdf::cuda_fail(&g, e, "get affected");
-  if (!g.perm_h.empty())  // back to the caller's numbering
-    for (int64_t i = 0; i < std::min<int64_t>(total, cap); i++) out[i] = g.perm_h[out[i]];
   *count = total;
   return PR_OK;
 }

@@ -29,6 +29,24 @@ static cudaError_t dalloc(T **p, uint64_t count) {
   return cudaMalloc((void **)p, sizeof(T) * (count ? count : 1));
 }
 
+cudaError_t alloc_pieces(std::initializer_list<Piece> pieces) {
+  auto room = [](uint64_t bytes) { return (bytes + 255) & ~255ull; };  // 256-byte aligned, as cudaMalloc's
+  uint64_t total = 0;
+  for (const Piece &x : pieces) {
+    *x.p = nullptr;
+    total += room(x.bytes);
+  }
+  if (alloc_fault()) return cudaErrorMemoryAllocation;
+  char *base = nullptr;
+  const cudaError_t e = cudaMalloc((void **)&base, total);
+  if (e != cudaSuccess) return e;
+  for (const Piece &x : pieces) {
+    *x.p = base;
+    base += room(x.bytes);
+  }
+  return cudaSuccess;
+}
+
 static inline unsigned grid_for(uint64_t n, int threads = 256) {
   uint64_t g = (n + threads - 1) / threads;
   return (unsigned)std::max<uint64_t>(1, g);
@@ -287,8 +305,7 @@ static pr_status build_adj(Graph *g, const uint64_t *keys, uint64_t m, Adj &A, u
                            uint32_t *scan_tmp, const uint32_t *at) {
   const uint32_t n = g->n;
   cudaStream_t st = g->st;
-  CK(dalloc(&A.rd, n));
-  CK(dalloc(&A.cap, n));
+  CK(alloc_pieces({piece(&A.rd, n), piece(&A.cap, n)}));
   k_row_bounds<<<grid_for(m + 1), 256, 0, st>>>(keys, m, g->b, n, off); count_launch();
   k_row_caps<<<grid_for(n), 256, 0, st>>>(off, n, A.cap); count_launch();
   exclusive_scan_u32(A.cap, tmp, n, scan_tmp, st);
@@ -346,18 +363,12 @@ pr_status graph_build(Graph *g, uint64_t m_in, const uint32_t *src_d, const uint
   const uint64_t mk1 = std::max<uint64_t>(mk, 1);
   const uint64_t big = std::max<uint64_t>(mk1 + 1, (uint64_t)n + 1);
   pr_status rc = PR_OK;
-  auto cleanup = [&]() {
-    cudaFree(keys); cudaFree(alt); cudaFree(flags); cudaFree(pos); cudaFree(hist); cudaFree(stmp); cudaFree(cnt);
-  };
-  cudaError_t e = cudaSuccess;
-  if ((e = dalloc(&keys, mk1)) != cudaSuccess || (e = dalloc(&alt, mk1)) != cudaSuccess ||
-      (e = dalloc(&flags, big)) != cudaSuccess || (e = dalloc(&pos, big)) != cudaSuccess ||
-      (e = dalloc(&hist, std::max(radix_hist_words(mk1), scan_tmp_words(big)) + 1)) != cudaSuccess ||
-      (e = dalloc(&stmp, scan_tmp_words(std::max<uint64_t>(big, radix_hist_words(mk1))) + 1)) != cudaSuccess ||
-      (e = dalloc(&cnt, 1)) != cudaSuccess) {
-    cleanup();
-    return cuda_fail(g, e, "graph build scratch");
-  }
+  auto cleanup = [&]() { cudaFree(keys); };
+  cudaError_t e = alloc_pieces(
+      {piece(&keys, mk1), piece(&alt, mk1), piece(&flags, big), piece(&pos, big),
+       piece(&hist, std::max(radix_hist_words(mk1), scan_tmp_words(big)) + 1),
+       piece(&stmp, scan_tmp_words(std::max<uint64_t>(big, radix_hist_words(mk1))) + 1), piece(&cnt, 1)});
+  if (e != cudaSuccess) return cuda_fail(g, e, "graph build scratch");
   do {
     if (mk) {
     k_make_keys<<<grid_for(mk), 256, 0, st>>>(src_d, dst_d, m_in, n, g->b, sl ? 1 : 0, keys);
@@ -393,38 +404,37 @@ pr_status graph_build(Graph *g, uint64_t m_in, const uint32_t *src_d, const uint
   if (e != cudaSuccess) return cuda_fail(g, e, "graph build");
   if (rc != PR_OK) return rc;
 
-  // what the vertex numbering needs of a transient build
-  CK(dalloc(&g->gen_tmp, (uint64_t)n + 8));  // also the sweep-item rebuild's 4 ceil(n / 4096) + 2 tile counts
-  CK(dalloc(&g->gen_tmp2, (uint64_t)n + 8));
-  CK(dalloc(&g->scan_tmp, scan_tmp_words((uint64_t)n + 8) + 1));
-  CK(dalloc(&g->actl, 1));
-  if (g->transient) return PR_OK;
-  // rank state
-  const size_t es = g->f32 ? 4 : 8;
-  for (int i = 0; i < 2; i++) {
-    CK(cudaMalloc(&g->R[i], es * n));
-    CK(cudaMalloc(&g->C[i], es * n));
+  // scratch (gen_tmp also holds the sweep-item rebuild's 4 ceil(n / 4096) + 2 tile counts): all
+  // that the vertex numbering needs of a transient build
+  const uint64_t scan_words = scan_tmp_words((uint64_t)n + 8) + 1;
+  if (g->transient) {
+    CK(alloc_pieces({piece(&g->gen_tmp, (uint64_t)n + 8), piece(&g->gen_tmp2, (uint64_t)n + 8),
+                     piece(&g->scan_tmp, scan_words), piece(&g->actl, 1)}));
+    return PR_OK;
   }
-  CK(cudaMalloc(&g->adeg, es * n));
+  // ... and the rank state
+  const uint64_t rank_bytes = (uint64_t)(g->f32 ? 4 : 8) * n;
   const uint32_t words = (n + 31) / 32;
-  CK(dalloc(&g->bitmap, words));
-  CK(cudaMemsetAsync(g->bitmap, 0, 4ull * words, st));
-  CK(dalloc(&g->xbits, words));
-  CK(cudaMemsetAsync(g->xbits, 0, 4ull * words, st));
-  CK(dalloc(&g->stamp, n));
-  CK(cudaMemsetAsync(g->stamp, 0xFF, 2ull * n, st));
-  CK(dalloc(&g->chunk_done, n));
-  CK(cudaMemsetAsync(g->chunk_done, 0, 4ull * n, st));
-  CK(dalloc(&g->item_pos, n));
-  CK(dalloc(&g->hub_v, n));
-  CK(dalloc(&g->hub_base, n));
-  for (int i = 0; i < 3; i++) CK(dalloc(&g->list[i], n));
-  CK(dalloc(&g->xlist, n));
-  CK(dalloc(&g->dead, n));
   g->pend_cap = std::max<uint32_t>(1u << 16, std::min<uint32_t>(n, 1u << 22));
-  CK(dalloc(&g->pend_src, g->pend_cap));
-  CK(dalloc(&g->pend_tgt, g->pend_cap));
-  CK(cudaMallocHost((void **)&g->actl_h, sizeof(ApplyCtl)));
+  CK(alloc_pieces({piece(&g->gen_tmp, (uint64_t)n + 8), piece(&g->gen_tmp2, (uint64_t)n + 8),
+                   piece(&g->scan_tmp, scan_words), piece(&g->actl, 1), piece(&g->ctl, 1),
+                   piece(&g->dpart, 2ull * kRankBlocksPerSm * g->sm_count),
+                   Piece{&g->R[0], rank_bytes}, Piece{&g->R[1], rank_bytes}, Piece{&g->C[0], rank_bytes},
+                   Piece{&g->C[1], rank_bytes}, Piece{&g->adeg, rank_bytes}, piece(&g->bitmap, words),
+                   piece(&g->xbits, words), piece(&g->stamp, n), piece(&g->emap, 2ull * n), piece(&g->chunk_done, n),
+                   piece(&g->item_pos, n), piece(&g->hub_v, n), piece(&g->hub_base, n), piece(&g->list[0], n),
+                   piece(&g->list[1], n), piece(&g->list[2], n), piece(&g->xlist, n), piece(&g->dead, n),
+                   piece(&g->pend_src, g->pend_cap), piece(&g->pend_tgt, g->pend_cap)}));
+  CK(cudaMemsetAsync(g->bitmap, 0, 4ull * words, st));
+  CK(cudaMemsetAsync(g->xbits, 0, 4ull * words, st));
+  CK(cudaMemsetAsync(g->stamp, 0xFF, 2ull * n, st));
+  CK(cudaMemsetAsync(g->emap, 0, 2ull * n, st));
+  CK(cudaMemsetAsync(g->chunk_done, 0, 4ull * n, st));
+  char *host = nullptr;
+  const size_t actl_room = (sizeof(ApplyCtl) + 255) & ~(size_t)255;
+  CK(cudaMallocHost((void **)&host, actl_room + sizeof(RankCtl)));
+  g->actl_h = (ApplyCtl *)host;
+  g->ctl_h = (RankCtl *)(host + actl_room);
   if (g->f32) {
     using S = Store<true>;
     k_init_rank<true><<<grid_for(n), 256, 0, st>>>(g->out.rd, n, g->p.alpha, (S::A *)g->adeg, (S::R *)g->R[0],
@@ -448,29 +458,18 @@ pr_status apply_scratch(Graph *g, uint64_t N) {
   uint64_t cap = std::max<uint64_t>(N, 4096);
   uint32_t *boff = s.boff;
   const int32_t boff_cap = s.boff_cap;
-  cudaFree(s.pairs); cudaFree(s.kd); cudaFree(s.vals); cudaFree(s.vals2); cudaFree(s.tmp); cudaFree(s.tmp2);
-  cudaFree(s.chg); cudaFree(s.chg_t); cudaFree(s.flags); cudaFree(s.pos); cudaFree(s.seg);
-  cudaFree(s.tagpref); cudaFree(s.radix_hist); cudaFree(s.scan_tmp);
+  cudaFree(s.pairs);
   s = ApplyScratch{};
   s.boff = boff;
   s.boff_cap = boff_cap;
-  CK(dalloc(&s.pairs, 2 * cap));
-  CK(dalloc(&s.kd, cap));
-  CK(dalloc(&s.vals, cap));
-  CK(dalloc(&s.vals2, cap));
-  CK(dalloc(&s.tmp, cap));
-  CK(dalloc(&s.tmp2, cap));
-  CK(dalloc(&s.chg, cap));
-  CK(dalloc(&s.chg_t, cap));
-  CK(dalloc(&s.flags, cap + 2));
-  CK(dalloc(&s.pos, cap + 2));
-  CK(dalloc(&s.seg, 2 * (cap + 2)));
-  CK(dalloc(&s.tagpref, 2 * (cap + 2)));
   // (the plan of an update in one launch keeps 256 + 8 words a block there)
   s.radix_hist_cap = std::max<uint64_t>(radix_hist_words(cap) + 256, 264ull * g->sm_count);
-  CK(dalloc(&s.radix_hist, s.radix_hist_cap));
   s.scan_tmp_cap = scan_tmp_words(std::max<uint64_t>(cap + 2, s.radix_hist_cap)) + 1;
-  CK(dalloc(&s.scan_tmp, s.scan_tmp_cap));
+  CK(alloc_pieces({piece(&s.pairs, 2 * cap), piece(&s.kd, cap), piece(&s.vals, cap), piece(&s.vals2, cap),
+                   piece(&s.tmp, cap), piece(&s.tmp2, cap), piece(&s.chg, cap), piece(&s.chg_t, cap),
+                   piece(&s.flags, cap + 2), piece(&s.pos, cap + 2), piece(&s.seg, 2 * (cap + 2)),
+                   piece(&s.tagpref, 2 * (cap + 2)), piece(&s.radix_hist, s.radix_hist_cap),
+                   piece(&s.scan_tmp, s.scan_tmp_cap)}));
   s.cap = cap;
   return PR_OK;
 }
@@ -529,8 +528,9 @@ pr_status graph_export(Graph *g, int dir, uint64_t *offs_h, uint32_t *cols_h) {
     return PR_OK;
   }
   // rows and columns back in the caller's numbering, each row sorted
-  const std::vector<uint32_t> &perm = g->perm_h;
-  std::vector<uint32_t> inv(n);
+  std::vector<uint32_t> perm(n), inv(n);
+  CK(cudaMemcpyAsync(perm.data(), g->perm, 4ull * n, cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
   for (uint32_t r = 0; r < n; r++) inv[perm[r]] = r;
   uint64_t at = 0;
   for (uint32_t v = 0; v < n; v++) {
@@ -568,16 +568,12 @@ pr_status graph_refresh_ident(Graph *g) {
   const uint32_t c01 = h[1], total = h[2] - n;
   if ((uint64_t)c01 + total > g->items_cap || total > g->chunk_cap) {  // items, and partials by chunk number
     cudaFree(g->items);
-    cudaFree(g->items_cmp);
-    cudaFree(g->partials);
     g->items = g->items_cmp = nullptr;
     g->partials = nullptr;
     g->items_cap = g->chunk_cap = 0;
     uint64_t chunks = (uint64_t)total + total / 4 + 1024;
     uint64_t cap = (uint64_t)n + chunks;
-    CK(dalloc(&g->items, cap));
-    CK(dalloc(&g->items_cmp, cap));
-    CK(cudaMalloc(&g->partials, 8 * chunks));
+    CK(alloc_pieces({piece(&g->items, cap), piece(&g->items_cmp, cap), Piece{&g->partials, 8 * chunks}}));
     g->items_cap = cap;
     g->chunk_cap = chunks;
   }
@@ -717,24 +713,15 @@ pr_status components_setup(Graph *g, const std::vector<uint32_t> &comp_n) {
 
 void graph_free(Graph *g) {
   Adj *adjs[2] = {&g->out, &g->in};
+  // (what alloc_pieces gave is owned by the first array of each group)
   for (Adj *A : adjs) {
     cudaFree(A->rd);
-    cudaFree(A->cap);
     cudaFree(A->col);
   }
-  for (int i = 0; i < 2; i++) {
-    cudaFree(g->R[i]);
-    cudaFree(g->C[i]);
-  }
-  cudaFree(g->adeg);
-  cudaFree(g->bitmap);
-  cudaFree(g->xbits);
-  cudaFree(g->stamp);
+  cudaFree(g->gen_tmp);
   cudaFree(g->items);
-  cudaFree(g->items_cmp);
-  cudaFree(g->item_pos);
-  cudaFree(g->hub_v);
-  cudaFree(g->hub_base);
+  cudaFree(g->sc.pairs);
+  cudaFree(g->sc.boff);
   cudaFree(g->comp);
   cudaFree(g->comp_base);
   cudaFree(g->comp_init);
@@ -745,32 +732,11 @@ void graph_free(Graph *g) {
   cudaFree(g->comp_item);
   cudaFree(g->comp_out);
   cudaFree(g->comp_last);
-  cudaFree(g->partials);
-  cudaFree(g->chunk_done);
-  for (int i = 0; i < 3; i++) cudaFree(g->list[i]);
-  cudaFree(g->xlist);
-  cudaFree(g->dead);
-  cudaFree(g->pend_src);
-  cudaFree(g->pend_tgt);
-  cudaFree(g->ctl);
-  if (g->ctl_h) cudaFreeHost(g->ctl_h);
-  cudaFree(g->dpart);
-  ApplyScratch &s = g->sc;
-  cudaFree(s.pairs); cudaFree(s.kd); cudaFree(s.vals); cudaFree(s.vals2); cudaFree(s.tmp); cudaFree(s.tmp2);
-  cudaFree(s.boff);
-  cudaFree(s.chg); cudaFree(s.chg_t); cudaFree(s.flags); cudaFree(s.pos); cudaFree(s.seg);
-  cudaFree(s.tagpref); cudaFree(s.radix_hist); cudaFree(s.scan_tmp);
-  cudaFree(g->actl);
   if (g->actl_h) cudaFreeHost(g->actl_h);
   cudaFree(g->big);
   cudaFree(g->longs);
-  cudaFree(g->gen_tmp);
-  cudaFree(g->gen_tmp2);
   cudaFree(g->perm);
-  cudaFree(g->inv);
   cudaFree(g->lab);
-  cudaFree(g->at);
-  cudaFree(g->scan_tmp);
   if (g->cg_exec) cudaGraphExecDestroy(g->cg_exec);
   if (g->cg) cudaGraphDestroy(g->cg);
   if (g->ev0) cudaEventDestroy(g->ev0);

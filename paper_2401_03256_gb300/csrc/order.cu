@@ -520,6 +520,17 @@ pr_status hot_order(Graph *g, const std::vector<uint32_t> &comp_n, uint32_t hot_
   return PR_OK;
 }
 
+__global__ void k_gather_ids(const uint32_t *perm, const uint32_t *ids, uint32_t *out, uint64_t k) {
+  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < k) out[i] = perm[ids[i]];
+}
+
+void gather_ids(const uint32_t *perm, const uint32_t *ids, uint32_t *out, uint64_t k, cudaStream_t st) {
+  if (k == 0) return;
+  k_gather_ids<<<grid_of(k), 256, 0, st>>>(perm, ids, out, k);
+  count_launch();
+}
+
 void map_ids(const uint32_t *inv, uint32_t *a, uint64_t m, cudaStream_t st) {
   if (m == 0) return;
   k_map_ids<<<grid_of(m), 256, 0, st>>>(inv, a, m);

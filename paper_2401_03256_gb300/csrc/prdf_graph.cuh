@@ -1,6 +1,7 @@
 // prdf_graph.cuh - the graph handle behind the opaque pr_graph of the C ABI.
 #pragma once
 
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -19,6 +20,20 @@ __host__ __device__ inline uint32_t move_cap(uint32_t len) {
   uint64_t c = 2ull * len + 2;
   return (uint32_t)((c + 3) & ~3ull);
 }
+
+// Arrays that live and die together come from one allocation, which the first of them owns:
+// each cudaMalloc and cudaFree takes 30 to 40 us beside the pages it maps.  A handle's creation and
+// destruction made 78 pairs of them; with about 20, a snapshot (create, Static, read, destroy)
+// of a graph of 1 M vertices and 16 M edges takes 15.3 ms instead of 18.7.
+struct Piece {
+  void **p;
+  uint64_t bytes;
+};
+template <class T>
+Piece piece(T **p, uint64_t count) { return Piece{(void **)p, sizeof(T) * (count ? count : 1)}; }
+cudaError_t alloc_pieces(std::initializer_list<Piece> pieces);
+
+constexpr int kRankBlocksPerSm = 4;  // most blocks of the rank kernel on an SM
 
 struct Graph {
   int device = 0;
@@ -45,7 +60,6 @@ struct Graph {
   // internal numbering (single-graph handles): perm[internal] = caller's id, inv the inverse;
   // null when the handle keeps the caller's numbering
   uint32_t *perm = nullptr, *inv = nullptr;
-  std::vector<uint32_t> perm_h;
   uint32_t hot = 0;                  // vertices of largest out-degree numbered first (multiple of 4; order.cu)
   // FP32 handles with hot vertices: in-rows are ordered by the numbering without the hot part
   // (lab[v] = v's place in it, at[place] = v), so that float sums are added in its order
@@ -155,6 +169,7 @@ pr_status order_cost(Graph *g, const uint32_t *perm, const uint32_t *inv, uint64
 pr_status hot_order(Graph *g, const std::vector<uint32_t> &comp_n, uint32_t hot_max, uint32_t *perm, uint32_t *inv,
                     std::vector<uint32_t> &hot, uint32_t *lab, uint32_t *at);
 uint32_t hot_limit(bool f32);  // sweep.cu: contributions a block's shared-memory copy holds (less a few)
+void gather_ids(const uint32_t *perm, const uint32_t *ids, uint32_t *out, uint64_t k, cudaStream_t st);  // out[i] = perm[ids[i]]
 void map_ids(const uint32_t *inv, uint32_t *a, uint64_t m, cudaStream_t st);
 pr_status graph_export(Graph *g, int dir, uint64_t *offs_h, uint32_t *cols_h);
 pr_status graph_refresh_ident(Graph *g);

@@ -1089,7 +1089,7 @@ static cudaError_t grid_blocks(int sm_count, size_t smem, int *blocks) {
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_df, k_rank<F32, true>, kRankBlock, smem);
   if (e != cudaSuccess) return e;
   per_sm = std::min(per_sm, per_sm_df);
-  per_sm = std::max(1, std::min(per_sm, 4));
+  per_sm = std::max(1, std::min(per_sm, kRankBlocksPerSm));
   *blocks = per_sm * sm_count;
   return cudaSuccess;
 }
@@ -1110,9 +1110,6 @@ pr_status rank_setup(Graph *g) {
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
       &per_sm, g->f32 ? (const void *)k_rank<true, true, 1> : (const void *)k_rank<false, true, 1>, kRankBlock, smem));
   g->few_grid_max = std::max(1, std::min(per_sm, kFewMarksBlocks)) * g->sm_count;
-  CK(cudaMalloc((void **)&g->ctl, sizeof(RankCtl)));
-  CK(cudaMallocHost((void **)&g->ctl_h, sizeof(RankCtl)));
-  CK(cudaMalloc((void **)&g->dpart, sizeof(DeadPart) * 2 * (size_t)blocks));
   CK(cudaEventCreate(&g->ev0));
   CK(cudaEventCreate(&g->ev1));
   pr_status rc = sweep_setup(g);

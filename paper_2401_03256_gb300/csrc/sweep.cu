@@ -1033,10 +1033,6 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
 uint32_t hot_limit(bool f32) { return kHotBytes / (f32 ? 4 : 8) - 8; }
 
 pr_status sweep_setup(Graph *g) {
-  if (!g->emap) {
-    CKG(cudaMalloc((void **)&g->emap, 2ull * g->n));
-    CKG(cudaMemsetAsync(g->emap, 0, 2ull * g->n, g->st));
-  }
   const void *fns[4] = {g->f32 ? (const void *)k_loop<true, false> : (const void *)k_loop<false, false>,
                         g->f32 ? (const void *)k_loop<true, true> : (const void *)k_loop<false, true>,
                         g->f32 ? (const void *)k_sweep<true, 1> : (const void *)k_sweep<false, 1>,
@@ -1079,8 +1075,6 @@ void sweep_free(Graph *g) {
     delete L;
     g->loops = nullptr;
   }
-  cudaFree(g->emap);
-  g->emap = nullptr;
 }
 
 }  // namespace prdf
