@@ -282,6 +282,7 @@ __device__ __noinline__ DtOut dt_search(const RankArgs<F32> &a, uint32_t epoch, 
   const uint32_t nthreads = gridDim.x * kRankBlock;
   const uint32_t gtid = blockIdx.x * kRankBlock + tid;
   const uint32_t nwarps = nthreads >> 5, gwarp = gtid >> 5;
+  const uint32_t swarp = (tid >> 5) * gridDim.x + blockIdx.x;
   RankCtl *ctl = a.ctl;
   DtOut o{{c0, c1, c2}, 0u, 0u, 0u, epoch, false, false};
   WarpBuf wb = *wbp;
@@ -292,8 +293,9 @@ __device__ __noinline__ DtOut dt_search(const RankArgs<F32> &a, uint32_t epoch, 
   for (; r <= (uint32_t)kMaxIterLimit; r++) {
 #pragma unroll
     for (int bb = 0; bb < 3; bb++) {
-      for (uint32_t k0 = done[bb] + gwarp * 32; k0 < o.cnt[bb]; k0 += nwarps * 32) {
-        const bool p = k0 + lane < o.cnt[bb];
+      const uint32_t per = warp_share(o.cnt[bb] - done[bb], nwarps);
+      for (uint32_t k0 = done[bb] + swarp * per; k0 < o.cnt[bb]; k0 += nwarps * per) {
+        const bool p = lane < per && k0 + lane < o.cnt[bb];
         const uint32_t x = p ? ldcg(lists[bb] + k0 + lane) : 0u;
         const ExpandOut e = expand_lanes(a, p ? 1 : 0, x, r, o.cnt[0], o.cnt[1], o.cnt[2], &wb);
         o.app += e.app;
@@ -355,6 +357,7 @@ __global__ void __launch_bounds__(kRankBlock, SPLIT == 1 ? kFewMarksBlocks : PRD
   const uint32_t nthreads = nblk * kRankBlock;
   const uint32_t gtid = blockIdx.x * kRankBlock + tid;
   const uint32_t nwarps = nthreads >> 5, gwarp = gtid >> 5;
+  const uint32_t swarp = wib * nblk + blockIdx.x;  // neighbours on different SMs
   RankCtl *ctl = a.ctl;
   uint32_t epoch = 0;
   constexpr bool df = DF;
@@ -480,10 +483,11 @@ __global__ void __launch_bounds__(kRankBlock, SPLIT == 1 ? kFewMarksBlocks : PRD
   // the sweeps append to the list once the first barrier is passed
   uint32_t xdone = 0;
   if (df && !a.start_full) {
-    // sources: mark G^t.out(u), 32 sources per warp round (short rows by their own lanes,
+    // sources: mark G^t.out(u), up to 32 sources per warp round (short rows by their own lanes,
     // medium rows flattened over the warp, long rows by the whole grid)
-    for (uint32_t k0 = gwarp * 32; k0 < a.n_pend_src; k0 += nwarps * 32) {
-      const bool p = k0 + lane < a.n_pend_src;
+    const uint32_t per = warp_share(a.n_pend_src, nwarps);
+    for (uint32_t k0 = swarp * per; k0 < a.n_pend_src; k0 += nwarps * per) {
+      const bool p = lane < per && k0 + lane < a.n_pend_src;
       const uint32_t u = p ? __ldg(a.pend_src + k0 + lane) : 0u;
       const ExpandOut o = expand_lanes(a, p ? 1 : 0, u, 0u, 0u, 0u, 0u, &wb);
       my_app += o.app;
@@ -750,11 +754,12 @@ __global__ void __launch_bounds__(kRankBlock, SPLIT == 1 ? kFewMarksBlocks : PRD
       my_app += io.my_app;
     } else {
       // sparse: thread bin, one thread per vertex, 32 consecutive list entries per warp
-      for (uint32_t b0 = gwarp * 32; b0 < cnt[0]; b0 += nwarps * 32) {
+      const uint32_t per = warp_share(cnt[0], nwarps);
+      for (uint32_t b0 = swarp * per; b0 < cnt[0]; b0 += nwarps * per) {
         const uint32_t i = b0 + lane;
         int push = 0;
         uint32_t v = 0;
-        bool mine = i < cnt[0];
+        bool mine = lane < per && i < cnt[0];
         if (mine) {
           v = ldcg(a.list0 + i);
           mine = live(v);
@@ -900,8 +905,9 @@ __global__ void __launch_bounds__(kRankBlock, SPLIT == 1 ? kFewMarksBlocks : PRD
       // out-rows of the vertices this iteration's sweep queued, 32 per warp round, one
       // vertex per lane; rows longer than 128 go to the hub queue
       const uint32_t xend = xdone + xi;
-      for (uint32_t k0 = xdone + gwarp * 32; k0 < xend; k0 += nwarps * 32) {
-        const bool p = k0 + lane < xend;
+      const uint32_t per = warp_share(xi, nwarps);
+      for (uint32_t k0 = xdone + swarp * per; k0 < xend; k0 += nwarps * per) {
+        const bool p = lane < per && k0 + lane < xend;
         const uint32_t x = p ? ldcg(a.xlist + k0 + lane) : 0u;
         const ExpandOut o = expand_lanes(a, p ? 1 : 0, x, slot, cnt[0], cnt[1], cnt[2], &wb);
         my_app += o.app;

@@ -563,8 +563,9 @@ __global__ void __launch_bounds__(kRankBlock, 2) k_df_push(const RankArgs<F32> a
   if (pn) {
     const uint32_t lo = ldcg_u32(&ctl->push_lo);
     WarpBuf wb{s_mbuf[wib], {0u, 0u, 0u, 0u}, false, it, items && !compact};
-    for (uint32_t k0 = gwarp * 32; k0 < pn; k0 += nwarps * 32) {
-      const bool p = k0 + lane < pn;
+    const uint32_t per = warp_share(pn, nwarps);
+    for (uint32_t k0 = (wib * gridDim.x + blockIdx.x) * per; k0 < pn; k0 += nwarps * per) {
+      const bool p = lane < per && k0 + lane < pn;
       const uint32_t x = p ? ldcg_u32(a.xlist + lo + k0 + lane) : 0u;
       const ExpandOut o = expand_lanes(a, p ? 1 : 0, x, it, cnt[0], cnt[1], cnt[2], &wb);
       app += o.app;
@@ -677,7 +678,7 @@ __global__ void __launch_bounds__(kRankBlock, 2) k_df_push_light(const RankArgs<
   __shared__ uint32_t s_mbuf[kWarps][4 * kMarkBuf];
   RankCtl *ctl = a.ctl;
   const uint32_t tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
-  const uint32_t nwarps = (gridDim.x * kRankBlock) >> 5, gwarp = (blockIdx.x * kRankBlock + tid) >> 5;
+  const uint32_t nwarps = (gridDim.x * kRankBlock) >> 5;
   const uint32_t it = ldcg_u32(&ctl->it_cur);
   if (blockIdx.x == 0 && tid == 0) atomicAdd(&ctl->launches, 1u);
   uint32_t cnt[3];
@@ -686,8 +687,9 @@ __global__ void __launch_bounds__(kRankBlock, 2) k_df_push_light(const RankArgs<
   const uint32_t pn = ldcg_u32(&ctl->push_n), lo = ldcg_u32(&ctl->push_lo);
   WarpBuf wb{s_mbuf[wib], {0u, 0u, 0u, 0u}, false, it, true};
   unsigned long long app = 0, xv = 0, xe = 0;
-  for (uint32_t k0 = gwarp * 32; k0 < pn; k0 += nwarps * 32) {
-    const bool p = k0 + lane < pn;
+  const uint32_t per = warp_share(pn, nwarps);
+  for (uint32_t k0 = (wib * gridDim.x + blockIdx.x) * per; k0 < pn; k0 += nwarps * per) {
+    const bool p = lane < per && k0 + lane < pn;
     const uint32_t x = p ? ldcg_u32(a.xlist + lo + k0 + lane) : 0u;
     const ExpandOut o = expand_lanes(a, p ? 1 : 0, x, it, cnt[0], cnt[1], cnt[2], &wb);
     app += o.app;
