@@ -795,16 +795,15 @@ def run_ours(args, rank: int, world: int, local_rank: int):
     all_bytes = static_bytes + sum(sum(rec[f]["naive_bytes"]) + sum(rec[f]["df_bytes"]) for f in FRACS)
     all_ms = static_ms + sum(sum(rec[f]["naive"]) + sum(rec[f]["df"]) for f in FRACS)
     peak, peak_kind = hbm_peak()
-    # the Static call is one k_full_init, one full-sweep k_sweep launch per iteration and one
-    # writeback, timed by CUDA events on its stream: the time per iteration bounds a sweep
-    # launch's duration from above (it includes the init and writeback and the loop's node
-    # switches), so `achieved` is a lower bound
+    # the Static call is one k_loop launch that runs all iterations and writes the ranks back,
+    # timed by CUDA events on its stream: the time per iteration bounds a sweep's duration from
+    # above (it includes the start from 1/n and the writeback), so `achieved` is a lower bound
     static_iters = sum(sum(rec[f]["static_iters"]) for f in FRACS)
     launch_bytes = static_bytes / static_iters
     launch_ms = static_ms / static_iters
     achieved = launch_bytes / (launch_ms * 1e-3) / 1e9
     traffic = None
-    tr_path = os.path.join(ROOT, "profiles", "k_sweep_traffic.json")
+    tr_path = os.path.join(ROOT, "profiles", "k_loop_traffic.json")
     try:
         with open(tr_path) as f:
             tr = json.load(f)
@@ -879,7 +878,7 @@ def run_ours(args, rank: int, world: int, local_rank: int):
         "gpu_launches": launches,
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
-                     "kernel": "k_sweep<64-bit, full sweep> (one launch per Static iteration)",
+                     "kernel": "k_loop<64-bit, every vertex> (all Static iterations in one launch; figures per iteration)",
                      "launch_bytes_algorithmic": launch_bytes, "launch_ms": launch_ms,
                      "all_rank_calls_gbs": all_bytes / (all_ms * 1e-3) / 1e9},
         "per_frac": per_f,

@@ -1254,7 +1254,7 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
   // the bytes and its barriers wait for half the blocks, and what follows is bound by
   // latency (sparse iterations of 4200 pairs on a graph of 20 M vertices of degree 2: 24 us
   // instead of 29, the call 3.87 to 3.63 ms).  Many marks at once want the warps (60,000
-  // sources with 17 M marks: 0.95 ms with 4 blocks, 1.22 with 2).  Few is judged by the marks
+  // sources with 17 M marks: 0.95 ms with 4 blocks, 1.22 with 2).  Few is told by the marks
   // expected when the first ones have expanded, sources times the mean degree squared: at 26,000
   // (the graph above) 2 blocks are ahead, at 48,000 (650 sources, R-MAT, 4.2 M vertices) the
   // first iteration takes 254 us with 4 and 290 with 2.
