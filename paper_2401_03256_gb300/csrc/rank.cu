@@ -895,7 +895,7 @@ __global__ void __launch_bounds__(kRankBlock, SPLIT == 1 ? kFewMarksBlocks : PRD
     // what the iteration left, read together: each of these in turn was a round trip to L2
     uint32_t xi = 0, tl[3] = {0, 0, 0};
     unsigned long long hub = 0, dR = __ldcg(&ctl->dR_bits[it]);
-    if (expand) {
+    if (expand && !defer) {  // (a deferring iteration pushes none, and its pulls add to tail[slot] meanwhile)
       xi = ldcg(&ctl->xit[slot]);
       hub = __ldcg(&ctl->hubq[slot]);
 #pragma unroll
