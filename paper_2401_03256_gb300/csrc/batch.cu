@@ -326,6 +326,10 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_batch(const BatchArgs<F32> p
     live = __syncthreads_or(tid < nc && s_state[tid] == kLive) != 0;
   }
 
+  // A call without iterations (max_iter 0) has passed no barrier: no block may write its status
+  // before every block has read the marking launch's
+  if (epoch == 0 && !run_barrier(ctl, epoch, &s_err)) return;
+
   // both parities take a graph's final values, which are in parity (its iterations) & 1; the
   // affected vertices are listed (list 0) and counted per graph, their per-call marks cleared
   auto copy_final = [&](uint32_t v, uint32_t c) {
