@@ -830,7 +830,8 @@ cudaError_t add_conditional(cudaGraphNode_t *node, cudaGraph_t graph, const cuda
   return e;
 }
 
-size_t hot_bytes(const Graph *g) { return (size_t)g->hot * (g->f32 ? 4 : 8); }
+template <bool F32>
+size_t hot_bytes(const SweepArgs<F32> &a) { return (size_t)a.hot * sizeof(typename Store<F32>::C); }
 
 template <bool F32>
 pr_status full_impl(Graph *g, bool from_init) {
@@ -845,7 +846,7 @@ pr_status full_impl(Graph *g, bool from_init) {
   else p.init = std::llrint(1.0 / (double)g->n * 4611686018427387904.0);
   void *args[] = {(void *)&p};
   CKG(cudaLaunchCooperativeKernel((const void *)k_loop<F32, false>, dim3(g->loop_grid), dim3(kSweepBlock), args,
-                                  hot_bytes(g), g->st));
+                                  hot_bytes(p.a), g->st));
   count_launch();
   return PR_OK;
 }
@@ -888,7 +889,7 @@ pr_status full_steps_impl(Graph *g, bool from_init) {
     CKG(add_conditional(&wnode, lg.graph, &lg.init, 1, lg.h_loop, cudaGraphCondTypeWhile, &body));
     void *sargs[] = {(void *)&a};
     CKG(add_kernel(&snode, body, nullptr, 0, (const void *)k_sweep<F32, 0>, dim3(g->sm_count), dim3(kSweepBlock), sargs,
-                   false, hot_bytes(g)));
+                   false, hot_bytes(a)));
     typename S::R *R0 = ip.R0, *R1 = ip.R1;
     typename S::C *C0 = ip.C0, *C1 = ip.C1;
     uint32_t n = g->n;
@@ -989,10 +990,10 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
     la.a = a;
     void *largs[] = {(void *)&la};
     CKG(add_kernel(&s0, sw[0], nullptr, 0, (const void *)k_loop<F32, true>, dim3(g->loop_grid), dim3(kSweepBlock), largs,
-                   true, hot_bytes(g)));
+                   true, hot_bytes(a)));
     void *sargs[] = {(void *)&a};
     CKG(add_kernel(&s1, sw[1], nullptr, 0, (const void *)k_sweep<F32, 1>, dim3(g->sm_count),
-                   dim3(kSweepBlock), sargs, false, hot_bytes(g)));
+                   dim3(kSweepBlock), sargs, false, hot_bytes(a)));
     void *iargs[] = {(void *)&ip};
     CKG(add_kernel(&lg.init, lg.graph, nullptr, 0, (const void *)k_dense_init, dim3(1), dim3(32), iargs, false));
     cudaGraphEdgeData ed{};

@@ -720,7 +720,9 @@ __device__ __forceinline__ bool run_tally(RankCtl *ctl, uint32_t &epoch, uint32_
   return *s_err == 0;
 }
 
-// Host side: a handle's sweep arguments (async: both parities aliased).
+// Host side: a handle's sweep arguments (async: both parities aliased, and no copy in shared
+// memory: contributions are written while the others' copies of them would still be read, and
+// a copy taken at the start of an iteration would hide what the iteration has updated since).
 template <bool F32>
 SweepArgs<F32> sweep_args(const Graph *g, bool async) {
   using S = Store<F32>;
@@ -744,7 +746,7 @@ SweepArgs<F32> sweep_args(const Graph *g, bool async) {
   a.emap = g->emap;
   a.out_rd = g->out.rd;
   a.ctl = g->ctl;
-  a.hot = g->hot;
+  a.hot = async ? 0u : g->hot;
   const double n = (double)g->n;
   if constexpr (F32) {
     a.base = (float)((1.0 - g->p.alpha) / n);
