@@ -416,13 +416,15 @@ pr_status graph_build(Graph *g, uint64_t m_in, const uint32_t *src_d, const uint
   const uint64_t rank_bytes = (uint64_t)(g->f32 ? 4 : 8) * n;
   const uint32_t words = (n + 31) / 32;
   g->pend_cap = std::max<uint32_t>(1u << 16, std::min<uint32_t>(n, 1u << 22));
+  // (a vertex is queued once per iteration, but initially once for every update of its row)
+  const uint32_t hubs = std::max(n, g->pend_cap);
   CK(alloc_pieces({piece(&g->gen_tmp, (uint64_t)n + 8), piece(&g->gen_tmp2, (uint64_t)n + 8),
                    piece(&g->scan_tmp, scan_words), piece(&g->actl, 1), piece(&g->ctl, 1),
                    piece(&g->dpart, 2ull * kRankBlocksPerSm * g->sm_count),
                    Piece{&g->R[0], rank_bytes}, Piece{&g->R[1], rank_bytes}, Piece{&g->C[0], rank_bytes},
                    Piece{&g->C[1], rank_bytes}, Piece{&g->adeg, rank_bytes}, piece(&g->bitmap, words),
                    piece(&g->xbits, words), piece(&g->stamp, n), piece(&g->emap, 2ull * n), piece(&g->chunk_done, n),
-                   piece(&g->item_pos, n), piece(&g->hub_v, n), piece(&g->hub_base, n), piece(&g->list[0], n),
+                   piece(&g->item_pos, n), piece(&g->hub_v, hubs), piece(&g->hub_base, hubs), piece(&g->list[0], n),
                    piece(&g->list[1], n), piece(&g->list[2], n), piece(&g->xlist, n), piece(&g->dead, n),
                    piece(&g->pend_src, g->pend_cap), piece(&g->pend_tgt, g->pend_cap)}));
   CK(cudaMemsetAsync(g->bitmap, 0, 4ull * words, st));
