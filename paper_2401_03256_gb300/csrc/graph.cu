@@ -476,7 +476,8 @@ pr_status apply_scratch(Graph *g, uint64_t N) {
   return PR_OK;
 }
 
-// Rebuilds adjacency A with fresh slack and at least `reserve` free tail words.
+// Rebuilds adjacency A with fresh slack and at least `reserve` free tail words.  The sweep items
+// hold the in-rows' starts, so they are rebuilt before the next sweep.
 pr_status repack_adj(Graph *g, Adj &A, uint64_t reserve) {
   const uint32_t n = g->n;
   cudaStream_t st = g->st;
@@ -504,6 +505,7 @@ pr_status repack_adj(Graph *g, Adj &A, uint64_t reserve) {
   A.col_cap = total + reserve;
   A.used = total;
   A.garbage = 0;
+  if (&A == &g->in) g->ident_dirty = true;
   return PR_OK;
 }
 

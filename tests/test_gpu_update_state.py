@@ -53,3 +53,32 @@ def test_a_row_updated_more_often_than_there_are_vertices(prdf, degree, call):
         getattr(h, call)()
         ref = oracle.static_pr(H)[0]
         assert np.abs(h.ranks() - ref).max() <= 2e-9  # both stop at a change of 1e-10: 2 tau / (1 - alpha)
+
+
+@pytest.mark.parametrize("f32", [False, True])
+def test_rows_repacked_without_a_change_of_tier(prdf, f32):
+    # in-rows of 21 entries (28 slots) grow to 31 (64 slots), 200 an update: the second one finds
+    # 1200 of 70,000 words left, so all rows are laid out anew, most of them elsewhere, and none
+    # changes its tier; the sweeps must follow
+    n = 2000
+    v = np.arange(n)
+    src = _u((np.repeat(v, 20) + np.tile(np.arange(1, 21), n)) % n)
+    dst = _u(np.repeat(v, 20))
+    G = oracle.Graph.build(n, src, dst)
+    p = prdf.pr_params_default()
+    p.vertex_order = 1
+    p.precision = prdf.PR_F32 if f32 else prdf.PR_F64
+    none = _u([])
+    with prdf.Graph(n, src, dst, p) as h:
+        h.static()
+        for lo in (0, 1000, 200, 1200):
+            rows = np.repeat(np.arange(lo, lo + 200), 10)
+            up = (none, none, _u((rows + 100 + 37 * np.tile(np.arange(10), 200)) % n), _u(rows))
+            h.apply(*up)
+            G = G.apply(*up)[0]
+            _check(h, G)
+            ref = oracle.static_pr(G)[0]
+            for call in ("frontier", "static"):
+                getattr(h, call)()
+                # a change of 1e-10 stops both: 2 tau / (1 - alpha) apart at most; FP32: its rounding
+                assert np.abs(h.ranks() - ref).max() <= (1e-6 if f32 else 2e-9)
