@@ -481,11 +481,13 @@ pr_status apply_scratch(Graph *g, uint64_t N) {
 pr_status repack_adj(Graph *g, Adj &A, uint64_t reserve) {
   const uint32_t n = g->n;
   cudaStream_t st = g->st;
-  k_len_caps<<<grid_for(n), 256, 0, st>>>(A.rd, n, A.cap); count_launch();
-  exclusive_scan_u32(A.cap, g->gen_tmp, n, g->scan_tmp, st);
+  // (the rows' own capacities change only once there is room: a failure leaves them as they are)
+  uint32_t *caps = g->gen_tmp2;
+  k_len_caps<<<grid_for(n), 256, 0, st>>>(A.rd, n, caps); count_launch();
+  exclusive_scan_u32(caps, g->gen_tmp, n, g->scan_tmp, st);
   uint32_t last[2];
   CK(cudaMemcpyAsync(&last[0], g->gen_tmp + (n - 1), 4, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(&last[1], A.cap + (n - 1), 4, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(&last[1], caps + (n - 1), 4, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   uint64_t total = (uint64_t)last[0] + last[1];
   reserve = std::max<uint64_t>(reserve, std::max<uint64_t>(total / 4, 1024));
@@ -496,7 +498,12 @@ pr_status repack_adj(Graph *g, Adj &A, uint64_t reserve) {
   }
   uint32_t *nc = nullptr;
   CK(dalloc(&nc, total + reserve));
-  CK(cudaMemsetAsync(nc, 0xFF, sizeof(uint32_t) * (total + reserve), st));
+  cudaError_t e = cudaMemsetAsync(nc, 0xFF, sizeof(uint32_t) * (total + reserve), st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(A.cap, caps, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st);
+  if (e != cudaSuccess) {
+    cudaFree(nc);
+    return cuda_fail(g, e, "repack");
+  }
   k_repack_rows<<<grid_for((uint64_t)n * 32), 256, 0, st>>>(A.rd, n, A.col, nc, g->gen_tmp); count_launch();
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));

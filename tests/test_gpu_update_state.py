@@ -82,3 +82,43 @@ def test_rows_repacked_without_a_change_of_tier(prdf, f32):
                 getattr(h, call)()
                 # a change of 1e-10 stops both: 2 tau / (1 - alpha) apart at most; FP32: its rounding
                 assert np.abs(h.ranks() - ref).max() <= (1e-6 if f32 else 2e-9)
+
+
+def _ring(n, k):
+    v = np.arange(n)
+    return _u((np.repeat(v, k) + np.tile(np.arange(1, k + 1), n)) % n), _u(np.repeat(v, k))
+
+
+def _more(lo, rows, k, at):
+    """k new in-edges for each of the rows from lo on, from vertices at, at + 37, ... further."""
+    r = np.repeat(np.arange(lo, lo + rows), k)
+    none = _u([])
+    return none, none, _u((r + at + 37 * np.tile(np.arange(k), rows)) % 2000), _u(r)
+
+
+def test_a_repack_without_room_leaves_the_rows_their_slots(prdf):
+    # rows 400 to 409 fill their 28 slots; the update after the next needs a repack, whose allocation
+    # fails; then the full rows must move, not grow over their neighbours
+    src, dst = _ring(2000, 20)
+    G = oracle.Graph.build(2000, src, dst)
+    p = prdf.pr_params_default()
+    p.vertex_order = 1
+    with prdf.Graph(2000, src, dst, p) as h:
+        for up in (_more(400, 10, 7, 500), _more(0, 200, 10, 100)):
+            h.apply(*up)
+            G = G.apply(*up)[0]
+        big = _more(1000, 200, 10, 100)
+        prdf.pr_inject_alloc_failure(0)
+        try:
+            with pytest.raises(prdf.PrdfError) as e:
+                h.apply(*big)
+        finally:
+            prdf.pr_inject_alloc_failure(-1)
+        assert e.value.status == prdf.PR_ERR_OUT_OF_MEMORY
+        _check(h, G)
+        for up in (_more(400, 10, 1, 900), big, _more(400, 10, 9, 1100)):
+            h.apply(*up)
+            G = G.apply(*up)[0]
+            _check(h, G)
+        h.static()
+        assert np.abs(h.ranks() - oracle.static_pr(G)[0]).max() <= 2e-9
