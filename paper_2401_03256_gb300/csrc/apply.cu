@@ -554,7 +554,8 @@ struct MergeArgs {
   typename S::C *C0, *C1;
   uint32_t *pend_src, *pend_tgt;
   uint32_t pend_cap, n_src, n_tgt;
-  // in-rows: sweep items (patched where tier and chunk count stay), the rows' order
+  // in-rows: sweep items (patched where tier and chunk count stay; null: rebuilt in any case,
+  // out of date since a repack, or an earlier call found no room for them), the rows' order
   uint32_t bin_lo, gmax, chunk;
   uint4 *items;
   const uint32_t *item_pos;
@@ -600,7 +601,7 @@ __device__ __forceinline__ void finish_row(const MergeArgs<F32> &p, uint32_t dir
   }
   // free slots of the row's last 16 bytes (the sweeps read rows by 16 bytes)
   for (uint32_t k = new_len + t; k < ((new_len + 3) & ~3u); k += nt) A.col[dest + k] = kNoCol;
-  if (dir == 1) {
+  if (dir == 1 && p.items) {
     const int tier = sweep_tier(new_len, p.bin_lo, p.gmax);
     const uint32_t nch = (new_len + p.chunk - 1) / p.chunk;
     if (sweep_tier(len, p.bin_lo, p.gmax) != tier || (tier == 2 && (len + p.chunk - 1) / p.chunk != nch)) {
@@ -842,7 +843,7 @@ static pr_status run_merge(Graph *g, const MergeAdj &out, const MergeAdj &in, ui
   p.bin_lo = (uint32_t)g->p.bin_lo;
   p.gmax = g->group_max;
   p.chunk = g->chunk_len;
-  p.items = g->items;
+  p.items = g->ident_dirty ? nullptr : g->items;
   p.item_pos = g->item_pos;
   p.lab = g->lab;
   p.at = g->at;
@@ -1000,17 +1001,19 @@ pr_status graph_apply(Graph *g, uint64_t nd, const uint32_t *ds, const uint32_t 
   if (n_src > g->pend_cap || n_tgt > g->pend_cap) g->pend_all = true;
   if (h.dead_changed) g->dead_dirty = true;
   if (h.bins_changed) g->ident_dirty = true;
-  // give abandoned slots back once they dominate
-  if (g->out.garbage > g->out.used / 2 && g->out.garbage > 1024) {
-    rc = repack_adj(g, g->out, 0);
-    if (rc != PR_OK) return rc;
-  }
-  if (g->in.garbage > g->in.used / 2 && g->in.garbage > 1024) {
-    rc = repack_adj(g, g->in, 0);
-    if (rc != PR_OK) return rc;
+  // The update is in place: where there is no room to give abandoned slots back once they dominate,
+  // or for larger sweep items, the call has not failed; later ones try again
+  const std::string err = g->err;
+  for (Adj *A : {&g->out, &g->in}) {
+    if (A->garbage <= A->used / 2 || A->garbage <= 1024) continue;
+    rc = repack_adj(g, *A, 0);
+    if (rc != PR_OK && rc != PR_ERR_OUT_OF_MEMORY) return rc;
   }
   // the degree-binned vertex order used by full and dense sweeps follows the graph
-  return graph_refresh_ident(g);
+  rc = graph_refresh_ident(g);
+  if (rc != PR_OK && rc != PR_ERR_OUT_OF_MEMORY) return rc;
+  g->err = err;
+  return PR_OK;
 }
 
 }  // namespace prdf

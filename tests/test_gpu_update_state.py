@@ -122,3 +122,66 @@ def test_a_repack_without_room_leaves_the_rows_their_slots(prdf):
             _check(h, G)
         h.static()
         assert np.abs(h.ranks() - oracle.static_pr(G)[0]).max() <= 2e-9
+
+
+def test_no_room_for_the_sweep_items(prdf):
+    # 32-edge chunks and no other tiers: the update takes every row from 21 entries to 33, so the
+    # items outgrow their arrays.  Whichever allocation fails, a call that fails leaves the
+    # graph as it was, one that does not has updated it, and both leave a usable handle
+    src, dst = _ring(2000, 20)
+    G = oracle.Graph.build(2000, src, dst)
+    p = prdf.pr_params_default()
+    p.vertex_order = 1
+    big = _more(0, 2000, 12, 100)
+    H = G.apply(*big)[0]
+    failed = []
+    for allowed in range(5):
+        with prdf.Graph(2000, src, dst, p) as h:
+            t = h.tuning()
+            h.set_tuning(1, t.bin_hi, t.dense_div, t.blocks_per_sm, 1, 0, 32, 0)
+            h.apply(*(_u([]), _u([]), big[3], big[3]))  # (self pairs: scratch for the real one)
+            prdf.pr_inject_alloc_failure(allowed)
+            try:
+                h.apply(*big)
+                now, ok = H, True
+            except prdf.PrdfError as e:
+                assert e.status == prdf.PR_ERR_OUT_OF_MEMORY
+                now, ok = G, False
+            finally:
+                prdf.pr_inject_alloc_failure(-1)
+            failed.append(not ok)
+            _check(h, now)
+            for up in (_more(5, 3, 2, 700), big):
+                h.apply(*up)
+                now = now.apply(*up)[0]
+                _check(h, now)
+            for call in ("frontier", "static"):
+                getattr(h, call)()
+                assert np.abs(h.ranks() - oracle.static_pr(now)[0]).max() <= 2e-9
+    assert failed[0] and not failed[-1]
+
+
+def test_a_rank_call_without_room_for_the_sweep_items(prdf):
+    src, dst = _ring(2000, 20)
+    G = oracle.Graph.build(2000, src, dst)
+    p = prdf.pr_params_default()
+    p.vertex_order = 1
+    big, small = _more(0, 2000, 12, 100), _more(5, 3, 2, 700)
+    with prdf.Graph(2000, src, dst, p) as h:
+        t = h.tuning()
+        h.set_tuning(1, t.bin_hi, t.dense_div, t.blocks_per_sm, 1, 0, 32, 0)
+        h.apply(*(_u([]), _u([]), big[3], big[3]))
+        prdf.pr_inject_alloc_failure(2)  # both adjacencies' new slots, not the items
+        try:
+            h.apply(*big)
+            for call in (h.static, h.frontier, h.naive):
+                with pytest.raises(prdf.PrdfError) as e:
+                    call()
+                assert e.value.status == prdf.PR_ERR_OUT_OF_MEMORY
+            h.apply(*small)  # in the rows' own slots
+        finally:
+            prdf.pr_inject_alloc_failure(-1)
+        G = G.apply(*big)[0].apply(*small)[0]
+        _check(h, G)
+        h.frontier()
+        assert np.abs(h.ranks() - oracle.static_pr(G)[0]).max() <= 2e-9
