@@ -518,8 +518,9 @@ __global__ void k_comp_items(const uint4 *items, uint32_t n0, uint32_t n1, uint3
 bool batch_eligible(const Graph *g) { return g->ncomp > 1 && g->split_df && g->emap; }
 
 pr_status batch_setup(Graph *g) {
+  // the limit belongs to the function: the same for every handle, whatever its number of graphs
   CKG(cudaFuncSetAttribute(g->f32 ? (const void *)k_batch<true> : (const void *)k_batch<false>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kHotBytes + state_bytes(g->ncomp))));
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kHotBytes + state_bytes(kMaxComponents))));
   return batch_items(g);
 }
 

@@ -45,3 +45,48 @@ def test_traversal_without_iterations_leaves_no_marks(prdf):
             for x in (h, one):
                 x.traversal()
             assert np.array_equal(np.sort(h.affected()), np.sort(one.affected())), k
+
+
+def _batch(gs, k):
+    """A few deleted edges of every graph that has some, spread by k."""
+    first = np.cumsum([0] + [g.n for g in gs])
+    at = [np.arange(k % 7, g.m, max(1, g.m // 9)) for g in gs]
+    return [np.concatenate([np.asarray(getattr(g, c), np.uint32)[i] + np.uint32(f)
+                            for g, i, f in zip(gs, at, first)]).astype(np.uint32) for c in ("src", "dst")]
+
+
+@pytest.mark.parametrize("replay", [False, True])
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("order", [(700, 3), (3, 700), (700, 3, 2)])
+def test_handles_of_different_graph_counts(prdf, order, f32, replay):
+    # all alive at once; every one must give what it gives alone, whichever was made last
+    none = np.zeros(0, np.uint32)
+    p = prdf.pr_params_default()
+    p.precision = prdf.PR_F32 if f32 else prdf.PR_F64
+
+    def make(c):
+        gs = [synth.rmat(4 + (i + c) % 6, 4, seed=9 + i % 13) for i in range(c)]
+        h = prdf.Graph.batched([g.n for g in gs], *_cat(gs), p)
+        h.set_graph_launch(replay)
+        return gs, h
+
+    def calls(gs, h):
+        out = [h.static().converged, h.ranks().copy()]
+        for k, call in enumerate(("frontier", "naive", "traversal", "frontier")):
+            d = _batch(gs, k)
+            h.apply(*(d if k % 2 == 0 else (none, none)), *((none, none) if k % 2 == 0 else _batch(gs, k - 1)))
+            st = getattr(h, call)()
+            out += [st.iterations, st.converged, st.affected_final, h.ranks().copy()]
+        return out
+
+    alone = []
+    for c in order:
+        gs, h = make(c)
+        with h:
+            alone.append(calls(gs, h))
+    made = [make(c) for c in order]
+    for (gs, h), want in zip(made, alone):
+        got = calls(gs, h)
+        assert all(np.array_equal(x, y) for x, y in zip(got, want))
+    for _, h in made:
+        h.close()
