@@ -87,6 +87,7 @@ struct Graph {
   uint32_t pend_cap = 0;
   uint32_t n_pend_src = 0, n_pend_tgt = 0;
   bool pend_all = false;
+  bool unfinished = false;           // the ranks are those of a call that did not finish
 
   RankCtl *ctl = nullptr;            // device
   RankCtl *ctl_h = nullptr;          // pinned host mirror

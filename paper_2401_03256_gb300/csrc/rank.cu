@@ -1326,6 +1326,22 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
   return PR_OK;
 }
 
+// After a rank call that did not finish (a wait ran out, or a launch failed behind another): its
+// blocks left where they were.  The per-call marks and the chunk counters start clean again.  The
+// ranks are a mixture of its iterations, which changed vertices that no pending mark leads to,
+// so the next marking call takes every vertex.  (Errors here: the stream's, reported by every later call.)
+static void abandon_call(Graph *g) {
+  const uint64_t words = ((uint64_t)g->n + 31) / 32;
+  cudaMemsetAsync(g->bitmap, 0, 4 * words, g->st);
+  cudaMemsetAsync(g->xbits, 0, 4 * words, g->st);
+  cudaMemsetAsync(g->stamp, 0xFF, 2ull * g->n, g->st);
+  cudaMemsetAsync(g->chunk_done, 0, 4ull * g->n, g->st);
+  cudaMemsetAsync(g->emap, 0, 2ull * g->n, g->st);
+  cudaStreamSynchronize(g->st);
+  cudaGetLastError();
+  g->unfinished = true;
+}
+
 pr_status rank_run(Graph *g, RankMode mode, pr_stats *stats) {
   pr_status rc;
   const bool marking = mode == kModeDF || mode == kModeDT || mode == kModeDFAsync;
@@ -1334,8 +1350,8 @@ pr_status rank_run(Graph *g, RankMode mode, pr_stats *stats) {
     return PR_ERR_INVALID_ARG;
   }
   // Dynamic Traversal in teleport mode: a changed dead-end mass moves every rank
-  const bool start_full = marking && (g->pend_all || (mode == kModeDT && g->teleport &&
-                                                      (g->n_pend_src > 0 || g->n_pend_tgt > 0)));
+  const bool start_full = marking && (g->pend_all || g->unfinished || (mode == kModeDT && g->teleport &&
+                                                                      (g->n_pend_src > 0 || g->n_pend_tgt > 0)));
   if (g->teleport && (rc = graph_refresh_dead(g)) != PR_OK) return rc;
   if ((rc = graph_refresh_ident(g)) != PR_OK) return rc;
   if (!g->use_graph) CK(cudaMemsetAsync(g->ctl, 0, sizeof(RankCtl), g->st));
@@ -1353,7 +1369,10 @@ pr_status rank_run(Graph *g, RankMode mode, pr_stats *stats) {
   }
   CK(cudaEventRecord(g->ev0, g->st));
   rc = g->f32 ? launch<true>(g, mode, start_full) : launch<false>(g, mode, start_full);
-  if (rc != PR_OK) return rc;
+  if (rc != PR_OK) {
+    abandon_call(g);
+    return rc;
+  }
   CK(cudaEventRecord(g->ev1, g->st));
   CK(cudaMemcpyAsync(g->ctl_h, g->ctl, offsetof(RankCtl, dR_bits), cudaMemcpyDeviceToHost, g->st));
   CK(cudaMemcpyAsync(&g->ctl_h->vproc, &g->ctl->vproc, 5 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
@@ -1365,14 +1384,7 @@ pr_status rank_run(Graph *g, RankMode mode, pr_stats *stats) {
   count_launches(g->ctl_h->launches);
   const RankCtl &h = *g->ctl_h;
   if (h.err) {
-    // the blocks left where they were: the per-call marks and the chunk counters start clean again
-    const uint64_t words = ((uint64_t)g->n + 31) / 32;
-    CK(cudaMemsetAsync(g->bitmap, 0, 4 * words, g->st));
-    CK(cudaMemsetAsync(g->xbits, 0, 4 * words, g->st));
-    CK(cudaMemsetAsync(g->stamp, 0xFF, 2ull * g->n, g->st));
-    CK(cudaMemsetAsync(g->chunk_done, 0, 4ull * g->n, g->st));
-    if (g->emap) CK(cudaMemsetAsync(g->emap, 0, 2ull * g->n, g->st));
-    CK(cudaStreamSynchronize(g->st));
+    abandon_call(g);
     g->err = (h.err & 1u) ? "rank kernel: a grid barrier wait timed out"
                           : "sweep kernel: a staged copy into shared memory did not complete";
     return PR_ERR_DEVICE_TIMEOUT;
@@ -1408,6 +1420,7 @@ pr_status rank_run(Graph *g, RankMode mode, pr_stats *stats) {
   g->n_pend_src = 0;
   g->n_pend_tgt = 0;
   g->pend_all = false;
+  g->unfinished = false;
   if (g->teleport) {
     g->D_ref = h.D_final;
     g->D_ref_n = h.D_final_n;
@@ -1613,6 +1626,7 @@ pr_status rank_set(Graph *g, const double *in_d) {
   }
   count_launch();
   CK(cudaGetLastError());
+  g->unfinished = false;
   if (g->teleport) {
     pr_status rc = graph_refresh_dead(g);
     if (rc != PR_OK) return rc;

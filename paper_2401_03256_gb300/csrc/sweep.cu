@@ -878,6 +878,7 @@ pr_status full_steps_impl(Graph *g, bool from_init) {
   ip.max_iter = g->p.max_iter;
   const dim3 init_grid(std::max(1, g->sm_count * 4)), init_block(256);
   if (!lg.exec) {
+    lg.release();  // what a failed call may have left of one
     CKG(cudaGraphCreate(&lg.graph, 0));
     CKG(cudaGraphConditionalHandleCreate(&lg.h_loop, lg.graph, 0, 0));
     ip.h_loop = lg.h_loop;
@@ -951,6 +952,7 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
   ip.n = g->n;
   ip.m = (uint32_t)g->m;
   if (!lg.exec) {
+    lg.release();  // what a failed call may have left of one
     CKG(cudaGraphCreate(&lg.graph, 0));
     CKG(cudaGraphConditionalHandleCreate(&lg.h_loop, lg.graph, 0, 0));
     CKG(cudaGraphConditionalHandleCreate(&lg.h_fin, lg.graph, 0, 0));
