@@ -723,6 +723,7 @@ pr_status components_setup(Graph *g, const std::vector<uint32_t> &comp_n) {
 }
 
 void graph_free(Graph *g) {
+  sweep_free(g);
   Adj *adjs[2] = {&g->out, &g->in};
   // (what alloc_pieces gave is owned by the first array of each group)
   for (Adj *A : adjs) {
