@@ -334,8 +334,10 @@ pr_status pr_static_noalloc(uint32_t n, int64_t m, const uint64_t *in_off, const
  * different graphs run concurrently on their graphs' streams (create each graph with its
  * own stream for overlap).  A request is admitted when one of `slots` device slots is free
  * and free device memory (cudaMemGetInfo) covers hbm_reserve_bytes plus the request's
- * estimate; an idle device always admits one request.  Attaching a graph sizes its
- * persistent launch to 1/slots of the resident blocks so concurrent launches fit together.
+ * estimate; an idle device always admits one request.  While attached, a graph's launches that
+ * run to the end of a call take at most 1/slots of the device, so that concurrent ones fit together;
+ * the iterations of a dense frontier take all of it, in turns of about 2 ms.  pr_server_destroy
+ * gives every graph its own launch sizes back.
  * An update = one pr_apply_batches over the coalesced requests in submission order + one
  * pr_dynamic_frontier;
  * results carry host-clock times in ms since the server was created.  While attached, a

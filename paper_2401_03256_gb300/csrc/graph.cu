@@ -723,6 +723,10 @@ pr_status components_setup(Graph *g, const std::vector<uint32_t> &comp_n) {
 }
 
 void graph_free(Graph *g) {
+  for (auto &at : g->served) {
+    std::lock_guard<std::mutex> lk(at->mu);
+    at->g = nullptr;
+  }
   sweep_free(g);
   Adj *adjs[2] = {&g->out, &g->in};
   // (what alloc_pieces gave is owned by the first array of each group)

@@ -186,6 +186,7 @@ struct RankCtl {
   uint32_t pull_all;      // the pull kernel also pulls tier-0/1 rows (the marks after the last iteration)
   unsigned long long bar_limit_ns;  // grid-barrier wait limit (0 = the default)
   uint32_t fin_only;      // a marking launch handed off only for the marks of its last iteration
+  uint32_t run_cap;       // iterations of a run of compacted ones at most (0: until it stops by itself)
   unsigned long long eprev;  // edges processed before the current iteration
   // trace (written by block 0): %globaltimer at kernel start, after phase 0 and after each
   // iteration's barrier; affected vertices at the start of each iteration; iteration kind

@@ -2,6 +2,8 @@
 #pragma once
 
 #include <initializer_list>
+#include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -34,6 +36,14 @@ Piece piece(T **p, uint64_t count) { return Piece{(void **)p, sizeof(T) * (count
 cudaError_t alloc_pieces(std::initializer_list<Piece> pieces);
 
 constexpr int kRankBlocksPerSm = 4;  // most blocks of the rank kernel on an SM
+
+// A handle's place in a server: the launch sizes it had before.  Either may go first.
+struct Graph;
+struct Served {
+  std::mutex mu;
+  Graph *g = nullptr;  // null once the handle is destroyed
+  int rank_grid = 0, few_grid_max = 0;
+};
 
 struct Graph {
   int device = 0;
@@ -143,10 +153,11 @@ struct Graph {
   // iterations and the CUDA graphs that loop over the iterations on the device
   uint8_t *emap = nullptr;           // [2][n] rank change above tau_f, by iteration parity; 0 between calls
   void *loops = nullptr;             // sweep.cu's cached graphs
-  int loop_grid = 0;                 // blocks of a run of iterations (one persistent launch)
+  int loop_grid = 0;                 // blocks of a persistent launch that runs to the end of its call
+  bool bounded_runs = false;         // runs of compacted iterations end early to let other handles' launches in
   int pro_grid = 0;                  // blocks of the cooperative prologue launch
-  int pro_grid_max = 0;              // blocks of it that can be resident
   bool loop_sweeps = true;           // single-graph self-loop handles iterate in per-iteration launches
+  std::vector<std::shared_ptr<Served>> served;  // the servers it is attached to
   std::string err;
 };
 
@@ -207,7 +218,9 @@ bool sweep_eligible(const Graph *g);  // single graph, self-loop mode, no graph-
 pr_status sweep_full(Graph *g, bool from_init);                  // all vertices, every iteration
 pr_status sweep_dense(Graph *g, RankMode mode, const void *rank_args);  // after the marking launch's handoff
 void sweep_free(Graph *g);
-void sweep_share(Graph *g, int slots);  // cooperative launches of at most 1/slots of the device
+// A handle in a server of `slots` slots (1: by itself): launches that run to the end of their call on at
+// most 1/slots of the device, bounded runs of the compacted iterations of a Dynamic Frontier call.
+void sweep_share(Graph *g, int slots);
 
 }  // namespace prdf
 

@@ -5,9 +5,11 @@
 // the graph at a time).  A request is admitted when one of `slots` device slots is free
 // and cudaMemGetInfo shows at least `hbm_reserve_bytes` plus the request's estimate free;
 // admitted requests of different graphs run at the same time on their graphs' own
-// streams.  Each graph's persistent rank launch is sized to 1/slots of the blocks that can
-// be resident, so the cooperative kernels of concurrent requests always fit on the device
-// together.  Continuous batching: when a graph's worker gets a slot it takes the requests
+// streams.  A graph's marking launch takes 1/slots of the blocks that can be resident.  Its dense
+// iterations take the whole device, about 2 ms at a time (sweep.cu), so that concurrent requests
+// take turns.  (On 1/slots each, a request alone left half of the device idle: eight R-MAT graphs of
+// 2^18 to 2^24 vertices, 2 slots: service p99 at 50 requests/s 61 ms, now 45; p50 and p99 at
+// saturation 94 and 404 ms, now 72 and 204.)  Continuous batching: when a graph's worker gets a slot it takes the requests
 // queued for that graph by then (up to max_coalesce), applies their batches in order with
 // one pr_apply_batches and runs one pr_dynamic_frontier over the net change;
 // each result records submit, start and completion times (host clock) and the stats.
@@ -44,6 +46,7 @@ struct pr_server {
   std::mutex mu;
   std::condition_variable cv_work, cv_done, cv_slot;
   std::vector<pr_graph *> graphs;
+  std::vector<std::shared_ptr<prdf::Served>> attached;
   std::vector<std::deque<Request>> queues;
   std::vector<std::thread> workers;
   std::map<uint64_t, pr_request_result> done;
@@ -213,7 +216,15 @@ pr_status pr_server_add_graph(pr_server *s, pr_graph *g, int32_t *index) {
   if (!s || !g) return PR_ERR_INVALID_ARG;
   std::lock_guard<std::mutex> lk(s->mu);
   if (s->stopping || s->graphs.size() >= 1024) return PR_ERR_INVALID_ARG;
-  // 1/slots of the resident blocks, so concurrent requests' cooperative launches fit together
+  auto at = std::make_shared<prdf::Served>();
+  at->g = &g->g;
+  at->rank_grid = g->g.rank_grid;
+  at->few_grid_max = g->g.few_grid_max;
+  auto &served = g->g.served;
+  served.erase(std::remove_if(served.begin(), served.end(), [](auto &x) { return x.use_count() == 1; }), served.end());
+  served.push_back(at);
+  s->attached.push_back(at);
+  // 1/slots of the resident blocks, so concurrent requests' marking launches fit together
   g->g.rank_grid = std::max(1, g->g.rank_grid_max / s->cfg.slots);
   // and no marking launches of 2 blocks an SM: those take the registers that the other slots'
   // sweeps wait for (5 graphs, 2 slots, 10 requests: 23.5 ms with them, 16.9 without)
@@ -281,6 +292,15 @@ pr_status pr_server_destroy(pr_server *s) {
   }
   s->cv_work.notify_all();
   for (auto &t : s->workers) t.join();
+  // the graphs get their launch sizes back (the last attachment of one first)
+  for (auto it = s->attached.rbegin(); it != s->attached.rend(); ++it) {
+    prdf::Served &a = **it;
+    std::lock_guard<std::mutex> lk(a.mu);
+    if (!a.g) continue;
+    a.g->rank_grid = a.rank_grid;
+    a.g->few_grid_max = a.few_grid_max;
+    prdf::sweep_share(a.g, 1);
+  }
   delete s;
   return PR_OK;
 }

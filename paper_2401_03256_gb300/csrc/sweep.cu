@@ -37,6 +37,12 @@ namespace prdf {
 
 constexpr uint32_t kPullDiv = 256;  // more than n / kPullDiv first expansions: the next iteration pulls
 constexpr uint32_t kPullMin = 64;   // and at least this many
+// A handle in a server: in-edges (of the whole graph) of a run's iterations at most, about 2 ms.  A
+// block of a run holds its SM's registers, so other requests' launches wait for its end.  Eight R-MAT
+// graphs of 2^18 to 2^24 vertices, 2 slots, 50 requests/s: 3 in 100 of the four smallest graphs'
+// requests take more than 21 to 27 ms (23 to 30 with unbounded runs), of the largest's 54 (49);
+// at saturation no difference, nor between 2^27 and 2^31.
+constexpr uint64_t kRunEdges = 1ull << 29;
 constexpr uint32_t kLightPush = 16384;  // at most this many first expansions: the light push may mark them
 
 // End of an all-item iteration, or of a run of compacted iterations it_first ... it, by one
@@ -273,7 +279,7 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_loop(const LoopArgs<F32> p) 
   Pass<F32> io{};
   io.sbase = smem_addr(s_hot);
   io.r = &s_rounds;
-  uint32_t it = 0, epoch = 0;
+  uint32_t it = 0, epoch = 0, it_cap = 0xFFFFFFFFu;  // it_cap: a bounded run ends with the iteration before
   unsigned long long seen[2] = {0, 0};
   // an error ends the device-side loop: nothing else would
   auto give_up = [&]() {
@@ -285,6 +291,7 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_loop(const LoopArgs<F32> p) 
   };
   if constexpr (CMP) {
     it = __ldcg(&ctl->it_cur);
+    if (const uint32_t cap = __ldcg(&ctl->run_cap)) it_cap = it + cap;
     if (tid == 0)
       deal_rounds(s_rounds, __ldcg(&ctl->cmp_cur[0]), __ldcg(&ctl->cmp_cur[1]), __ldcg(&ctl->cmp_cur[2]),
                   __ldcg(&ctl->sw_off[0]), __ldcg(&ctl->sw_off[1]), a.hot);
@@ -332,7 +339,7 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_loop(const LoopArgs<F32> p) 
         ctl->it_kind[it] = 3;
       }
     }
-    if (s_left != 1u || (int)it + 1 >= a.max_iter) break;  // (nothing above the tolerance, or first expansions)
+    if (s_left != 1u || (int)it + 1 >= a.max_iter || it + 1 >= it_cap) break;  // (nothing above the tolerance, or first expansions)
   }
   if constexpr (CMP) {
     if (tid == 0) {
@@ -438,6 +445,7 @@ struct DenseInit {
   uint32_t sw_all[3], sw_off[2];
   uint32_t n, m;
   uint32_t traversal;
+  uint32_t run_cap;
   int max_iter;
   cudaGraphConditionalHandle h_loop, h_pro, h_mode, h_fin;
 };
@@ -473,6 +481,7 @@ __global__ void k_dense_init(const DenseInit p) {
   ctl->sw_off[0] = p.sw_off[0];
   ctl->sw_off[1] = p.sw_off[1];
   ctl->m_cur = p.m;
+  ctl->run_cap = p.run_cap;
   ctl->xdone = ctl->xcnt;
   ctl->xcap = max(kPullMin, p.n / kPullDiv) + 1;  // first iteration: a pull may follow
   ctl->x_long = 0;
@@ -939,8 +948,6 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
   std::vector<unsigned char> key;
   append_key(key, a);
   append_key(key, ra);
-  append_key(key, g->loop_grid);
-  append_key(key, g->pro_grid);
   if (lg.exec && key != lg.key) lg.release();
   DenseInit ip{};
   ip.ctl = g->ctl;
@@ -948,6 +955,7 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
   ip.sw_off[0] = g->item_cnt[0];
   ip.sw_off[1] = g->item_cnt[0] + g->item_cnt[1];
   ip.traversal = mode == kModeDT ? 1u : 0u;
+  if (g->bounded_runs) ip.run_cap = (uint32_t)std::max<uint64_t>(1, kRunEdges / std::max<uint64_t>(1, g->m));
   ip.max_iter = g->p.max_iter;
   ip.n = g->n;
   ip.m = (uint32_t)g->m;
@@ -991,7 +999,7 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
     LoopArgs<F32> la{};
     la.a = a;
     void *largs[] = {(void *)&la};
-    CKG(add_kernel(&s0, sw[0], nullptr, 0, (const void *)k_loop<F32, true>, dim3(g->loop_grid), dim3(kSweepBlock), largs,
+    CKG(add_kernel(&s0, sw[0], nullptr, 0, (const void *)k_loop<F32, true>, dim3(g->sm_count), dim3(kSweepBlock), largs,
                    true, hot_bytes(a)));
     void *sargs[] = {(void *)&a};
     CKG(add_kernel(&s1, sw[1], nullptr, 0, (const void *)k_sweep<F32, 1>, dim3(g->sm_count),
@@ -1047,14 +1055,14 @@ pr_status sweep_setup(Graph *g) {
   int per_sm_pro = 0;
   CKG(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
       &per_sm_pro, g->f32 ? (const void *)k_df_push<true> : (const void *)k_df_push<false>, kRankBlock, 0));
-  g->pro_grid = g->pro_grid_max = std::max(1, std::min(per_sm_pro, 4)) * g->sm_count;
+  g->pro_grid = std::max(1, std::min(per_sm_pro, 4)) * g->sm_count;
   if (!g->loops) g->loops = new Loops();
   return PR_OK;
 }
 
 void sweep_share(Graph *g, int slots) {
   g->loop_grid = std::max(1, g->sm_count / slots);
-  g->pro_grid = std::max(1, g->pro_grid_max / slots);
+  g->bounded_runs = slots > 1;
 }
 
 bool sweep_eligible(const Graph *g) {
