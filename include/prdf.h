@@ -176,8 +176,9 @@ pr_status pr_set_tuning(pr_graph *g, const pr_tuning *t);
 pr_status pr_get_tuning(const pr_graph *g, pr_tuning *t);
 
 /* Autotuner: times sweep_iters-iteration Naive-dynamic sweeps of this graph for each
- * candidate bin_lo (4, 8, 16, 32) and blocks per SM, keeps the fastest, restores the ranks
- * and pending marks, and returns the choice in *chosen (may be NULL). */
+ * candidate bin_lo (4, 8, 16, 32) and blocks per SM (handles whose sweeps run in the persistent
+ * launch, see df_split; others keep theirs), then each sweep tile, keeps the fastest, restores the
+ * ranks and pending marks, and returns the choice in *chosen (may be NULL). */
 pr_status pr_autotune(pr_graph *g, int32_t sweep_iters, pr_tuning *chosen);
 
 /* enable != 0: rank calls replay one CUDA graph (control-block reset + the cooperative

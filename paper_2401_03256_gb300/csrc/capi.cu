@@ -224,7 +224,8 @@ pr_status pr_set_graph_launch(pr_graph *h, int32_t enable) {
 }
 
 // Autotuner: times Naive-dynamic sweeps of sweep_iters iterations (the full-sweep cost the
-// thresholds steer) for every candidate bin_lo x blocks-per-SM, then, at the fastest of
+// thresholds steer) for every candidate bin_lo x blocks-per-SM (where those sweeps run in the
+// launch of that size; else the blocks stay as they are), then, at the fastest of
 // those, every sweep tile (chunk_len x group_max); keeps the fastest and restores the ranks.
 // FP64 results do not depend on the choice; FP32 ones only through the order of additions.
 pr_status pr_autotune(pr_graph *h, int32_t sweep_iters, pr_tuning *chosen) {
@@ -244,7 +245,9 @@ pr_status pr_autotune(pr_graph *h, int32_t sweep_iters, pr_tuning *chosen) {
   pr_tuning best = cur;
   best.ms = 1e30;
   const int32_t los[] = {4, 8, 16, 32};
-  const int per_sm_max = std::max(1, g.rank_grid_max / g.sm_count);
+  const bool blocks = !prdf::sweep_eligible(&g) && !prdf::batch_eligible(&g);
+  const int per_sm_max = blocks ? std::max(1, g.rank_grid_max / g.sm_count) : std::max(1, cur.blocks_per_sm);
+  const int per_sm_min = blocks ? std::max(1, per_sm_max - 2) : std::max(1, cur.blocks_per_sm);
   g.p.max_iter = sweep_iters;
   // time candidate t (best of two); a capacity refusal of a tile only skips that tile
   auto trial = [&](const pr_tuning &t) -> pr_status {
@@ -266,7 +269,7 @@ pr_status pr_autotune(pr_graph *h, int32_t sweep_iters, pr_tuning *chosen) {
     return r;
   };
   for (int32_t lo : los) {
-    for (int bps = std::max(1, per_sm_max - 2); bps <= per_sm_max && rc == PR_OK; bps++) {
+    for (int bps = per_sm_min; bps <= per_sm_max && rc == PR_OK; bps++) {
       pr_tuning t = cur;
       t.bin_lo = lo;
       t.bin_hi = std::max(cur.bin_hi, lo);
