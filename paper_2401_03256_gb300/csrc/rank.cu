@@ -1082,6 +1082,7 @@ __global__ void __launch_bounds__(kRankBlock, SPLIT == 1 ? kFewMarksBlocks : PRD
 
 static constexpr double kOne62 = 4611686018427387904.0;  // 2^62
 static constexpr double kFewMarks = 32768.0;
+static constexpr uint32_t kFewVertices = 1u << 21;
 
 // Dynamic shared memory of k_rank: per-component max key, base, iteration count, active flag.
 static size_t rank_smem(uint32_t ncomp) { return ((size_t)ncomp * 19 + 15) & ~(size_t)15; }
@@ -1255,12 +1256,18 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
   // latency (sparse iterations of 4200 pairs on a graph of 20 M vertices of degree 2: 24 us
   // instead of 29, the call 3.87 to 3.63 ms).  Many marks at once want the warps (60,000
   // sources with 17 M marks: 0.95 ms with 4 blocks, 1.22 with 2).  Few is told by the marks
-  // expected when the first ones have expanded, sources times the mean degree squared: at 26,000
-  // (the graph above) 2 blocks are ahead, at 48,000 (650 sources, R-MAT, 4.2 M vertices) the
-  // first iteration takes 254 us with 4 and 290 with 2.
+  // expected when the first ones have expanded, sources times the mean degree squared, and by how
+  // far marks spread: where long rows (hubs) take the frontier over millions of vertices, 2 blocks
+  // lose from the first edge on.  Calls with 2 blocks, time over that with 4, 1 to 300 changed edges, both
+  // precisions, Dynamic Frontier and Traversal: chains of 4 M vertices 0.78-0.99 and 0.80-0.88, a
+  // grid of 4 M 0.78-0.99 and 0.96-0.98; R-MAT of 2^14 and 2^18 vertices 0.95-1.01 and 0.91-0.97, of
+  // 2^20 0.93-1.01 and 0.99-1.02, of 2^22 (edge factors 4 to 16) 0.95-1.13, mostly 1.01-1.03, and
+  // 1.00-1.04.  With more changed edges than the limit the two are within 2% of one another except
+  // for Traversal on chains (0.82-0.92) and large R-MAT graphs (1.02-1.03).
   const bool split = marking && a.split && !g->use_graph;
   const double degree = (double)g->m / (double)g->n;
-  const bool few = split && g->few_grid_max && (double)g->n_pend_src * degree * degree <= kFewMarks;
+  const bool far = g->n > kFewVertices && (uint64_t)g->item_cnt[2] * 1024 >= g->n;
+  const bool few = split && g->few_grid_max && !far && (double)g->n_pend_src * degree * degree <= kFewMarks;
   const void *fn = few      ? (const void *)k_rank<F32, true, 1>
                    : split   ? (const void *)k_rank<F32, true, 3>
                    : marking ? (const void *)k_rank<F32, true>
