@@ -161,10 +161,11 @@ pr_status pr_get_component_stats(const pr_graph *g, pr_stats *stats, int32_t nco
 typedef struct {
     int32_t bin_lo, bin_hi, dense_div, blocks_per_sm;
     int32_t df_split;
-    int32_t barrier_us;  /* bounded wait of a grid barrier in the persistent launches, in
-                            microseconds (0 = the default 4 s); a wait that runs out ends the
-                            launch and the call returns PR_ERR_DEVICE_TIMEOUT.  A short value
-                            exercises that path in tests. */
+    int32_t barrier_us;  /* bounded wait of a grid barrier in the persistent launches and in the
+                            planning of an update, in microseconds (0 = the default 4 s); a
+                            wait that runs out ends the launch and the call returns
+                            PR_ERR_DEVICE_TIMEOUT (an update leaves the graph as it was).  A
+                            short value exercises that path in tests. */
     int32_t chunk_len;   /* a multiple of 32 in [32, 512]; a vertex may have at most
                             2^21 chunks (else PR_ERR_CAPACITY) */
     int32_t group_max;   /* [0, 64] */

@@ -235,6 +235,7 @@ struct ApplyCtl {
   unsigned long long longq;                 // long rows queued by the merge (high word) and their slices (low)
   uint32_t n_long;                          // long rows among the touched ones
   uint32_t bar, err;                        // grid barrier of the plan; a wait of it ran out
+  unsigned long long bar_limit_ns;          // its wait limit (0 = the default)
 };
 
 // ------------------------------------------------------------------- primitives ---

@@ -185,3 +185,34 @@ def test_a_rank_call_without_room_for_the_sweep_items(prdf):
         _check(h, G)
         h.frontier()
         assert np.abs(h.ranks() - oracle.static_pr(G)[0]).max() <= 2e-9
+
+
+@pytest.mark.parametrize("k", [2049, 5000, 200000])
+def test_a_barrier_wait_of_the_plan_runs_out(prdf, k):
+    # (updates of at most 2048 pairs are planned by one block, which waits for no other)
+    n = 40000
+    src, dst = _u(np.arange(n)), _u((np.arange(n) + 1) % n)
+    rng = np.random.default_rng(k)
+    none = _u([])
+    G = oracle.Graph.build(n, src, dst)
+    with prdf.Graph(n, src, dst) as h:
+        t = h.tuning()
+        ended = 0
+        for _ in range(6):
+            up = (none, none, *(rng.integers(0, n, k).astype(np.uint32) for _ in range(2)))
+            h.set_tuning(t.bin_lo, t.bin_hi, t.dense_div, t.blocks_per_sm, 1, 1)  # 1 us
+            try:
+                h.apply(*up)
+                G = G.apply(*up)[0]
+            except prdf.PrdfError as e:
+                assert e.status == prdf.PR_ERR_DEVICE_TIMEOUT
+                ended += 1
+                _check(h, G)
+                h.set_tuning(t.bin_lo, t.bin_hi, t.dense_div, t.blocks_per_sm, 1, 0)
+                h.apply(*up)
+                G = G.apply(*up)[0]
+            _check(h, G)
+        assert ended > 0 or k < 200000  # a few blocks may always meet within the limit
+        h.set_tuning(t.bin_lo, t.bin_hi, t.dense_div, t.blocks_per_sm, 1, 0)
+        h.frontier()
+        assert np.abs(h.ranks() - oracle.static_pr(G)[0]).max() <= 2e-9
