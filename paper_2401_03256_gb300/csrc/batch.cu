@@ -515,7 +515,23 @@ __global__ void k_comp_items(const uint4 *items, uint32_t n0, uint32_t n1, uint3
 
 }  // namespace
 
-bool batch_eligible(const Graph *g) { return g->ncomp > 1 && g->split_df && g->emap; }
+// Where this launch is ahead of the one persistent launch (k_rank).  An iteration here sweeps a block's
+// graphs one after another and starts a copy for each; there all rows are dealt to all warps, at
+// the general kernel's rate.  Calls over every vertex, R-MAT graphs of equal size (edge factor 8), us
+// an iteration here and there: 1024 graphs of 32 vertices 47 and 9, 512 of 1024 49.5 and 30, of 2048 69
+// and 56 (FP32 53 and 52), 128 of 4096 34 and 34 (27 and 36), 8 of 2^14 (1.1 M edges) 19 and 14 (17 and
+// 15), 32 of 2^14 (4.4 M) 33 and 36 (27 and 37), 2 of 2^18 (4.6 M) 34 and 33 (28 and 34), 32 of 2^16 92 and
+// 138 (70 and 124): from 4 M edges (FP32 2 M) in graphs of 4096 (2048) vertices on average.
+// Marking calls gain from the cheaper growth of the frontier too (time here over there mostly 0.55
+// to 0.95), except where a block has several small graphs: 512 graphs of 1024 vertices 1.76 at
+// 1e-5 of the edges and 1.00 at 1e-3, of 256 0.93 and 1.26, of 32 0.95 and 1.49; 128 of 32 0.96 and 1.25,
+// of 256 0.94 and 0.94, of 1024 0.93 and 0.85.
+bool batch_eligible(const Graph *g, bool marking) {
+  if (g->ncomp <= 1 || !g->split_df) return false;
+  const uint64_t mean = g->n / g->ncomp;
+  if (marking) return mean >= 2048 || g->ncomp <= std::min<uint64_t>((uint64_t)g->sm_count, 2 * mean);
+  return g->f32 ? g->m >= (2u << 20) && mean >= 2048 : g->m >= (4u << 20) && mean >= 4096;
+}
 
 pr_status batch_setup(Graph *g) {
   // the limit belongs to the function: the same for every handle, whatever its number of graphs

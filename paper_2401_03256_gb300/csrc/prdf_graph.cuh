@@ -200,10 +200,10 @@ pr_status rank_get(Graph *g, double *out_d);
 pr_status rank_dead_mass(Graph *g, double *D);
 pr_status components_setup(Graph *g, const std::vector<uint32_t> &comp_n);  // after graph_build
 
-// batch.cu: the iterations of batched handles (unless df_split is 0), one persistent launch
-// after the marking launch of marking calls.
+// batch.cu: the iterations of batched handles (unless df_split is 0 or the graphs are small), one
+// persistent launch after the marking launch of marking calls.
 constexpr int kGraphWhole = 0, kGraphMarking = 1, kGraphBatchMarking = 2, kGraphBatchEvery = 3;
-bool batch_eligible(const Graph *g);
+bool batch_eligible(const Graph *g, bool marking);  // of a call that marks, or of one over every vertex
 pr_status batch_setup(Graph *g);
 pr_status batch_items(Graph *g);  // after a rebuild of the sweep items
 pr_status batch_run(Graph *g, RankMode mode, bool marking, const void *rank_args);

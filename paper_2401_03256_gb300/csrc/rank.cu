@@ -1222,7 +1222,7 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
   a.emap = g->emap;
   a.item_pos = g->item_pos;
   const bool marking = mode == kModeDF || mode == kModeDT || async;
-  const bool loops = sweep_eligible(g), batch = batch_eligible(g);
+  const bool loops = sweep_eligible(g), batch = batch_eligible(g, marking && !start_full);
   a.split = marking && (loops || batch) && g->split_df && !start_full;
   // expected marks of a set of k vertices: k * m / n; deferring to a pull pays once they
   // would make the next set dense (more than n / dense_div) several times over: a pull

@@ -57,7 +57,7 @@ def _batch(gs, k):
 
 @pytest.mark.parametrize("replay", [False, True])
 @pytest.mark.parametrize("f32", [False, True])
-@pytest.mark.parametrize("order", [(700, 3), (3, 700), (700, 3, 2)])
+@pytest.mark.parametrize("order", [(150, 3), (3, 150), (150, 3, 2), (700, 3)])
 def test_handles_of_different_graph_counts(prdf, order, f32, replay):
     # all alive at once; every one must give what it gives alone, whichever was made last
     none = np.zeros(0, np.uint32)
@@ -90,3 +90,33 @@ def test_handles_of_different_graph_counts(prdf, order, f32, replay):
         assert all(np.array_equal(x, y) for x, y in zip(got, want))
     for _, h in made:
         h.close()
+
+
+@pytest.mark.parametrize("f32", [False, True])
+def test_calls_over_every_vertex(prdf, f32):
+    # graphs large enough for a launch of their own (4 M edges, 4096 vertices on average), from one
+    # vertex up to more than an SM's copy holds: bit for bit the one persistent launch, whatever
+    # handle is made in between
+    gs = [synth.rmat(17, 16, seed=3), synth.rmat(16, 16, seed=4), synth.from_pairs(1, [], "one"),
+          synth.rmat(17, 16, seed=5), synth.rmat(11, 8, seed=6)]
+    p = prdf.pr_params_default()
+    p.precision = prdf.PR_F32 if f32 else prdf.PR_F64
+    out = []
+    for split, max_iter in ((1, 500), (0, 500), (1, 3), (0, 3), (1, 0), (0, 0)):
+        p.max_iter = max_iter
+        with prdf.Graph.batched([g.n for g in gs], *_cat(gs), p) as h:
+            assert h.info()[1] >= 4 << 20
+            t = h.tuning()
+            h.set_tuning(t.bin_lo, t.bin_hi, t.dense_div, t.blocks_per_sm, split)
+            with prdf.Graph.batched([2, 3], np.array([0], np.uint32), np.array([1], np.uint32), p) as small:
+                small.static()
+            res = []
+            for k, call in enumerate(("static", "naive", "naive", "static")):
+                st = getattr(h, call)()
+                res.append((h.ranks().copy(), st.iterations, st.converged,
+                            [(c.iterations, c.converged, c.last_delta) for c in h.component_stats()]))
+                h.apply(*_batch(gs, k), np.zeros(0, np.uint32), np.zeros(0, np.uint32))
+            out.append(res)
+    for a, b in zip(out[::2], out[1::2]):
+        for x, y in zip(a, b):
+            assert np.array_equal(x[0], y[0]) and x[1:] == y[1:]
