@@ -89,6 +89,13 @@ __global__ void k_na_check_deg(const uint32_t *deg, uint32_t n, NaCtl *ctl) {
 // a call), because of its hub rows; segments of 512 edges summed by warps and finished by one
 // lane 35 us (2.4 ms); this 20 us (1.47 ms).
 //
+// A block whose rows are alike gives each of them a thread, which needs no tree and finishes the row
+// at once: most rows longer than kLaneRow (limit x 4 until at most one row in eight is above it; those
+// are listed), or none and kShortRows edges on average.  262,144 vertices with 25 in-edges each 0.37 ms
+// a call (four lanes, segments and warps for what the lists have no room for: 1.18), 131,072 with 81 each
+// 0.42 (0.57), the same with 25 and 130 hubs of 5000 0.43 (0.69), a path of 200,000 0.94 (1.43), a grid of
+// 250,000 0.70 (1.01).  With a mean of up to 10 for short rows nothing else changes.
+//
 // One Jacobi iteration of Eq. 1: R[v] = (1 - alpha) / n + alpha * sum over in-edges (u, v)
 // of c_in[u]; c_out[v] = R[v] / |out(v)|.  The rank is updated in place (the sums read only
 // c_in, through L2: other SMs wrote it during this launch).  After each iteration's barrier
@@ -98,6 +105,8 @@ constexpr int kLoopWarps = kLoopThreads / 32;
 constexpr uint32_t kRowWeight = 4;     // work of a row beside its edges, in edges
 constexpr uint32_t kLaneRow = 16;      // edges of a row summed by four lanes at once
 constexpr uint32_t kSegment = 64;      // edges of a segment of a longer row
+constexpr uint32_t kThreadRow = 16384; // edges of a row summed by one thread at most
+constexpr uint32_t kShortRows = 6;     // mean edges of rows that are short enough for a thread each
 constexpr uint32_t kMaxSegs = 1024;    // segments of one row at most (more edges each for huge rows)
 constexpr uint32_t kLongCap = 1024, kSegCap = 2048;  // listed rows and their segments per block
 constexpr uint32_t kTile = 2048;       // rows whose sums are in shared memory together
@@ -154,21 +163,32 @@ __global__ void __launch_bounds__(kLoopThreads, 1)
     c0[v] = r0 / (double)deg[v];
   }
   __syncthreads();
-  const uint32_t lo = s_range[0], hi = s_range[1];
-  uint32_t listed_rows = 0;  // rows longer than kLaneRow so far, in row order
-  for (uint32_t b0 = lo; b0 < hi; b0 += kLoopThreads) {
-    const uint32_t v = b0 + tid;
-    const bool f = v < hi && __ldg(off + v + 1) - __ldg(off + v) > kLaneRow;
-    const uint32_t mask = __ballot_sync(0xffffffffu, f);
-    if (lane == 0) s_cnt[wib] = __popc(mask);
-    __syncthreads();
-    uint32_t at = listed_rows + __popc(mask & prdf::lanemask_lt());
-    for (uint32_t w = 0; w < (uint32_t)kLoopWarps; w++) {
-      at += w < wib ? s_cnt[w] : 0u;
-      listed_rows += s_cnt[w];
+  const uint32_t lo = s_range[0], hi = s_range[1], rows = hi - lo;
+  uint32_t listed_rows = 0;  // rows longer than the limit so far, in row order
+  auto list_rows = [&](uint32_t limit) {
+    listed_rows = 0;
+    for (uint32_t b0 = lo; b0 < hi; b0 += kLoopThreads) {
+      const uint32_t v = b0 + tid;
+      const bool f = v < hi && __ldg(off + v + 1) - __ldg(off + v) > limit;
+      const uint32_t mask = __ballot_sync(0xffffffffu, f);
+      if (lane == 0) s_cnt[wib] = __popc(mask);
+      __syncthreads();
+      uint32_t at = listed_rows + __popc(mask & prdf::lanemask_lt());
+      for (uint32_t w = 0; w < (uint32_t)kLoopWarps; w++) {
+        at += w < wib ? s_cnt[w] : 0u;
+        listed_rows += s_cnt[w];
+      }
+      if (f && at < kLongCap) s_long[at] = v;
+      __syncthreads();
     }
-    if (f && at < kLongCap) s_long[at] = v;
-    __syncthreads();
+  };
+  // how this block takes its rows (see above): four lanes each, or a thread each up to `limit` edges
+  uint32_t limit = kLaneRow;
+  list_rows(limit);
+  bool by_thread = listed_rows == 0 && rows && __ldg(off + hi) - __ldg(off + lo) <= (uint64_t)kShortRows * rows;
+  if (listed_rows * 2 > rows) {
+    by_thread = true;
+    while (listed_rows * 8 > rows && limit < kThreadRow) list_rows(limit *= 4);
   }
   if (tid == 0) {
     // segments of the listed rows; rows from s_list_end on, which the lists have no room for,
@@ -257,7 +277,47 @@ __global__ void __launch_bounds__(kLoopThreads, 1)
       t += __shfl_xor_sync(0xffffffffu, t, 2);
       if (gl == 0 && k < nseg) s_part[k] = t;
     }
-    for (uint32_t t0 = lo; t0 < hi; t0 += kTile) {
+    if (by_thread) {
+      // a row a lane, eight gathers in flight, the next columns on their way meanwhile
+      for (uint32_t b0 = lo + wib * 32; b0 < hi; b0 += kLoopThreads) {
+        const uint32_t v = b0 + lane;
+        uint64_t s = 0, e = 0;
+        if (v < hi) {
+          s = __ldg(off + v);
+          e = __ldg(off + v + 1);
+        }
+        const uint64_t len = e - s;
+        const bool mine = v < hi && len <= limit;
+        double t = 0.0;
+        if (mine) {
+          const uint32_t k = (uint32_t)len;
+          const uint32_t *c = col + s;
+          for (uint32_t j0 = 0; j0 < k; j0 += 8) {
+            double x[8];
+#pragma unroll
+            for (int q = 0; q < 8; q++) x[q] = j0 + q < k ? __ldcg(c_in + __ldg(c + j0 + q)) : 0.0;
+            const uint32_t left = k - j0;  // (no additions of zeros: the FP64 rate is the bound)
+            double u = x[0];
+            if (left > 1) u += x[1];
+            if (left > 2) u += left > 3 ? x[2] + x[3] : x[2];
+            if (left > 4) u += left > 6 ? (x[4] + x[5]) + (left > 7 ? x[6] + x[7] : x[6]) : (left > 5 ? x[4] + x[5] : x[4]);
+            t += u;
+          }
+        }
+        uint32_t more = __ballot_sync(0xffffffffu, v < hi && !mine && v >= list_end);
+        const bool listed = v < hi && !mine && v < list_end;
+        while (more) {
+          const int src = __ffs(more) - 1;
+          more &= more - 1;
+          const uint64_t rs = __shfl_sync(0xffffffffu, s, src), re = __shfl_sync(0xffffffffu, e, src);
+          const double x = na_warp_row(col, c_in, rs, re, lane);
+          if ((int)lane == src) t = x;
+        }
+        if (v < hi && !listed) finish(v, t);
+      }
+      __syncthreads();  // the segments of the listed rows
+    }
+    for (uint32_t t0 = lo; t0 < hi && !by_thread; t0 += kTile) {
       const uint32_t t1 = hi - t0 < kTile ? hi : t0 + kTile;
       // eight rows a warp, four lanes a row
       for (uint32_t b0 = t0 + wib * 8; b0 < t1; b0 += kLoopWarps * 8) {
