@@ -343,6 +343,13 @@ pr_status vertex_order(Graph *g, int kind, uint32_t *perm, uint32_t *inv, const 
   pr_status rc = apply_scratch(g, n);
   if (rc != PR_OK) return rc;
   ApplyScratch &s = g->sc;
+  // a level's counters, side by side: chains have a thousand levels, and each clears and reads them
+  struct Level {
+    uint32_t cnt, pad;
+    unsigned long long queue;
+  };
+  static_assert(offsetof(ApplyCtl, reloc_out) - offsetof(ApplyCtl, n_seg_out) == offsetof(Level, queue),
+                "the counters' place in the control block of updates");
   uint32_t *cand = s.flags, *next = s.pos, *cnt = (uint32_t *)&g->actl->n_seg_out;
   uint32_t *long_v = s.seg, *long_base = s.tagpref;  // 2 (cap + 2) words: both rows of every vertex
   unsigned long long *queue = &g->actl->reloc_out;
@@ -391,17 +398,15 @@ pr_status vertex_order(Graph *g, int kind, uint32_t *perm, uint32_t *inv, const 
   }
   const unsigned egrid = (unsigned)std::max(1, g->sm_count * 8);
   for (int level = 0; hi > lo && level < kMaxLevels; level++) {
-    CK(cudaMemsetAsync(cnt, 0, 4, st));
-    CK(cudaMemsetAsync(queue, 0, 8, st));
+    CK(cudaMemsetAsync(cnt, 0, sizeof(Level), st));
     k_order_expand<<<egrid, 256, 0, st>>>(g->out.rd, g->out.col, g->in.rd, g->in.col, perm, lo, hi, inv, cand,
                                           next, cnt, queue, long_v, long_base);
     count_launch();
-    uint32_t c = 0;
-    unsigned long long q = 0;
-    CK(cudaMemcpyAsync(&c, cnt, 4, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(&q, queue, 8, cudaMemcpyDeviceToHost, st));
+    Level h{};
+    CK(cudaMemcpyAsync(&h, cnt, sizeof(Level), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    if (q) {
+    uint32_t c = h.cnt;
+    if (h.queue) {
       k_order_expand_long<<<egrid, 256, 0, st>>>(g->out.rd, g->out.col, g->in.rd, g->in.col, perm, lo, inv, cand,
                                                  next, cnt, queue, long_v, long_base);
       count_launch();
