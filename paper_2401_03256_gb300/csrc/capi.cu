@@ -630,22 +630,30 @@ pr_status pr_get_affected(pr_graph *h, uint32_t *out, int64_t cap, int64_t *coun
     return PR_OK;
   }
   int64_t total = 0;
-  for (int b = 0; b < 3; b++) {
-    int64_t c = g.last_list_cnt[b];
-    int64_t take = std::max<int64_t>(0, std::min<int64_t>(c, cap - total));
-    if (take > 0) {
-      const uint32_t *ids = g.list[b];
-      if (g.perm) {  // back to the caller's numbering (the three lists hold at most n ids)
-        prdf::gather_ids(g.perm, ids, g.gen_tmp + total, (uint64_t)take, g.st);
-        ids = g.gen_tmp + total;
-      }
-      cudaError_t e = cudaMemcpyAsync(out + total, ids, 4ull * take, cudaMemcpyDeviceToHost, g.st);
+  for (int b = 0; b < 3; b++) total += g.last_list_cnt[b];
+  const int64_t take = std::min<int64_t>(total, cap);
+  // one launch whatever the lists hold (at most n ids together).  Short ones go straight to pinned
+  // memory: 700 ids 17 us, 21 with a copy from the device
+  const bool pinned = take > 0 && take <= (int64_t)prdf::kPinnedIds;
+  if (pinned) {
+    prdf::gather_lists(&g, g.ids_h, (uint64_t)take);
+  } else if (g.perm && take > 0) {
+    prdf::gather_lists(&g, g.gen_tmp, (uint64_t)take);
+    cudaError_t e = cudaMemcpyAsync(out, g.gen_tmp, 4ull * take, cudaMemcpyDeviceToHost, g.st);
+    if (e != cudaSuccess) return prdf::cuda_fail(&g, e, "get affected");
+  } else {
+    int64_t at = 0;
+    for (int b = 0; b < 3; b++) {
+      const int64_t k = std::min<int64_t>(g.last_list_cnt[b], take - at);
+      if (k <= 0) continue;
+      cudaError_t e = cudaMemcpyAsync(out + at, g.list[b], 4ull * k, cudaMemcpyDeviceToHost, g.st);
       if (e != cudaSuccess) return prdf::cuda_fail(&g, e, "get affected");
+      at += k;
     }
-    total += c;
   }
   cudaError_t e = cudaStreamSynchronize(g.st);
   if (e != cudaSuccess) return prdf::cuda_fail(&g, e, "get affected");
+  if (pinned) std::memcpy(out, g.ids_h, 4ull * take);
   *count = total;
   return PR_OK;
 }

@@ -434,9 +434,11 @@ pr_status graph_build(Graph *g, uint64_t m_in, const uint32_t *src_d, const uint
   CK(cudaMemsetAsync(g->chunk_done, 0, 4ull * n, st));
   char *host = nullptr;
   const size_t actl_room = (sizeof(ApplyCtl) + 255) & ~(size_t)255;
-  CK(cudaMallocHost((void **)&host, actl_room + sizeof(RankCtl)));
+  const size_t ctl_room = (sizeof(RankCtl) + 255) & ~(size_t)255;
+  CK(cudaMallocHost((void **)&host, actl_room + ctl_room + 4ull * kPinnedIds));
   g->actl_h = (ApplyCtl *)host;
   g->ctl_h = (RankCtl *)(host + actl_room);
+  g->ids_h = (uint32_t *)(host + actl_room + ctl_room);
   if (g->f32) {
     using S = Store<true>;
     k_init_rank<true><<<grid_for(n), 256, 0, st>>>(g->out.rd, n, g->p.alpha, (S::A *)g->adeg, (S::R *)g->R[0],

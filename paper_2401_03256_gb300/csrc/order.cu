@@ -525,14 +525,29 @@ pr_status hot_order(Graph *g, const std::vector<uint32_t> &comp_n, uint32_t hot_
   return PR_OK;
 }
 
-__global__ void k_gather_ids(const uint32_t *perm, const uint32_t *ids, uint32_t *out, uint64_t k) {
+// The three affected lists of a call one after another, in the caller's numbering.
+struct IdLists {
+  const uint32_t *ids[3];
+  uint32_t count[3];
+};
+__global__ void k_gather_lists(const uint32_t *perm, const IdLists l, uint32_t *out, uint64_t k) {
   const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < k) out[i] = perm[ids[i]];
+  if (i >= k) return;
+  uint64_t j = i;
+  int b = 0;
+  for (; b < 2 && j >= l.count[b]; b++) j -= l.count[b];
+  const uint32_t v = l.ids[b][j];
+  out[i] = perm ? perm[v] : v;
 }
 
-void gather_ids(const uint32_t *perm, const uint32_t *ids, uint32_t *out, uint64_t k, cudaStream_t st) {
+void gather_lists(const Graph *g, uint32_t *out, uint64_t k) {
   if (k == 0) return;
-  k_gather_ids<<<grid_of(k), 256, 0, st>>>(perm, ids, out, k);
+  IdLists l;
+  for (int b = 0; b < 3; b++) {
+    l.ids[b] = g->list[b];
+    l.count[b] = g->last_list_cnt[b];
+  }
+  k_gather_lists<<<grid_of(k), 256, 0, g->st>>>(g->perm, l, out, k);
   count_launch();
 }
 

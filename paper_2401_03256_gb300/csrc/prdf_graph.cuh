@@ -35,6 +35,7 @@ template <class T>
 Piece piece(T **p, uint64_t count) { return Piece{(void **)p, sizeof(T) * (count ? count : 1)}; }
 cudaError_t alloc_pieces(std::initializer_list<Piece> pieces);
 
+constexpr uint32_t kPinnedIds = 16384;
 constexpr int kRankBlocksPerSm = 4;  // most blocks of the rank kernel on an SM
 
 // A handle's place in a server: the launch sizes it had before.  Either may go first.
@@ -117,6 +118,7 @@ struct Graph {
 
   ApplyScratch sc;
   ApplyCtl *actl = nullptr, *actl_h = nullptr;
+  uint32_t *ids_h = nullptr;         // [kPinnedIds] pinned: short affected sets on their way to the caller
   uint32_t *big = nullptr;           // updates: staging of the long rows' entries
   uint64_t big_cap = 0;
   void *longs = nullptr;             // updates: long rows' merge entries
@@ -181,7 +183,8 @@ pr_status order_cost(Graph *g, const uint32_t *perm, const uint32_t *inv, uint64
 pr_status hot_order(Graph *g, const std::vector<uint32_t> &comp_n, uint32_t hot_max, uint32_t *perm, uint32_t *inv,
                     std::vector<uint32_t> &hot, uint32_t *lab, uint32_t *at);
 uint32_t hot_limit(bool f32);  // sweep.cu: contributions a block's shared-memory copy holds (less a few)
-void gather_ids(const uint32_t *perm, const uint32_t *ids, uint32_t *out, uint64_t k, cudaStream_t st);  // out[i] = perm[ids[i]]
+// the first k entries of the affected lists, one after another, in the caller's numbering
+void gather_lists(const Graph *g, uint32_t *out, uint64_t k);
 void map_ids(const uint32_t *inv, uint32_t *a, uint64_t m, cudaStream_t st);
 pr_status graph_export(Graph *g, int dir, uint64_t *offs_h, uint32_t *cols_h);
 pr_status graph_refresh_ident(Graph *g);
