@@ -245,7 +245,7 @@ pr_status pr_autotune(pr_graph *h, int32_t sweep_iters, pr_tuning *chosen) {
   pr_tuning best = cur;
   best.ms = 1e30;
   const int32_t los[] = {4, 8, 16, 32};
-  const bool blocks = !prdf::sweep_eligible(&g) && !prdf::batch_eligible(&g, false);
+  const bool blocks = !prdf::sweep_eligible(&g, false) && !prdf::batch_eligible(&g, false);
   const int per_sm_max = blocks ? std::max(1, g.rank_grid_max / g.sm_count) : std::max(1, cur.blocks_per_sm);
   const int per_sm_min = blocks ? std::max(1, per_sm_max - 2) : std::max(1, cur.blocks_per_sm);
   g.p.max_iter = sweep_iters;

@@ -158,7 +158,6 @@ struct Graph {
   int loop_grid = 0;                 // blocks of a persistent launch that runs to the end of its call
   bool bounded_runs = false;         // runs of compacted iterations end early to let other handles' launches in
   int pro_grid = 0;                  // blocks of the cooperative prologue launch
-  bool loop_sweeps = true;           // single-graph self-loop handles iterate in per-iteration launches
   std::vector<std::shared_ptr<Served>> served;  // the servers it is attached to
   std::string err;
 };
@@ -205,7 +204,7 @@ pr_status components_setup(Graph *g, const std::vector<uint32_t> &comp_n);  // a
 
 // batch.cu: the iterations of batched handles (unless df_split is 0 or the graphs are small), one
 // persistent launch after the marking launch of marking calls.
-constexpr int kGraphWhole = 0, kGraphMarking = 1, kGraphBatchMarking = 2, kGraphBatchEvery = 3;
+constexpr int kGraphWhole = 0, kGraphMarking = 1, kGraphBatchMarking = 2, kGraphBatchEvery = 3, kGraphEvery = 4;
 bool batch_eligible(const Graph *g, bool marking);  // of a call that marks, or of one over every vertex
 pr_status batch_setup(Graph *g);
 pr_status batch_items(Graph *g);  // after a rebuild of the sweep items
@@ -217,9 +216,11 @@ size_t marking_smem(const Graph *g);
 // Frontier, Dynamic Traversal or asynchronous call, one launch per iteration inside a
 // CUDA-graph loop whose condition the last block of each sweep sets on the device.
 pr_status sweep_setup(Graph *g);
-bool sweep_eligible(const Graph *g);  // single graph, self-loop mode, no graph-launch mode
+bool sweep_eligible(const Graph *g, bool marking);  // single graph, self-loop mode; replayed: calls over every vertex
 pr_status sweep_full(Graph *g, bool from_init);                  // all vertices, every iteration
 pr_status sweep_dense(Graph *g, RankMode mode, const void *rank_args);  // after the marking launch's handoff
+// graph-launch mode: a control-block reset and one cooperative kernel, by a graph kept for this kind of call
+pr_status graph_replay(Graph *g, int kind, const cudaKernelNodeParams &kp);
 void sweep_free(Graph *g);
 // A handle in a server of `slots` slots (1: by itself): launches that run to the end of their call on at
 // most 1/slots of the device, bounded runs of the compacted iterations of a Dynamic Frontier call.

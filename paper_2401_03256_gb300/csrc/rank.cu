@@ -1222,7 +1222,7 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
   a.emap = g->emap;
   a.item_pos = g->item_pos;
   const bool marking = mode == kModeDF || mode == kModeDT || async;
-  const bool loops = sweep_eligible(g), batch = batch_eligible(g, marking && !start_full);
+  const bool loops = sweep_eligible(g, marking), batch = batch_eligible(g, marking && !start_full);
   a.split = marking && (loops || batch) && g->split_df && !start_full;
   // expected marks of a set of k vertices: k * m / n; deferring to a pull pays once they
   // would make the next set dense (more than n / dense_div) several times over: a pull
@@ -1290,47 +1290,13 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
     }
     return copy_async_parity();
   }
-  // CUDA-graph launch: the control-block reset, the event records and the cooperative
-  // kernel are captured once; later calls only replace the kernel's arguments and replay
   cudaKernelNodeParams kp{};
   kp.func = const_cast<void *>(fn);
   kp.gridDim = dim3(g->rank_grid);
   kp.blockDim = dim3(kRankBlock);
   kp.sharedMemBytes = (unsigned)rank_smem(g->ncomp);
   kp.kernelParams = args;
-  const int kind = marking ? kGraphMarking : kGraphWhole;
-  if (g->cg_exec && g->cg_kind != kind) {
-    cudaGraphExecDestroy(g->cg_exec);
-    cudaGraphDestroy(g->cg);
-    g->cg_exec = nullptr;
-    g->cg = nullptr;
-  }
-  if (!g->cg_exec) {
-    cudaGraph_t graph = nullptr;
-    CK(cudaGraphCreate(&graph, 0));
-    cudaGraphNode_t reset = nullptr, kern = nullptr;
-    cudaMemsetParams mp{};
-    mp.dst = g->ctl;
-    mp.value = 0;
-    mp.elementSize = 1;
-    mp.width = sizeof(RankCtl);
-    mp.height = 1;
-    mp.pitch = sizeof(RankCtl);
-    CK(cudaGraphAddMemsetNode(&reset, graph, nullptr, 0, &mp));
-    CK(cudaGraphAddKernelNode(&kern, graph, &reset, 1, &kp));
-    cudaLaunchAttributeValue coop{};
-    coop.cooperative = 1;
-    CK(cudaGraphKernelNodeSetAttribute(kern, cudaLaunchAttributeCooperative, &coop));
-    CK(cudaGraphInstantiate(&g->cg_exec, graph, 0));
-    g->cg = graph;
-    g->cg_kernel = kern;
-    g->cg_kind = kind;
-  } else {
-    CK(cudaGraphExecKernelNodeSetParams(g->cg_exec, g->cg_kernel, &kp));
-  }
-  CK(cudaGraphLaunch(g->cg_exec, g->st));
-  count_launch();
-  return PR_OK;
+  return graph_replay(g, marking ? kGraphMarking : kGraphWhole, kp);
 }
 
 // After a rank call that did not finish (a wait ran out, or a launch failed behind another): its

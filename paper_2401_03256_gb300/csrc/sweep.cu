@@ -839,6 +839,42 @@ cudaError_t add_conditional(cudaGraphNode_t *node, cudaGraph_t graph, const cuda
   return e;
 }
 
+}  // namespace
+
+// A control-block reset and one cooperative kernel as a CUDA graph: built once per kind of call,
+// later calls replace the kernel's arguments and replay.
+pr_status graph_replay(Graph *g, int kind, const cudaKernelNodeParams &kp) {
+  if (g->cg_exec && g->cg_kind != kind) {
+    cudaGraphExecDestroy(g->cg_exec);
+    g->cg_exec = nullptr;
+  }
+  if (!g->cg_exec) {
+    if (g->cg) cudaGraphDestroy(g->cg);
+    g->cg = nullptr;
+    CKG(cudaGraphCreate(&g->cg, 0));
+    cudaGraphNode_t reset = nullptr;
+    cudaMemsetParams mp{};
+    mp.dst = g->ctl;
+    mp.value = 0;
+    mp.elementSize = 1;
+    mp.width = sizeof(RankCtl);
+    mp.height = 1;
+    mp.pitch = sizeof(RankCtl);
+    CKG(cudaGraphAddMemsetNode(&reset, g->cg, nullptr, 0, &mp));
+    CKG(add_kernel(&g->cg_kernel, g->cg, &reset, 1, kp.func, kp.gridDim, kp.blockDim, kp.kernelParams, true,
+                   kp.sharedMemBytes));
+    CKG(cudaGraphInstantiate(&g->cg_exec, g->cg, 0));
+    g->cg_kind = kind;
+  } else {
+    CKG(cudaGraphExecKernelNodeSetParams(g->cg_exec, g->cg_kernel, &kp));
+  }
+  CKG(cudaGraphLaunch(g->cg_exec, g->st));
+  count_launch();
+  return PR_OK;
+}
+
+namespace {
+
 template <bool F32>
 size_t hot_bytes(const SweepArgs<F32> &a) { return (size_t)a.hot * sizeof(typename Store<F32>::C); }
 
@@ -854,6 +890,15 @@ pr_status full_impl(Graph *g, bool from_init) {
   if constexpr (F32) p.init = (float)(1.0 / (double)g->n);
   else p.init = std::llrint(1.0 / (double)g->n * 4611686018427387904.0);
   void *args[] = {(void *)&p};
+  if (g->use_graph) {
+    cudaKernelNodeParams kp{};
+    kp.func = (void *)k_loop<F32, false>;
+    kp.gridDim = dim3(g->loop_grid);
+    kp.blockDim = dim3(kSweepBlock);
+    kp.sharedMemBytes = (unsigned)hot_bytes(p.a);
+    kp.kernelParams = args;
+    return graph_replay(g, kGraphEvery, kp);
+  }
   CKG(cudaLaunchCooperativeKernel((const void *)k_loop<F32, false>, dim3(g->loop_grid), dim3(kSweepBlock), args,
                                   hot_bytes(p.a), g->st));
   count_launch();
@@ -1065,8 +1110,8 @@ void sweep_share(Graph *g, int slots) {
   g->bounded_runs = slots > 1;
 }
 
-bool sweep_eligible(const Graph *g) {
-  return g->loop_sweeps && g->ncomp == 1 && !g->teleport && !g->use_graph && g->loops != nullptr;
+bool sweep_eligible(const Graph *g, bool marking) {
+  return g->ncomp == 1 && !g->teleport && g->loops != nullptr && (!g->use_graph || (!marking && g->split_df));
 }
 
 pr_status sweep_full(Graph *g, bool from_init) {
