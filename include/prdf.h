@@ -94,8 +94,8 @@ typedef struct {
                              Ids are translated at every call: results, ranks, affected sets
                              and the CSR export are in the caller's numbering (a renumbered
                              handle keeps 8 B per vertex of translation tables on the device,
-                             16 B in FP32 where it has vertices of large out-degree, and 4 B on
-                             the host).  Those vertices come first in the numbering.  Computing a numbering takes a second,
+                             16 B in FP32 where it has vertices of large out-degree, which come
+                             first in the numbering).  Computing a numbering takes a second,
                              transient build of the graph on the device; without room for it
                              the caller's numbering is kept (0) or creation fails with
                              PR_ERR_OUT_OF_MEMORY (2, 3).  Other values: PR_ERR_INVALID_ARG. */
@@ -283,7 +283,7 @@ pr_status pr_get_affected(pr_graph *g, uint32_t *out, int64_t cap, int64_t *coun
  * entries written): iter_ms[i] its duration, affected[i] the vertices affected after it,
  * kind[i]: in the persistent marking launch 0 = affected lists, 1 = compacted sweep items
  * reused, 2 = sweep items compacted in this iteration, 4 = all sweep items scanned, those
- * of vertices stamped later skipped; 3 = all vertices; in the per-iteration launches of a
+ * of vertices stamped later skipped; 3 = all vertices; in the sweep launches of a
  * split call 5 = compacted items, 6 = all items with the stamp check, 7 = all items, vertices
  * not yet affected joining by pull from the previous iteration's change flags, 8 = compacted
  * items rebuilt before the sweep.  Any of the output arrays may be NULL (host memory). */

@@ -155,7 +155,7 @@ struct RankCtl {
   uint32_t xit[kMaxIterLimit + 2];                    // entries appended for each slot: read after the
                                                       // barrier, when no block can append to that slot
   uint32_t xneed[kMaxIterLimit + 2];                  // continuation: a recorded expansion would mark
-  // per-iteration sweep launches (sweep.cu): what one launch leaves for the next
+  // sweep launches (sweep.cu): what one launch leaves for the next
   uint32_t ticket;        // blocks of the current sweep launch that have finished
   uint32_t lbar;          // grid barrier arrivals of the current run of iterations (k_batch)
   unsigned long long tally[2];  // the same of k_loop, with what the iteration left (sweep_dev.cuh)
@@ -163,7 +163,6 @@ struct RankCtl {
   uint32_t sw_all[3];     // sweep items per tier (all vertices)
   uint32_t sw_off[2];     // first item of tiers 1 and 2 (in the item and compacted arrays)
   uint32_t m_cur;         // stored edges (in-edges of all vertices)
-  uint32_t dmode;         // dense Dynamic Frontier: 1 = every item swept with the stamp check, 0 = compacted items
   uint32_t pull_check;    // this iteration pulls marks from the previous iteration's changes
   uint32_t erec;          // this iteration records per-vertex change flags (the next may pull)
   uint32_t push_items;    // pushed marks append their sweep items to the compacted items
@@ -181,7 +180,7 @@ struct RankCtl {
   uint32_t xcap;          // expansion-list entries this iteration writes at most (more: it only counts)
   uint32_t x_long;        // a compacted iteration listed a vertex with an out-row longer than kInlineOut
   uint32_t jtotal;        // vertices that joined by pulls (not in the lists)
-  uint32_t dense_ran;     // the per-iteration loop ran: its writeback listed the affected set
+  uint32_t dense_ran;     // the sweep launches ran: their writeback listed the affected set
   uint32_t aff_total;     // affected vertices listed by that writeback (list 0)
   uint32_t pull_all;      // the pull kernel also pulls tier-0/1 rows (the marks after the last iteration)
   unsigned long long bar_limit_ns;  // grid-barrier wait limit (0 = the default)

@@ -143,7 +143,7 @@ struct Graph {
   unsigned long long *comp_last = nullptr;
   std::vector<pr_stats> comp_stats;  // per graph, from the last rank call
   uint32_t dense_div = 16;           // dense iterations once affected > n / dense_div
-  bool split_df = true;              // dense iterations of marking calls continue in per-iteration launches
+  bool split_df = true;              // dense iterations of marking calls continue in the sweep launches
   int32_t barrier_us = 0;            // grid-barrier wait limit of the persistent launches (0 = 4 s)
   uint32_t chunk_len = kChunk;       // sweep order: edges per chunk of a tier-2 row (128, 256 or 512)
   uint32_t group_max = kGroupMax;    // sweep order: longest row of an 8-lane group (16, 32 or 64)
@@ -151,8 +151,8 @@ struct Graph {
   std::vector<int64_t> trace_aff;    // affected vertices at the start of each iteration
   std::vector<int32_t> trace_kind;   // 0 sparse, 1 dense, 2 dense after compaction, 3 all vertices
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-  // per-iteration sweep launches (sweep.cu): change flags of the dense Dynamic Frontier
-  // iterations and the CUDA graphs that loop over the iterations on the device
+  // sweep launches (sweep.cu): change flags of the dense Dynamic Frontier iterations and the
+  // CUDA graphs that string the launches of a call together on the device
   uint8_t *emap = nullptr;           // [2][n] rank change above tau_f, by iteration parity; 0 between calls
   void *loops = nullptr;             // sweep.cu's cached graphs
   int loop_grid = 0;                 // blocks of a persistent launch that runs to the end of its call
@@ -212,9 +212,9 @@ pr_status batch_run(Graph *g, RankMode mode, bool marking, const void *rank_args
 const void *marking_kernel(bool f32);  // rank.cu: the marking launch of batched handles
 size_t marking_smem(const Graph *g);
 
-// sweep.cu: Static / Naive-dynamic iterations, and the dense iterations of a Dynamic
-// Frontier, Dynamic Traversal or asynchronous call, one launch per iteration inside a
-// CUDA-graph loop whose condition the last block of each sweep sets on the device.
+// sweep.cu: Static / Naive-dynamic iterations in one persistent launch, and the dense iterations of a
+// Dynamic Frontier, Dynamic Traversal or asynchronous call: while the set grows a launch each, then
+// runs of them, in a CUDA graph whose conditions the launches set on the device.
 pr_status sweep_setup(Graph *g);
 bool sweep_eligible(const Graph *g, bool marking);  // single graph, self-loop mode; replayed: calls over every vertex
 pr_status sweep_full(Graph *g, bool from_init);                  // all vertices, every iteration

@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(kRankBlock, SPLIT == 1 ? kFewMarksBlocks : PRD
       return;
     }
     if (a.split) {
-      // the set is fixed: every iteration runs in the per-iteration launches
+      // the set is fixed: every iteration runs in the sweep launches
       fold_counters();
       if (blockIdx.x == 0 && tid == 0) {
 #pragma unroll
@@ -611,7 +611,7 @@ __global__ void __launch_bounds__(kRankBlock, SPLIT == 1 ? kFewMarksBlocks : PRD
                           (prev_total == 0xFFFFFFFFu || total_now - prev_total > total_now / 16);
     prev_total = total_now;
     // split calls: once the affected set is dense, the iterations continue in the
-    // per-iteration launches (which grow the set by pulling or pushing); this launch stops
+    // sweep launches (which grow the set by pulling or pushing); this launch stops
     // before the iteration, whose marks are in place
     if (df && a.split && dense) {
       if (blockIdx.x == 0 && tid == 0) {
@@ -627,7 +627,7 @@ __global__ void __launch_bounds__(kRankBlock, SPLIT == 1 ? kFewMarksBlocks : PRD
     // split calls: a sparse iteration over a set whose out-rows would likely make the next
     // set dense (defer_at, from the average degree) pushes nothing; it records each
     // vertex's change flag (and marks the first expansions as done), and the next
-    // iteration, the first of the per-iteration launches, pulls its marks from them
+    // iteration, the first of the sweep launches, pulls its marks from them
     // (pushing that many out-rows costs more than one pull over every item)
     const bool defer = expand && a.split && !dense && total_now > a.defer_at;
     const uint32_t slot = (uint32_t)it + 1;
@@ -981,7 +981,7 @@ __global__ void __launch_bounds__(kRankBlock, SPLIT == 1 ? kFewMarksBlocks : PRD
     last_key = dR;
     if (blockIdx.x == 0 && tid == 0) ctl->t_ns[it + 2] = globaltimer_ns();
     if (defer) {
-      // tier-2 rows pull before the handoff (the first per-iteration sweep pulls tier-0/1
+      // tier-2 rows pull before the handoff (the first sweep launch pulls tier-0/1
       // rows itself).  If this was the last iteration (converged or max_iter), the launches
       // that follow only make its marks, which belong to the affected set (Algorithm 1
       // marks in every iteration, the last included)
@@ -1241,7 +1241,7 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
   if (batch) return batch_run(g, mode, a.split != 0, &a);
   if (loops && (!marking || start_full)) {
     // every vertex every iteration (Static; Naive-dynamic, also for a marking call whose
-    // affected set is all of V): per-iteration launches in a device-side loop
+    // affected set is all of V): one persistent launch (df_split 0: a launch each)
     pr_status rc = sweep_full(g, mode == kModeStatic);
     if (rc != PR_OK) return rc;
     return copy_async_parity();
@@ -1279,7 +1279,7 @@ static pr_status launch(Graph *g, RankMode mode, bool start_full) {
     if (a.split) {
       // the marking launch stops once the affected set is dense (or, for Dynamic
       // Traversal, after its search); the host reads the status it left and starts the
-      // per-iteration loop, or the full sweeps if every vertex turned out affected
+      // sweep launches, or the full sweeps if every vertex turned out affected
       CK(cudaMemcpyAsync(g->ctl_h, g->ctl, offsetof(RankCtl, final_cnt), cudaMemcpyDeviceToHost, g->st));
       CK(cudaStreamSynchronize(g->st));
       const RankCtl &h = *g->ctl_h;
@@ -1350,7 +1350,7 @@ pr_status rank_run(Graph *g, RankMode mode, pr_stats *stats) {
   CK(cudaMemcpyAsync(g->ctl_h, g->ctl, offsetof(RankCtl, dR_bits), cudaMemcpyDeviceToHost, g->st));
   CK(cudaMemcpyAsync(&g->ctl_h->vproc, &g->ctl->vproc, 5 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                      g->st));
-  // the per-iteration loop's state (launch count, whether it ran, its affected count)
+  // the sweep launches' state (launch count, whether it ran, its affected count)
   CK(cudaMemcpyAsync(&g->ctl_h->ticket, &g->ctl->ticket, offsetof(RankCtl, eprev) - offsetof(RankCtl, ticket),
                      cudaMemcpyDeviceToHost, g->st));
   CK(cudaStreamSynchronize(g->st));
@@ -1385,7 +1385,7 @@ pr_status rank_run(Graph *g, RankMode mode, pr_stats *stats) {
   g->last_full = full;
   uint32_t fcnt[3] = {h.final_cnt[0], h.final_cnt[1], h.final_cnt[2]};
   if (h.dense_ran) {
-    // the per-iteration loop's writeback listed the whole affected set in list 0
+    // the sweep launches' writeback listed the whole affected set in list 0
     fcnt[0] = h.aff_total;
     fcnt[1] = fcnt[2] = 0;
   }

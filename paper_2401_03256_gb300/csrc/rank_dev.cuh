@@ -1,5 +1,5 @@
 // rank_dev.cuh - device-side pieces shared by the rank kernels (rank.cu) and the
-// per-iteration sweep kernels (sweep.cu): the rank arithmetic of each mode, the kernel
+// sweep kernels (sweep.cu, batch.cu): the rank arithmetic of each mode, the kernel
 // arguments, memory-access helpers with L2 eviction policies, the bounded grid barrier,
 // and the frontier marking of Algorithm 1 (push: out-rows of expanding vertices).
 #pragma once
@@ -16,14 +16,14 @@ constexpr uint64_t kStageTimeoutNs = 1000000000ull;    // 1 s: a staged copy tha
 constexpr int kWarps = kRankBlock / 32;
 constexpr uint32_t kFull = 0xffffffffu;
 constexpr uint16_t kNoStamp = 0xFFFF;
-// Dense per-iteration Dynamic Frontier launches set the stamp's top bit of an affected
+// The sweeps of a dense Dynamic Frontier call set the stamp's top bit of an affected
 // vertex whose out-row has been marked from (a cache of its expanded bit: the stamp is read
 // anyway); iteration numbers stay below it (max_iter <= 1000)
 constexpr uint16_t kStampExp = 0x8000;
 constexpr uint16_t kStampIt = 0x7FFF;
 // RankCtl::status after a launch of a split call
 constexpr uint32_t kStatusDone = 1;     // the call is complete (writeback done)
-constexpr uint32_t kStatusDense = 2;    // the dense iterations continue in per-iteration launches from next_it
+constexpr uint32_t kStatusDense = 2;    // the dense iterations continue in the sweep launches from next_it
 constexpr uint32_t kStatusFull = 5;     // every vertex is affected: the full-sweep iterations follow
 constexpr uint32_t kInlineOut = 128;  // longer out-rows are marked by the whole grid (hub queue)
 #ifndef PRDF_RANK_MIN_BLOCKS
@@ -111,9 +111,9 @@ struct RankArgs {
   uint32_t bin_lo, bin_hi;
   uint32_t gmax, chunk;    // sweep tiers (sweep_tier) and edges per tier-2 chunk
   RankCtl *ctl;
-  // split calls (single graph, self-loop mode): once the affected set is dense the marking
-  // launch stops and the iterations continue in per-iteration launches (sweep.cu)
-  int split;              // this call hands its dense iterations to per-iteration launches
+  // split calls (self-loop mode): once the affected set is dense the marking
+  // launch stops and the iterations continue in the sweep launches (sweep.cu; batch.cu)
+  int split;              // this call hands its dense iterations to the sweep launches
   uint32_t defer_at;      // split calls: a sparse set larger than this defers its marks to a pull
   uint32_t *xlist;        // vertices to expand, recorded by dense sweeps (n)
   uint8_t *emap;          // [2][n] rank change above tau_f, by iteration parity (pull marking)
@@ -141,27 +141,14 @@ __device__ __forceinline__ X warp_sum(X x) {
   return x;
 }
 
-// ------------------------------------------------- bulk copies into shared memory ----
-// A warp stages a contiguous run of sweep items (16-byte aligned, a multiple of 16 bytes)
-// into its own shared-memory buffer with one cp.async.bulk issued by lane 0; completion is
-// tracked by an mbarrier (arrival count 1: lane 0's arrive with the expected bytes).
+// ---------------------------------------------------------- mbarriers in shared memory ----
+// Arrival count 1: the thread that issues a bulk copy arrives with its bytes (sweep_dev.cuh).
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init1(uint32_t bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-// lane 0: expect `bytes` on `bar` and copy them from global `src` to shared `dst`.  The
-// buffer's previous contents were read by the warp before (a __syncwarp orders those
-// reads; the proxy fence orders them before the copy's writes).
-__device__ __forceinline__ void bulk_stage(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-  asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
 }
 
 // Bounded wait for the phase of `bar` with the given parity to complete; false after

@@ -493,7 +493,6 @@ __global__ void k_dense_init(const DenseInit p) {
   ctl->app_since = 0;
   ctl->push_n = 0;  // pull_check: set by a marking launch that deferred its marks to a pull
   ctl->push_items = 0;
-  ctl->dmode = 1;
   ctl->compact_now = 0;
   ctl->dexpand = p.traversal ? 0u : 1u;
   ctl->erec = p.traversal ? 0u : 1u;
