@@ -43,6 +43,11 @@ constexpr uint32_t kPullMin = 64;   // and at least this many
 // requests take more than 21 to 27 ms (23 to 30 with unbounded runs), of the largest's 54 (49);
 // at saturation no difference, nor between 2^27 and 2^31.
 constexpr uint64_t kRunEdges = 1ull << 29;
+// ... and a graph of fewer edges than this runs on 1/slots of the device: its iterations are bound by
+// latency, so two side by side end sooner than in turns.  Five graphs of 2^16 to 2^20 vertices, 2
+// slots, all requests at once: 16.9 ms with those of up to 2^24 edges on half of the device, 17.2 of 2^22,
+// 17.4 none, 18.2 of 2^25.
+constexpr uint64_t kShareEdges = 1ull << 24;
 constexpr uint32_t kLightPush = 16384;  // at most this many first expansions: the light push may mark them
 
 // End of an all-item iteration, or of a run of compacted iterations it_first ... it, by one
@@ -968,6 +973,8 @@ pr_status full_steps_impl(Graph *g, bool from_init) {
   return PR_OK;
 }
 
+int run_grid(const Graph *g) { return g->bounded_runs && g->m < kShareEdges ? g->loop_grid : g->sm_count; }
+
 template <bool F32>
 pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
   const bool async = mode == kModeDFAsync;
@@ -992,6 +999,7 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
   std::vector<unsigned char> key;
   append_key(key, a);
   append_key(key, ra);
+  append_key(key, run_grid(g));
   if (lg.exec && key != lg.key) lg.release();
   DenseInit ip{};
   ip.ctl = g->ctl;
@@ -1043,7 +1051,7 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
     LoopArgs<F32> la{};
     la.a = a;
     void *largs[] = {(void *)&la};
-    CKG(add_kernel(&s0, sw[0], nullptr, 0, (const void *)k_loop<F32, true>, dim3(g->sm_count), dim3(kSweepBlock), largs,
+    CKG(add_kernel(&s0, sw[0], nullptr, 0, (const void *)k_loop<F32, true>, dim3(run_grid(g)), dim3(kSweepBlock), largs,
                    true, hot_bytes(a)));
     void *sargs[] = {(void *)&a};
     CKG(add_kernel(&s1, sw[1], nullptr, 0, (const void *)k_sweep<F32, 1>, dim3(g->sm_count),
