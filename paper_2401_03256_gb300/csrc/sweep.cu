@@ -45,8 +45,8 @@ constexpr uint32_t kPullMin = 64;   // and at least this many
 constexpr uint64_t kRunEdges = 1ull << 29;
 // ... and a graph of fewer edges than this runs on 1/slots of the device: its iterations are bound by
 // latency, so two side by side end sooner than in turns.  Five graphs of 2^16 to 2^20 vertices, 2
-// slots, all requests at once: 16.9 ms with those of up to 2^24 edges on half of the device, 17.2 of 2^22,
-// 17.4 none, 18.2 of 2^25.
+// slots, all requests at once: 16.8 ms with those of up to 2^24 edges on half of the device, 17.2 of 2^22,
+// 17.4 none, 18.2 of 2^25; 16.1 with their prologues (k_df_push) on half of it too.
 constexpr uint64_t kShareEdges = 1ull << 24;
 constexpr uint32_t kLightPush = 16384;  // at most this many first expansions: the light push may mark them
 
@@ -974,6 +974,7 @@ pr_status full_steps_impl(Graph *g, bool from_init) {
 }
 
 int run_grid(const Graph *g) { return g->bounded_runs && g->m < kShareEdges ? g->loop_grid : g->sm_count; }
+int push_grid(const Graph *g) { return std::max(1, g->pro_grid * run_grid(g) / g->sm_count); }
 
 template <bool F32>
 pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
@@ -1039,7 +1040,7 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
     void *pargs[] = {(void *)&ra};
     CKG(add_kernel(&pull_node, pb[1], nullptr, 0, (const void *)k_df_pull<F32>, dim3(std::max(1, g->sm_count * 8)),
                    dim3(kRankBlock), pargs, false));
-    CKG(add_kernel(&pnode, pb[2], nullptr, 0, (const void *)k_df_push<F32>, dim3(g->pro_grid), dim3(kRankBlock), pargs,
+    CKG(add_kernel(&pnode, pb[2], nullptr, 0, (const void *)k_df_push<F32>, dim3(push_grid(g)), dim3(kRankBlock), pargs,
                    true));
     cudaGraphNode_t lnode = nullptr;
     CKG(add_kernel(&lnode, pb[3], nullptr, 0, (const void *)k_df_push_light<F32>, dim3(std::max(1, g->sm_count)),
@@ -1067,7 +1068,7 @@ pr_status dense_impl(Graph *g, RankMode mode, const RankArgs<F32> &ra_in) {
     CKG(cudaGraphAddEmptyNode(&fe, fb[0], nullptr, 0));
     CKG(add_kernel(&fpull, fb[1], nullptr, 0, (const void *)k_df_pull<F32>, dim3(std::max(1, g->sm_count * 8)),
                    dim3(kRankBlock), pargs, false));
-    CKG(add_kernel(&fpush, fb[2], nullptr, 0, (const void *)k_df_push<F32>, dim3(g->pro_grid), dim3(kRankBlock),
+    CKG(add_kernel(&fpush, fb[2], nullptr, 0, (const void *)k_df_push<F32>, dim3(push_grid(g)), dim3(kRankBlock),
                    pargs, true));
     void *fargs[] = {(void *)&ra};
     CKG(add_kernel(&fnode, lg.graph, &fsw, 1, (const void *)k_df_finish<F32>, dim3(std::max(1, g->sm_count * 4)),
