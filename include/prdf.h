@@ -338,7 +338,7 @@ pr_status pr_static_noalloc(uint32_t n, int64_t m, const uint64_t *in_off, const
  * and free device memory (cudaMemGetInfo) covers hbm_reserve_bytes plus the request's
  * estimate; an idle device always admits one request.  While attached, a graph's launches that
  * run to the end of a call take at most 1/slots of the device, so that concurrent ones fit together;
- * the iterations of a dense frontier take all of it, in turns of about 2 ms, from 2^24 edges on.  pr_server_destroy
+ * the iterations of a dense frontier take all of it (half below 2^24 edges), in turns of about 2 ms.  pr_server_destroy
  * gives every graph its own launch sizes back.
  * An update = one pr_apply_batches over the coalesced requests in submission order + one
  * pr_dynamic_frontier;

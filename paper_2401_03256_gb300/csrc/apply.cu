@@ -923,7 +923,7 @@ pr_status graph_apply(Graph *g, uint64_t nd, const uint32_t *ds, const uint32_t 
   const unsigned grid =
       N <= kPlanBlockSort ? 1u
                           : (unsigned)std::min<uint64_t>((N + kPlanThreads - 1) / kPlanThreads,
-                                                         (uint64_t)std::max(2, std::min(g->loop_grid, g->sm_count)));
+                                                         (uint64_t)std::max(2, g->share_grid));
   p.hist = s.radix_hist;
   p.part = s.radix_hist + 256ull * grid;
   p.in_rd = g->in.rd;

@@ -156,6 +156,7 @@ struct Graph {
   uint8_t *emap = nullptr;           // [2][n] rank change above tau_f, by iteration parity; 0 between calls
   void *loops = nullptr;             // sweep.cu's cached graphs
   int loop_grid = 0;                 // blocks of a persistent launch that runs to the end of its call
+  int share_grid = 0;                // blocks of a short launch beside which another may run (updates' plan, small graphs' runs)
   bool bounded_runs = false;         // runs of compacted iterations end early to let other handles' launches in
   int pro_grid = 0;                  // blocks of the cooperative prologue launch
   std::vector<std::shared_ptr<Served>> served;  // the servers it is attached to

@@ -7,9 +7,11 @@
 // admitted requests of different graphs run at the same time on their graphs' own
 // streams.  A graph's marking launch takes 1/slots of the blocks that can be resident.  Its dense
 // iterations take the whole device, about 2 ms at a time (sweep.cu), so that concurrent requests
-// take turns (1/slots for graphs of less than 2^24 edges, whose iterations would not fill it).  (On 1/slots each, a request alone left half of the device idle: eight R-MAT graphs of
-// 2^18 to 2^24 vertices, 2 slots: service p99 at 50 requests/s 61 ms, now 45; p50 and p99 at
-// saturation 94 and 404 ms, now 72 and 204.)  Continuous batching: when a graph's worker gets a slot it takes the requests
+// take turns (half of it for graphs of less than 2^24 edges, whose iterations would not fill it).  On
+// 1/slots each, a request alone left the rest of the device idle: eight R-MAT graphs of 2^18 to 2^24
+// vertices, 2 slots, service p99 at 50 requests/s 61 ms, now 46 to 51; p50 and p99 at saturation 94
+// and 404 ms, now 70 to 76 and 202 to 239.
+// Continuous batching: when a graph's worker gets a slot it takes the requests
 // queued for that graph by then (up to max_coalesce), applies their batches in order with
 // one pr_apply_batches and runs one pr_dynamic_frontier over the net change;
 // each result records submit, start and completion times (host clock) and the stats.

@@ -43,7 +43,7 @@ constexpr uint32_t kPullMin = 64;   // and at least this many
 // requests take more than 21 to 27 ms (23 to 30 with unbounded runs), of the largest's 54 (49);
 // at saturation no difference, nor between 2^27 and 2^31.
 constexpr uint64_t kRunEdges = 1ull << 29;
-// ... and a graph of fewer edges than this runs on 1/slots of the device: its iterations are bound by
+// ... and a graph of fewer edges than this runs on half of the device: its iterations are bound by
 // latency, so two side by side end sooner than in turns.  Five graphs of 2^16 to 2^20 vertices, 2
 // slots, all requests at once: 16.8 ms with those of up to 2^24 edges on half of the device, 17.2 of 2^22,
 // 17.4 none, 18.2 of 2^25; 16.1 with their prologues (k_df_push) on half of it too.
@@ -973,7 +973,7 @@ pr_status full_steps_impl(Graph *g, bool from_init) {
   return PR_OK;
 }
 
-int run_grid(const Graph *g) { return g->bounded_runs && g->m < kShareEdges ? g->loop_grid : g->sm_count; }
+int run_grid(const Graph *g) { return g->bounded_runs && g->m < kShareEdges ? g->share_grid : g->sm_count; }
 int push_grid(const Graph *g) { return std::max(1, g->pro_grid * run_grid(g) / g->sm_count); }
 
 template <bool F32>
@@ -1104,7 +1104,7 @@ pr_status sweep_setup(Graph *g) {
                         g->f32 ? (const void *)k_sweep<true, 1> : (const void *)k_sweep<false, 1>,
                         g->f32 ? (const void *)k_sweep<true, 0> : (const void *)k_sweep<false, 0>};
   for (const void *fn : fns) CKG(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHotBytes));
-  g->loop_grid = g->sm_count;
+  g->loop_grid = g->share_grid = g->sm_count;
   int per_sm_pro = 0;
   CKG(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
       &per_sm_pro, g->f32 ? (const void *)k_df_push<true> : (const void *)k_df_push<false>, kRankBlock, 0));
@@ -1115,6 +1115,7 @@ pr_status sweep_setup(Graph *g) {
 
 void sweep_share(Graph *g, int slots) {
   g->loop_grid = std::max(1, g->sm_count / slots);
+  g->share_grid = std::max(1, g->sm_count / std::min(slots, 2));
   g->bounded_runs = slots > 1;
 }
 
